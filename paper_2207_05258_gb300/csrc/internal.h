@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include "dfloat.cuh"
 #include "hweno.h"
 #include <stdint.h>
 
@@ -114,6 +115,7 @@ constexpr TileVariant kVariants1D[] = {{128, 1}, {64, 1}, {256, 1}, {128, 2}, {6
 constexpr int kNumVariants1D = HWENO_TILE_VARIANTS;
 static_assert(sizeof(kVariants1D) / sizeof(kVariants1D[0]) == kNumVariants1D, "variant table");
 constexpr int tile_points(int v) { return kVariants1D[v].threads * kVariants1D[v].ppt - 4; }
+constexpr int kVariants1DPoints = 252;  // largest tile of any variant
 constexpr int kThreads1D = 128;
 constexpr int kTile1D = tile_points(0);
 constexpr int kMinTile1D = 60;  // smallest tile of any variant
@@ -147,6 +149,11 @@ struct SchemeParams {
   // p0 - g1 p1 - g2 p2 in f_{i-1}, f_i, f_{i+1}, H_i
   double wd[kConstTable];
   float wf[kConstTable];
+  // g0, g1, g2, d0, d1, d2, eps and gas gamma - 1 as FP32 pairs, and the
+  // largest scaled indicator for which the pairs' products stay in the FP32
+  // range (weno_df.cuh): eps / beta no smaller than 2^-90
+  D2 wp[8];
+  float wp_bmax;
 };
 
 // The constant table of SchemeParams. p0 - g1 p1 - g2 p2 (the quintic's
@@ -164,6 +171,9 @@ inline void fill_constant_table(SchemeParams& sp, const double g[3], const doubl
                                    11.0 / 60.0 - g[2] / 6.0,
                                    0.5 - 2.0 * g[1] / 3.0 - g[2] / 3.0};
   for (int i = 0; i < kConstTable; ++i) { sp.wd[i] = tab[i]; sp.wf[i] = (float)tab[i]; }
+  for (int i = 0; i < 7; ++i) sp.wp[i] = dconst(tab[i]);
+  sp.wp[7] = dconst(gas_gamma - 1.0);
+  sp.wp_bmax = (float)(eps * 0x1p90 < 0x1p100 ? eps * 0x1p90 : 0x1p100);
 }
 
 // Arguments of one 1D launch (all instances of the batch).
@@ -202,13 +212,16 @@ struct Args1D {
   SchemeParams sp;
 };
 
-// Minimum resident CTAs per SM requested from the compiler for the stage
-// kernels, per precision (register budget = 64K / (threads x this)); chosen
-// by measurement: the FP64 kernels are FP64-pipe bound at any occupancy
-// (1..4 CTAs gave the same throughput), the FP32 ones gain from more warps
-// (1D: 8 CTAs, 64 registers, +12%; 2D: 5 CTAs).
+// Minimum resident CTAs (of 128 threads) per SM requested from the compiler
+// for the stage kernels, per precision (register budget = 64K / (threads x
+// this)); chosen by measurement: the all-FP64 kernels are FP64-pipe bound at
+// any occupancy (1..4 CTAs gave the same throughput); the 1D FP64 kernel,
+// most of whose instructions are FP32, needs warps to hide their latency (4
+// CTAs, 128 registers: 2048-instance Riemann batch 4.41 ms per step against
+// 6.88 with 2 CTAs of 184); the FP32 ones gain from more warps (1D: 8 CTAs,
+// 64 registers, +12%; 2D: 5 CTAs).
 #ifndef HWENO_MINB_1D_F64
-#define HWENO_MINB_1D_F64 1
+#define HWENO_MINB_1D_F64 4
 #endif
 #ifndef HWENO_MINB_1D_F32
 #define HWENO_MINB_1D_F32 8
@@ -387,6 +400,7 @@ struct PersistArgs {
   int* active;                // instances with t < t_end after the last step
   unsigned long long* pu;     // point-updates of stepping instances (nullable)
   int steps, ntiles, batch;
+  int tile;                   // FP64: points per tile
   unsigned wait_extra;        // test hook: tiles of instance 0 wait for this many more
 };
 

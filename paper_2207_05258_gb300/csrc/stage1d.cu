@@ -15,8 +15,11 @@
 //   4. per point: the flux differences L^1, L^2, the HWENO limiter
 //      (characteristic-wise for Euler), the SSP-RK3 combination, the stores,
 //      and the maximum wave speed of the new state for the next stage.
-// The FP64 pipe bounds these kernels, so every point and interface quantity is
-// computed once and divisions are folded (see hweno_math.cuh).
+// Every point and interface quantity is computed once. FP64 states: the FP64
+// pipe would bound the stage, so only what the result's last bits depend on
+// runs there and the nonlinear corrections run in pairs of FP32 numbers
+// (stage1d_df.cuh); in the cluster step's latency form divisions are folded
+// instead (hweno_math.cuh).
 #include "stage1d_impl.cuh"
 
 namespace hweno {

@@ -1,0 +1,267 @@
+// One stage of the 1D scheme on a tile for FP64 states (included by
+// stage1d_impl.cuh; the structure of a stage is described in stage1d.cu).
+//
+// What bounds it: the FP64 pipe takes one warp instruction per 65 to 77
+// cycles and sub-partition, and an all-FP64 stage needs about 830 per point
+// (Euler; it ran the pipe at 86%). Here FP64 keeps what the result's last
+// bits depend on (fluxes, the differences of F and U, the linear derivative
+// flux, the linear limited derivative, the Runge-Kutta update), about 150
+// per point; the corrections relative to it are taken in pairs of FP32
+// numbers (weno_df.cuh), about 7 300 FP32 instructions per point, which issue
+// next to the FP64 pipe. Interfaces and points whose correction is not small
+// (1-5% of them in flows with shocks) go on a list and are evaluated in FP64.
+// Measured, 2048 Riemann problems (2.5 M points): 12.8 -> 3.99 ms per step
+// (FP64 pipe 55% busy, issue slots 49%); Buckley-Leverett, 246 k points:
+// 0.40 -> 0.15 ms; one instance of 200 points: 131 -> 92 us. The loops over
+// sides and fields stay rolled: unrolled, the straight code outruns the
+// instruction caches (6.9 ms per step).
+//
+// Phases, with a barrier after each:
+//   1 points      load with ghosts; F, h = f'(u) v in FP64; H^{+-} = dx h^{+-},
+//                 dx v and the eigen-system's inputs as pairs
+//   2 edges       differences of F and U (FP64, then pairs)
+//   3 interfaces  c = f-hat - (F_i + F_{i+1})/2 and the limited derivative
+//     and points  from pairs; the derivative flux in FP64
+//   3b            the list, in FP64
+//   4 points      flux differences, update, wave speed
+// The tile shape (threads, points per thread) and the stage are run-time
+// arguments: one copy of the code for all of them.
+
+template <int EQ>
+using Tile1D = LineTile<Dim1<EQ>::M, 0, EQ == HWENO_EULER>;
+
+constexpr int kMaxPPT1D = 2;  // points per thread of any tile variant
+constexpr int kMaxTile1D = 508;
+
+template <int EQ, int NT, int PPT>
+struct Layout1D<EQ, double, NT, PPT> {
+  static constexpr int P = NT * PPT - 4;
+  static constexpr size_t bytes = Tile1D<EQ>::bytes(P + 4, P + 1);
+};
+
+// A value no speed of the state `u` exceeds by more than 2^-11 relative, in
+// FP32 (NaN where FP32 cannot tell: p below 2^-8 E, where the subtraction
+// costs too many bits, and anything outside the float range).
+template <int EQ>
+__device__ __forceinline__ float rough_speed(const double* u, float gam) {
+  if constexpr (EQ == HWENO_BURGERS) {
+    return fabsf(to_float(u[0]));
+  } else if constexpr (EQ == HWENO_BUCKLEY) {
+    const float x = to_float(u[0]), y = 1.f - x, D = 4.f * x * x + y * y;
+    return fabsf(8.f * x * y) / (D * D);
+  } else {
+    const float r = to_float(u[0]), m = to_float(u[1]), E = to_float(u[2]);
+    const float ir = 1.f / r, vel = m * ir, e = E - 0.5f * m * vel;
+    const float s = fabsf(vel) + sqrtf(gam * (gam - 1.f) * e * ir);
+    return e >= 0.00390625f * E ? s : __int_as_float(0x7fc00000);
+  }
+}
+
+// Phase 1, point g of the tile that starts at s.
+template <int EQ>
+__device__ __forceinline__ void load_point_df(const Tile1D<EQ>& r, const Args1D& a,
+                                              const double* U, const double* V, int n, int s,
+                                              int g, D2 alp, D2 dxp) {
+  constexpr int M = Dim1<EQ>::M;
+  int kind;
+  const int src = map_1d(s - 2 + g, n, a.sp.bc[0], a.sp.bc[1], kind);
+  HWENO_CHECK(kind == 2 || (src >= 0 && src < n), a.status);
+  double u[M], v[M], h[M];
+#pragma unroll
+  for (int c = 0; c < M; ++c) {
+    if (kind == 2) {
+      u[c] = a.sp.inflow[c];
+      v[c] = 0.0;
+    } else {
+      u[c] = U[(long long)c * n + src];
+      v[c] = V[(long long)c * n + src];
+      if (kind == 1) {  // one of the two changes sign
+        const bool odd = refl_sign<EQ>(c) < 0.f;
+        if (odd) u[c] = -u[c];
+        else v[c] = -v[c];
+      }
+    }
+    r.U(c, g) = u[c];
+    r.N(c, g) = v[c];
+  }
+  if constexpr (EQ == HWENO_BURGERS) {
+    r.F(0, g) = 0.5 * u[0] * u[0];
+    h[0] = u[0] * v[0];
+    r.h(0, g) = h[0];
+  } else if constexpr (EQ == HWENO_BUCKLEY) {
+    const double w = 1.0 - u[0], u4 = 4.0 * u[0], iD = recip_fp64(fma(w, w, u4 * u[0]));
+    r.F(0, g) = u4 * u[0] * iD;
+    h[0] = 2.0 * u4 * w * iD * iD * v[0];
+    r.h(0, g) = h[0];
+  } else {
+    const double gm1 = a.sp.wd[9] - 1.0;
+    const double ir = recip_fp64(u[0]);
+    const double vel = u[1] * ir;
+    const double p = gm1 * (u[2] - 0.5 * u[1] * vel);
+    const double Ep = u[2] + p;
+    const double dvel = (v[1] - vel * v[0]) * ir;
+    const double dp = gm1 * (v[2] - vel * v[1] + 0.5 * vel * vel * v[0]);
+    h[0] = v[1];
+    h[1] = v[1] * vel + u[1] * dvel + dp;
+    h[2] = (v[2] + dp) * vel + Ep * dvel;
+    r.F(1, g) = u[1] * vel + p;
+    r.F(2, g) = Ep * vel;
+    r.h(1, g) = h[1];
+    r.h(2, g) = h[2];
+    point_eigen(r, g, u[0], ir, Ep, vel, 0.0);
+  }
+  point_pairs(r, g, v, h, alp, dxp);
+}
+
+// One stage (mode) on the tile of P points of instance k starting at s.
+template <int EQ>
+__device__ __forceinline__ void stage_tile_df(const Args1D& a, const StageIO& io, const int mode,
+                                              const int P, const int k, const int s) {
+  constexpr int M = Dim1<EQ>::M;
+  extern __shared__ __align__(16) unsigned char smem1d[];
+  const Tile1D<EQ> r{reinterpret_cast<double*>(smem1d), P + 4, P + 1, a.status};
+  __shared__ double s_dt;
+  __shared__ unsigned s_top;
+  __shared__ int s_nf, s_nl;  // items of the lists
+  __shared__ unsigned short s_f[kMaxTile1D + 1], s_l[kMaxTile1D];
+  const int nt = blockDim.x;
+
+  const int n = a.inst_n[k];
+  if (a.skip_done && !(a.t[k] < a.t_end)) return;
+  const int np = min(P, n - s);
+  HWENO_CHECK(s >= 0 && np >= 1 && P <= kMaxTile1D, a.status);
+  const long long off = a.inst_off[k] * M;
+  const double* geo = a.inst_geo + 3 * k;
+  const double dx = geo[0], idx = geo[1], idx2 = geo[2];
+  const double alpha = io.alpha_in[k];
+
+  // time step: once per CTA (thread 0), read back after the barriers below
+  if (threadIdx.x == 0) {
+    double dt = 0.0;
+    if (mode == MODE_STAGE1) {
+      int lands = 0;
+      dt = a.dt_in ? a.dt_in[k]
+                   : time_step(a.sp, io.alpha_in[k], a.inst_hx[k], a.t[k], a.t_end, lands);
+      if (s == 0) { a.dt[k] = dt; a.lands[k] = lands; }
+    } else if (mode != MODE_RHS) {
+      dt = a.dt[k];
+    }
+    s_dt = dt;
+    s_top = 0u;
+    s_nf = s_nl = 0;
+  }
+
+  // 1: points
+  {
+    const D2 alp = scale_pair(alpha), dxp = to_pair(dx);
+    const double* U = static_cast<const double*>(io.U) + off;
+    const double* V = static_cast<const double*>(io.V) + off;
+    for (int g = threadIdx.x; g < np + 4; g += nt)
+      load_point_df<EQ>(r, a, U, V, n, s, g, alp, dxp);
+    __syncthreads();
+    // 2: edges
+    for (int g = threadIdx.x; g < np + 3; g += nt) edge_pairs(r, g, 1, alp);
+  }
+  __syncthreads();
+
+  // 3: interfaces x_{s+j-1/2}, j = 0..np (left point at loaded index j + 1),
+  // and the limited derivatives of points j = 0..np-1 (loaded index j + 2)
+  const bool limited = a.sp.limiter != 0;
+  for (int j = threadIdx.x; j <= np; j += nt) {
+    double x[M];
+    // (the mean state's eigenvectors are taken in FP64)
+    if (!((M == 1 || a.sp.eig_avg == 0) && interface_line<D2, 0>(r, j + 1, 1, alpha, dx, a.sp, x)))
+      s_f[atomicAdd(&s_nf, 1)] = (unsigned short)j;
+    const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      r.C(c, j) = x[c];
+      r.D(c, j) = derivative_flux_fp64(r, c, j + 1, 1, kU, kh, kv);
+    }
+    if (j < np && limited) {
+      if (!limiter_line<D2, 0>(r, j + 2, 1, dx, idx, a.sp, x))
+        s_l[atomicAdd(&s_nl, 1)] = (unsigned short)j;
+#pragma unroll
+      for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
+    }
+  }
+  __syncthreads();
+
+  // 3b: the lists
+  if (s_nf + s_nl > 0) {  // uniform
+    listed_items<0>(r, s_f, s_nf, s_l, s_nl, [](int j, bool lim) { return lim ? j + 2 : j + 1; }, 1,
+                    k + s / P, alpha, dx, idx, a.sp);
+    __syncthreads();
+  }
+
+  // 4: points
+  // SSP-RK3: x_out = a x0 + b x + k dF, as stage_update
+  const double b = mode == MODE_STAGE1 ? 1.0 : mode == MODE_STAGE2 ? 0.25 : 2.0 / 3.0;
+  const double a0 = mode == MODE_STAGE2 ? 0.75 : 1.0 / 3.0;
+  const double k1 = -(b * s_dt) * idx, k2 = -(b * s_dt) * idx2;
+  const bool want_alpha = mode != MODE_RHS && io.alpha_out != nullptr;  // uniform
+  float top = 0.f;
+  for (int j = threadIdx.x; j < np; j += nt) {
+    const int g = j + 2;
+    HWENO_CHECK(s + j < n, a.status);
+    const long long at = off + s + j;
+    double un[M];
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      const long long q = at + (long long)c * n;
+      const double dF = fma(0.5, r.F(c, g + 1) - r.F(c, g - 1), r.C(c, j + 1) - r.C(c, j));
+      const double dD = r.D(c, j + 1) - r.D(c, j);
+      const double vt = limited ? r.lim(c, j) : r.N(c, g);
+      if (mode == MODE_RHS) {
+        static_cast<double*>(a.L1)[q] = -dF * idx;
+        static_cast<double*>(a.L2)[q] = -dD * idx2;
+        if (a.Vlim) static_cast<double*>(a.Vlim)[q] = vt;
+      } else {
+        double x = r.U(c, g), y = vt;
+        if (mode == MODE_STAGE1) {
+          static_cast<double*>(io.Vt0out)[q] = vt;
+        } else {
+          x = a0 * static_cast<const double*>(io.U0)[q] + b * x;
+          y = a0 * static_cast<const double*>(io.Vt0)[q] + b * y;
+        }
+        un[c] = x + k1 * dF;
+        static_cast<double*>(io.Uout)[q] = un[c];
+        static_cast<double*>(io.Vout)[q] = y + k2 * dD;
+        // kept for the wave speed below in a row that this phase does not read
+        reinterpret_cast<double&>(r.H(0, c, g)) = un[c];
+      }
+    }
+    if (want_alpha) {
+      const float f = rough_speed<EQ>(un, a.sp.wf[9]);
+      reinterpret_cast<float&>(r.H(1, 0, g)) = f;
+      top = fmaxf(top, f);  // a NaN is no bound
+    }
+  }
+  // The wave speed of the stage output (stages 1 and 2; stage 3 as well when
+  // the persistent run asks for the next step's alpha): the FP64 speed is
+  // evaluated only where the FP32 one comes within 2^-9 of the tile's largest
+  // (or is not usable), which cannot miss the maximum.
+  if (want_alpha) {
+    const unsigned tw = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, tw);
+    __syncthreads();
+    top = __uint_as_float(s_top) * (1.f - 0x1p-9f);
+    double amax = 0.0;
+    bool bad = false;
+    for (int j = threadIdx.x; j < np; j += nt) {
+      const int g = j + 2;
+      if (reinterpret_cast<float&>(r.H(1, 0, g)) < top) continue;
+      double u[M];
+#pragma unroll
+      for (int c = 0; c < M; ++c) u[c] = reinterpret_cast<double&>(r.H(0, c, g));
+      const double sp = wave_speed<EQ>(u, a.sp.wd[9], a.sp.wd[10]);
+      bad |= !(sp <= real_max<double>());
+      amax = fmax(amax, sp);
+    }
+    if (bad) atomicOr(a.status, STATUS_NONFINITE);
+    if (__any_sync(0xffffffffu, amax > 0.0)) {
+      const unsigned long long m = warp_max_bits(amax);
+      if ((threadIdx.x & 31) == 0) atomicMax(&io.alpha_out[k], m);
+    }
+  }
+}

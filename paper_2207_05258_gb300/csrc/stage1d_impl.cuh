@@ -12,6 +12,7 @@
 #include "hweno.h"
 #include "hweno_math.cuh"
 #include "internal.h"
+#include "line_df.cuh"
 
 namespace hweno {
 namespace {
@@ -360,8 +361,11 @@ __device__ __forceinline__ void stage_update(const StageIO& io, long long base, 
   }
 }
 
+#include "stage1d_df.cuh"
+
 // One stage on the tile of instance k starting at point s (the whole CTA;
-// contains barriers, so every thread calls it with the same k, s).
+// contains barriers, so every thread calls it with the same k, s), FP32
+// states; stage_tile_df is its FP64 counterpart.
 template <int EQ, class Real, int MODE, int NT, int PPT, bool FAC = false>
 __device__ __forceinline__ void stage_tile(const Args1D& a, const StageIO& io, const int k,
                                            const int s) {
@@ -550,6 +554,40 @@ __device__ __forceinline__ void stage_tile(const Args1D& a, const StageIO& io, c
   }
 }
 
+// One stage of either precision on an NT * PPT - 4 point tile.
+template <int EQ, class Real, int NT, int PPT, bool FAC = false>
+__device__ __forceinline__ void stage_any(const Args1D& a, const StageIO& io, int mode, int k,
+                                          int s) {
+  if constexpr (std::is_same<Real, double>::value)
+    stage_tile_df<EQ>(a, io, mode, NT * PPT - 4, k, s);
+  else if (mode == MODE_STAGE1)
+    stage_tile<EQ, Real, MODE_STAGE1, NT, PPT, FAC>(a, io, k, s);
+  else if (mode == MODE_STAGE2)
+    stage_tile<EQ, Real, MODE_STAGE2, NT, PPT, FAC>(a, io, k, s);
+  else
+    stage_tile<EQ, Real, MODE_STAGE3, NT, PPT, FAC>(a, io, k, s);
+}
+
+// FP64: tile shape (blockDim.x threads, P points) and stage at run time.
+template <int EQ>
+__global__ void __launch_bounds__(256, (MinBlocks1D<double, 256>::value))
+k_stage_1d_f64(const __grid_constant__ Args1D a, int mode, int P) {
+  stage_tile_df<EQ>(a, io_of(a), mode, P, a.tile_inst[blockIdx.x], a.tile_start[blockIdx.x]);
+}
+
+template <int EQ>
+cudaError_t stage_launch_f64(int variant, int mode, const Args1D& a, int ntiles, cudaStream_t s) {
+  const int P = tile_points(variant);
+  const size_t bytes = Tile1D<EQ>::bytes(P + 4, P + 1);
+  static unsigned configured = 0;  // devices whose limit is raised
+  if (const cudaError_t e = ensure_smem_limit(
+          k_stage_1d_f64<EQ>, Tile1D<EQ>::bytes(kVariants1DPoints + 4, kVariants1DPoints + 1),
+          configured))
+    return e;
+  k_stage_1d_f64<EQ><<<ntiles, kVariants1D[variant].threads, bytes, s>>>(a, mode, P);
+  return cudaGetLastError();
+}
+
 template <int EQ, class Real, int MODE, int NT, int PPT>
 __global__ void __launch_bounds__(NT, (MinBlocks1D<Real, NT>::value))
 k_stage_1d(const __grid_constant__ Args1D a) {
@@ -579,7 +617,9 @@ cudaError_t stage_modes(int mode, const Args1D& a, int ntiles, cudaStream_t s) {
 // Variants of kVariants1D: (threads, points per thread).
 template <int EQ, class Real>
 cudaError_t stage_variants(int variant, int mode, const Args1D& a, int ntiles, cudaStream_t s) {
-  switch (variant) {
+  if constexpr (std::is_same<Real, double>::value)
+    return stage_launch_f64<EQ>(variant, mode, a, ntiles, s);
+  else switch (variant) {
     case 1: return stage_modes<EQ, Real, 64, 1>(mode, a, ntiles, s);
     case 2: return stage_modes<EQ, Real, 256, 1>(mode, a, ntiles, s);
     case 3: return stage_modes<EQ, Real, 128, 2>(mode, a, ntiles, s);
@@ -680,20 +720,21 @@ k_run_1d(const __grid_constant__ Args1D a, const __grid_constant__ PersistArgs p
       io.Uout = p.U1; io.Vout = p.V1; io.Vt0out = p.Vt0;
       io.alpha_in = reinterpret_cast<const double*>(slot0);
       io.alpha_out = slot0 + p.batch;
-      stage_tile<EQ, Real, MODE_STAGE1, NT, PPT, kFactoredRun<Real>>(a, io, k, s);
     } else if (stage == 1) {
       io.U = p.U1; io.V = p.V1; io.U0 = a.U; io.Vt0 = p.Vt0;
       io.Uout = p.U2; io.Vout = p.V2; io.Vt0out = nullptr;
       io.alpha_in = reinterpret_cast<const double*>(slot0 + p.batch);
       io.alpha_out = slot0 + 2 * p.batch;
-      stage_tile<EQ, Real, MODE_STAGE2, NT, PPT, kFactoredRun<Real>>(a, io, k, s);
     } else {
       io.U = p.U2; io.V = p.V2; io.U0 = a.U; io.Vt0 = p.Vt0;
       io.Uout = const_cast<void*>(a.U); io.Vout = const_cast<void*>(a.V); io.Vt0out = nullptr;
       io.alpha_in = reinterpret_cast<const double*>(slot0 + 2 * p.batch);
       io.alpha_out = p.alpha + (size_t)((par ^ 1) * 3) * p.batch;  // alpha(U^{n+1})
-      stage_tile<EQ, Real, MODE_STAGE3, NT, PPT, kFactoredRun<Real>>(a, io, k, s);
     }
+    if constexpr (std::is_same<Real, double>::value)
+      stage_tile_df<EQ>(a, io, MODE_STAGE1 + stage, p.tile, k, s);
+    else
+      stage_any<EQ, Real, NT, PPT, kFactoredRun<Real>>(a, io, MODE_STAGE1 + stage, k, s);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
@@ -744,10 +785,40 @@ int run_occupancy() {
   return nb;
 }
 
+template <int EQ>
+cudaError_t run_launch_f64(int variant, const Args1D& a, PersistArgs p, int ctas, cudaStream_t s) {
+  p.tile = tile_points(variant);
+  const size_t bytes = Tile1D<EQ>::bytes(p.tile + 4, p.tile + 1);
+  static unsigned configured = 0;  // devices whose limit is raised
+  if (const cudaError_t e = ensure_smem_limit(
+          k_run_1d<EQ, double, 256, 1>,
+          Tile1D<EQ>::bytes(kVariants1DPoints + 4, kVariants1DPoints + 1), configured))
+    return e;
+  k_run_1d<EQ, double, 256, 1><<<ctas, kVariants1D[variant].threads, bytes, s>>>(a, p);
+  return cudaGetLastError();
+}
+
+template <int EQ>
+int run_occupancy_f64(int variant) {
+  const int P = tile_points(variant);
+  if (cudaFuncSetAttribute(
+          k_run_1d<EQ, double, 256, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+          (int)Tile1D<EQ>::bytes(kVariants1DPoints + 4, kVariants1DPoints + 1)) != cudaSuccess)
+    return 0;
+  int nb = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &nb, k_run_1d<EQ, double, 256, 1>, kVariants1D[variant].threads,
+          Tile1D<EQ>::bytes(P + 4, P + 1)) != cudaSuccess)
+    return 0;
+  return nb;
+}
+
 template <int EQ, class Real>
 cudaError_t run_variants(int variant, const Args1D& a, const PersistArgs& p, int ctas,
                          cudaStream_t s) {
-  switch (variant) {
+  if constexpr (std::is_same<Real, double>::value)
+    return run_launch_f64<EQ>(variant, a, p, ctas, s);
+  else switch (variant) {
     case 1: return run_launch<EQ, Real, 64, 1>(a, p, ctas, s);
     case 2: return run_launch<EQ, Real, 256, 1>(a, p, ctas, s);
     case 3: return run_launch<EQ, Real, 128, 2>(a, p, ctas, s);
@@ -758,7 +829,8 @@ cudaError_t run_variants(int variant, const Args1D& a, const PersistArgs& p, int
 
 template <int EQ, class Real>
 int occupancy_variants(int variant) {
-  switch (variant) {
+  if constexpr (std::is_same<Real, double>::value) return run_occupancy_f64<EQ>(variant);
+  else switch (variant) {
     case 1: return run_occupancy<EQ, Real, 64, 1>();
     case 2: return run_occupancy<EQ, Real, 256, 1>();
     case 3: return run_occupancy<EQ, Real, 128, 2>();
@@ -784,6 +856,24 @@ int occupancy_prec(int eq, int variant) {
 // ---------------------------------------------------------------------------
 // Fused step of small instances (FusedArgs): one CTA per instance.
 // ---------------------------------------------------------------------------
+// The arrays of one stage (0, 1, 2) of a fused step.
+__device__ __forceinline__ StageIO step_io(const Args1D& a, const FusedArgs& f, int stage,
+                                           const double* alpha_in, unsigned long long* alpha_out) {
+  StageIO io = io_of(a);
+  io.alpha_in = alpha_in;
+  io.alpha_out = alpha_out;
+  if (stage == 0) {
+    io.Uout = f.U1; io.Vout = f.V1; io.Vt0out = f.Vt0;
+    return io;
+  }
+  io.U = stage == 1 ? f.U1 : f.U2;
+  io.V = stage == 1 ? f.V1 : f.V2;
+  io.U0 = a.U; io.Vt0 = f.Vt0; io.Vt0out = nullptr;
+  io.Uout = stage == 1 ? f.U2 : const_cast<void*>(a.U);
+  io.Vout = stage == 1 ? f.V2 : const_cast<void*>(a.V);
+  return io;
+}
+
 template <int EQ, class Real>
 __global__ void __launch_bounds__(kFusedThreads)
 k_step_small_1d(const __grid_constant__ Args1D a, const __grid_constant__ FusedArgs f) {
@@ -818,20 +908,14 @@ k_step_small_1d(const __grid_constant__ Args1D a, const __grid_constant__ FusedA
     }
     __syncthreads();
   }
-  StageIO io = io_of(a);
-  io.Uout = f.U1; io.Vout = f.V1; io.Vt0out = f.Vt0;
-  io.alpha_in = reinterpret_cast<const double*>(s0); io.alpha_out = s1;
-  stage_tile<EQ, Real, MODE_STAGE1, kFusedThreads, kFusedPPT>(a, io, k, 0);
-  __syncthreads();
-  io.U = f.U1; io.V = f.V1; io.U0 = a.U; io.Vt0 = f.Vt0; io.Uout = f.U2; io.Vout = f.V2;
-  io.Vt0out = nullptr;
-  io.alpha_in = reinterpret_cast<const double*>(s1); io.alpha_out = s2;
-  stage_tile<EQ, Real, MODE_STAGE2, kFusedThreads, kFusedPPT>(a, io, k, 0);
-  __syncthreads();
-  io.U = f.U2; io.V = f.V2; io.Uout = const_cast<void*>(a.U); io.Vout = const_cast<void*>(a.V);
-  io.alpha_in = reinterpret_cast<const double*>(s2); io.alpha_out = nullptr;
-  stage_tile<EQ, Real, MODE_STAGE3, kFusedThreads, kFusedPPT>(a, io, k, 0);
-  __syncthreads();
+#pragma unroll 1
+  for (int stage = 0; stage < 3; ++stage) {
+    stage_any<EQ, Real, kFusedThreads, kFusedPPT>(
+        a, step_io(a, f, stage, reinterpret_cast<const double*>(f.alpha + stage * f.batch),
+                   stage < 2 ? f.alpha + (stage + 1) * f.batch : nullptr),
+        MODE_STAGE1 + stage, k, 0);
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {  // time update (as k_finalize)
     double tk = a.t[k];
     const double d = a.dt[k];
@@ -1136,20 +1220,15 @@ k_step_cluster_1d(const __grid_constant__ Args1D a, const __grid_constant__ Fuse
       }
     }
     cl.sync();
-    StageIO io = io_of(a);
-    io.Uout = f.U1; io.Vout = f.V1; io.Vt0out = f.Vt0;
-    io.alpha_in = reinterpret_cast<const double*>(s0); io.alpha_out = s1;
-    if (has) stage_tile<EQ, Real, MODE_STAGE1, kThreads1D, 1>(a, io, k, s);
-    cl.sync();
-    io.U = f.U1; io.V = f.V1; io.U0 = a.U; io.Vt0 = f.Vt0; io.Uout = f.U2; io.Vout = f.V2;
-    io.Vt0out = nullptr;
-    io.alpha_in = reinterpret_cast<const double*>(s1); io.alpha_out = s2;
-    if (has) stage_tile<EQ, Real, MODE_STAGE2, kThreads1D, 1>(a, io, k, s);
-    cl.sync();
-    io.U = f.U2; io.V = f.V2; io.Uout = const_cast<void*>(a.U); io.Vout = const_cast<void*>(a.V);
-    io.alpha_in = reinterpret_cast<const double*>(s2); io.alpha_out = nullptr;
-    if (has) stage_tile<EQ, Real, MODE_STAGE3, kThreads1D, 1>(a, io, k, s);
-    cl.sync();  // every CTA is past its reads of t[k]
+#pragma unroll 1
+    for (int stage = 0; stage < 3; ++stage) {
+      if (has)
+        stage_any<EQ, Real, kThreads1D, 1>(
+            a, step_io(a, f, stage, reinterpret_cast<const double*>(f.alpha + stage * f.batch),
+                       stage < 2 ? f.alpha + (stage + 1) * f.batch : nullptr),
+            MODE_STAGE1 + stage, k, s);
+      cl.sync();  // after the third: every CTA is past its reads of t[k]
+    }
     if (rank == 0 && threadIdx.x == 0) {
       if (!live) {  // finished: nothing moves (as k_finalize)
         if (f.dt_used) f.dt_used[k] = 0.0;
