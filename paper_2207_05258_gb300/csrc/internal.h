@@ -226,6 +226,9 @@ struct Args1D {
 #ifndef HWENO_MINB_1D_F32
 #define HWENO_MINB_1D_F32 8
 #endif
+#ifndef HWENO_MINB_2D_F64
+#define HWENO_MINB_2D_F64 4
+#endif
 #ifndef HWENO_MINB_X_F64
 #define HWENO_MINB_X_F64 1
 #endif

@@ -23,19 +23,20 @@ namespace hweno {
 // (edges k, k + S), and for Euler sqrt(rho), un, H and (2D) ut. Then
 // the outputs: c = f-hat - (F_i + F_{i+1})/2, the derivative flux D, and the
 // limited derivative.
-template <int M_, int DIR, bool EUL_, int MX = 0>
+template <int M_, int DIR, bool EUL_, int MX = 0, bool SLIM_ = false>
 struct LineTile {
   static constexpr int M = M_, kn = EUL_ ? 1 + DIR : 0;
-  static constexpr bool EUL = EUL_;
+  static constexpr bool EUL = EUL_, SLIM = SLIM_;
   static constexpr int NE = EUL ? M : 0;
   static constexpr int MF = EUL ? M - 1 : M;  // stored rows of F and h
-  static constexpr int nd = 2 * M + 2 * MF + MX, np = 6 * M + NE, no = 3 * M;
+  static constexpr int nd = 2 * M + 2 * MF + MX, np = (SLIM ? 4 : 6) * M + NE, no = 3 * M;
   static constexpr size_t bytes(int L, int LI) {
     return sizeof(double) * ((size_t)(nd + np) * L + (size_t)no * LI);
   }
   double* base;
   int L, LI;
   unsigned* st;  // checked builds: every row and column is checked
+  D2 ial;        // SLIM: 1 / alpha
   __device__ __forceinline__ int at(int row, int rows, int k, int len) const {
 #if defined(HWENO_CHECKS) && HWENO_CHECKS
     if ((unsigned)row >= (unsigned)rows || (unsigned)k >= (unsigned)len) {
@@ -66,9 +67,15 @@ struct LineTile {
   // split pairs of side sd (0: H^+, P; 1: H^-, M)
   __device__ __forceinline__ D2& H(int sd, int c, int k) const { return p(sd * M + c, k); }
   __device__ __forceinline__ D2& X(int sd, int c, int k) const { return p((2 + sd) * M + c, k); }
-  __device__ __forceinline__ D2& dU(int c, int k) const { return p(4 * M + c, k); }
-  __device__ __forceinline__ D2& Nx(int c, int k) const { return p(5 * M + c, k); }
-  __device__ __forceinline__ D2& E(int e, int k) const { return p(6 * M + e, k); }
+  __device__ __forceinline__ D2 dU(int c, int k) const {
+    if constexpr (SLIM) return mul(sub(X(0, c, k), X(1, c, k)), ial);
+    else return p(4 * M + c, k);
+  }
+  __device__ __forceinline__ D2 Nx(int c, int k) const {
+    if constexpr (SLIM) return mul(sub(H(0, c, k), H(1, c, k)), ial);
+    else return p(5 * M + c, k);
+  }
+  __device__ __forceinline__ D2& E(int e, int k) const { return p((SLIM ? 4 : 6) * M + e, k); }
   __device__ __forceinline__ double& C(int c, int j) const { return o(c, j); }
   __device__ __forceinline__ double& D(int c, int j) const { return o(M + c, j); }
   __device__ __forceinline__ double& lim(int c, int j) const { return o(2 * M + c, j); }
@@ -102,7 +109,7 @@ __device__ __forceinline__ void point_pairs(const T& r, int k, const double* N, 
 #pragma unroll
   for (int c = 0; c < T::M; ++c) {
     const D2 nx = mul(dxp, to_pair(N[c])), x = mul(dxp, to_pair(h[c])), y = mul(alp, nx);
-    r.Nx(c, k) = nx;
+    if constexpr (!T::SLIM) r.p(5 * T::M + c, k) = nx;
     r.H(0, c, k) = scale(add(x, y), 0.5f);
     r.H(1, c, k) = scale(sub(x, y), 0.5f);
   }
@@ -127,7 +134,10 @@ template <class T>
 __device__ __forceinline__ void edge_pairs(const T& r, int k, int S, D2 alp) {
   D2 dU[T::M];
 #pragma unroll
-  for (int c = 0; c < T::M; ++c) r.dU(c, k) = dU[c] = to_pair(r.U(c, k + S) - r.U(c, k));
+  for (int c = 0; c < T::M; ++c) {
+    dU[c] = to_pair(r.U(c, k + S) - r.U(c, k));
+    if constexpr (!T::SLIM) r.p(4 * T::M + c, k) = dU[c];
+  }
 #pragma unroll
   for (int c = 0; c < T::M; ++c) {
     const D2 dF = T::EUL && c == 0 ? dU[T::kn] : to_pair(r.F(c, k + S) - r.F(c, k));

@@ -119,7 +119,7 @@ __device__ __forceinline__ void stage_tile_df(const Args1D& a, const StageIO& io
                                               const int P, const int k, const int s) {
   constexpr int M = Dim1<EQ>::M;
   extern __shared__ __align__(16) unsigned char smem1d[];
-  const Tile1D<EQ> r{reinterpret_cast<double*>(smem1d), P + 4, P + 1, a.status};
+  const Tile1D<EQ> r{reinterpret_cast<double*>(smem1d), P + 4, P + 1, a.status, D2{}};
   __shared__ double s_dt;
   __shared__ unsigned s_top;
   __shared__ int s_nf, s_nl;  // items of the lists
@@ -217,16 +217,18 @@ __device__ __forceinline__ void stage_tile_df(const Args1D& a, const StageIO& io
         static_cast<double*>(a.L2)[q] = -dD * idx2;
         if (a.Vlim) static_cast<double*>(a.Vlim)[q] = vt;
       } else {
-        double x = r.U(c, g), y = vt;
+        // b (x + dt L) first, then a x0 added in one operation: one rounding
+        // of the full value
+        double x = fma(k1, dF, b * r.U(c, g)), y = fma(k2, dD, b * vt);
         if (mode == MODE_STAGE1) {
           static_cast<double*>(io.Vt0out)[q] = vt;
         } else {
-          x = a0 * static_cast<const double*>(io.U0)[q] + b * x;
-          y = a0 * static_cast<const double*>(io.Vt0)[q] + b * y;
+          x = fma(a0, static_cast<const double*>(io.U0)[q], x);
+          y = fma(a0, static_cast<const double*>(io.Vt0)[q], y);
         }
-        un[c] = x + k1 * dF;
-        static_cast<double*>(io.Uout)[q] = un[c];
-        static_cast<double*>(io.Vout)[q] = y + k2 * dD;
+        un[c] = x;
+        static_cast<double*>(io.Uout)[q] = x;
+        static_cast<double*>(io.Vout)[q] = y;
         // kept for the wave speed below in a row that this phase does not read
         reinterpret_cast<double&>(r.H(0, c, g)) = un[c];
       }

@@ -14,9 +14,10 @@
 //           motion), adds the x parts, forms the y-limited w~, combines the
 //           SSP-RK3 stage and reduces the wave speeds of the new state.
 //
-// The FP64 pipe bounds both kernels; the scratch round trip between them is
-// a few percent of the HBM time budget and keeps each tile's shared memory
-// small enough for several CTAs per SM.
+// The scratch round trip between them is a few percent of the HBM time budget
+// and keeps each tile's shared memory small enough for several CTAs per SM.
+// The kernels in this file run FP32 states; stage2d_df.cuh holds the sweeps of
+// FP64 states, which the FP64 pipe would bound in this form.
 #include <algorithm>
 #include <cfloat>
 
@@ -27,6 +28,7 @@
 #include "stage2d_common.cuh"
 #include "hweno_math.cuh"
 #include "internal.h"
+#include "line_df.cuh"
 
 namespace hweno {
 namespace {
@@ -633,6 +635,8 @@ __global__ void __launch_bounds__(kThreads2D, (MinBlocks<Real, HWENO_MINB_Y_F64,
   }
 }
 
+#include "stage2d_df.cuh"
+
 template <int EQ, class Real, int MODE>
 cudaError_t ysweep_launch(const Args2D& a, cudaStream_t s) {
   constexpr size_t bytes = YLayout<EQ, Real>::bytes;
@@ -645,7 +649,8 @@ cudaError_t ysweep_launch(const Args2D& a, cudaStream_t s) {
 
 template <int EQ, class Real>
 cudaError_t ysweep_mode(int mode, const Args2D& a, cudaStream_t s) {
-  switch (mode) {
+  if constexpr (std::is_same<Real, double>::value) return ysweep_f64<EQ>(mode, a, s);
+  else switch (mode) {
     case MODE_RHS: return ysweep_launch<EQ, Real, MODE_RHS>(a, s);
     case MODE_STAGE1: return ysweep_launch<EQ, Real, MODE_STAGE1>(a, s);
     case MODE_STAGE2: return ysweep_launch<EQ, Real, MODE_STAGE2>(a, s);
@@ -655,10 +660,14 @@ cudaError_t ysweep_mode(int mode, const Args2D& a, cudaStream_t s) {
 
 template <int EQ, class Real>
 cudaError_t xsweep_mode(int mode, const Args2D& a, cudaStream_t s) {
+  if constexpr (std::is_same<Real, double>::value) {
+    return xsweep_f64<EQ>(mode, a, s);
+  } else {
   const dim3 grid((a.nx + kTileX2D - 1) / kTileX2D, a.ny);
   if (mode == MODE_STAGE1) k_xsweep_2d<EQ, Real, MODE_STAGE1><<<grid, kThreads2D, 0, s>>>(a);
   else k_xsweep_2d<EQ, Real, MODE_RHS><<<grid, kThreads2D, 0, s>>>(a);
   return cudaGetLastError();
+  }
 }
 
 }  // namespace

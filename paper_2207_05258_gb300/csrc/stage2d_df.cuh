@@ -1,0 +1,378 @@
+// The two sweeps of a 2D stage for FP64 states (included by stage2d.cu, which
+// describes the sweeps): FP64 for what the result's last bits depend on,
+// pairs of FP32 numbers for the corrections (line_df.cuh, weno_df.cuh), the
+// items whose correction is not small listed and evaluated in FP64.
+//
+// What bounds them: an all-FP64 stage (x- and y-sweep) needs about 2 200 FP64
+// instructions per point at 65 to 77 cycles per warp and sub-partition; here
+// about 400 remain, next to about 17 000 FP32 instructions. Measured: double
+// Mach 1920 x 480, 13.2 -> 4.09 ms per step (FP64 pipe 86% -> 60% busy); 256^2,
+// 1.06 -> 0.37 ms per step; Burgers rhs 321 x 203, 95 -> 50 us.
+//
+// Tiles: the x-sweep takes row segments of 124 points. The y-sweep takes
+// blocks of 4 columns x 31 rows: 35 rows loaded for 31 (16 columns x 7 rows
+// load 11 for 7, and the point phase is FP64 work), while the 4 columns are
+// one 32-byte sector of a row. Both give 128 interfaces, one per thread, and
+// 51 to 55 KB of shared memory, four CTAs per SM.
+
+constexpr int kColsF64 = 4, kRowsF64 = kThreads2D / kColsF64 - 1;
+
+template <int EQ, int DIR>
+using Tile2D = LineTile<Dim2<EQ>::M, DIR, EQ == HWENO_EULER, Dim2<EQ>::M, true>;
+
+struct Lists2D {  // items evaluated in FP64
+  int nf, nl;
+  unsigned short f[kThreads2D], l[kThreads2D];
+};
+
+// Phase 1, loaded point k: state u, the derivatives v along and w across the
+// line; stores the flux, the two Jacobian-vector products and the pairs.
+template <int EQ, int DIR>
+__device__ __forceinline__ void load_point_2d(const Tile2D<EQ, DIR>& r, int k, const double* u,
+                                              const double* v, const double* w, double gm1,
+                                              D2 alp, D2 hp) {
+  constexpr int M = Dim2<EQ>::M;
+  double F[M], h[M], E[M];
+  Prim2<double> q{};
+  if constexpr (EQ == HWENO_EULER) q = prim2_ir(u, gm1, recip_fp64(u[0]));
+  flux2<EQ, DIR>(u, q, F);
+  jvp2<EQ, DIR>(u, q, v, gm1, h);
+  jvp2<EQ, DIR>(u, q, w, gm1, E);
+#pragma unroll
+  for (int c = 0; c < M; ++c) {
+    r.U(c, k) = u[c];
+    r.N(c, k) = v[c];
+    if (EQ != HWENO_EULER || c > 0) {
+      r.F(c, k) = F[c];
+      r.h(c, k) = h[c];
+    }
+    r.extra(c, k) = E[c];
+  }
+  if constexpr (EQ == HWENO_EULER)
+    point_eigen(r, k, u[0], q.ir, q.Ep, DIR == 0 ? q.u : q.v, DIR == 0 ? q.v : q.u);
+  point_pairs(r, k, v, h, alp, hp);
+}
+
+// Phase 3 of one thread: interface j (left point kf) and limiter point j
+// (point kl), where there are such.
+template <int EQ, int DIR>
+__device__ __forceinline__ void items_2d(const Tile2D<EQ, DIR>& r, int j, bool has_f, int kf,
+                                         bool has_l, int kl, int S, double alpha, double dx,
+                                         double idx, const SchemeParams& sp, Lists2D& ls) {
+  constexpr int M = Dim2<EQ>::M;
+  double x[M];
+  if (has_f) {
+    // (the mean state's eigenvectors are taken in FP64)
+    if (!((M == 1 || sp.eig_avg == 0) && interface_line<D2, DIR>(r, kf, S, alpha, dx, sp, x)))
+      ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
+    const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      r.C(c, j) = x[c];
+      r.D(c, j) = derivative_flux_fp64(r, c, kf, S, kU, kh, kv);
+    }
+  }
+  if (has_l && sp.limiter != 0) {
+    if (!limiter_line<D2, DIR>(r, kl, S, dx, idx, sp, x))
+      ls.l[atomicAdd(&ls.nl, 1)] = (unsigned short)j;
+#pragma unroll
+    for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
+  }
+}
+
+// The differences of a point k between interfaces ja and jb: of f-hat, of the
+// derivative flux, and of the central flux of Eq. mixed (times 12).
+template <int EQ, int DIR>
+__device__ __forceinline__ void differences_2d(const Tile2D<EQ, DIR>& r, int c, int k, int S,
+                                               int ja, int jb, double& dF, double& dD,
+                                               double& dE) {
+  dF = fma(0.5, r.F(c, k + S) - r.F(c, k - S), r.C(c, jb) - r.C(c, ja));
+  dD = r.D(c, jb) - r.D(c, ja);
+  dE = fma(8.0, r.extra(c, k + S) - r.extra(c, k - S),
+           r.extra(c, k - 2 * S) - r.extra(c, k + 2 * S));
+}
+
+template <int EQ>
+__global__ void __launch_bounds__(kThreads2D, HWENO_MINB_2D_F64)
+k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
+  constexpr int M = Dim2<EQ>::M;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ Lists2D ls;
+  if (a.skip_done && !(a.t[0] < a.t_end)) return;
+  const int nx = a.nx;
+  const long long N = (long long)nx * a.ny;
+  // block -> (row segment, row): the full segments of every row first, the
+  // ragged last segments (shorter work) at the end of the dispatch order
+  int tile = blockIdx.x, row_ = blockIdx.y;
+  {
+    const int T = gridDim.x, F = T - 1;
+    if (F > 0 && nx % kTileX2D != 0) {
+      const long long b = (long long)blockIdx.y * T + blockIdx.x, full = (long long)a.ny * F;
+      if (b < full) { tile = (int)(b % F); row_ = (int)(b / F); }
+      else { tile = F; row_ = (int)(b - full); }
+    }
+  }
+  const int i0 = tile * kTileX2D, np = min(kTileX2D, nx - i0);
+  HWENO_CHECK(np >= 1 && row_ >= 0 && row_ < a.ny, a.status);
+  const long long row = (long long)row_ * nx;
+  const double dx = a.geod[0], idx = a.geod[1], idx2 = a.geod[2];
+  const double alpha = a.alpha_in[0], gm1 = a.sp.wd[9] - 1.0;
+  if (threadIdx.x == 0) {
+    ls.nf = ls.nl = 0;
+    if (mode == MODE_STAGE1 && blockIdx.x == 0 && blockIdx.y == 0) {
+      int lands;
+      const double dt = time_step2(a, lands);
+      a.dt[0] = dt;
+      a.lands[0] = lands;
+    }
+  }
+  const D2 alp = scale_pair(alpha), hp = to_pair(dx);
+  const Tile2D<EQ, 0> r{reinterpret_cast<double*>(smem_raw), kTileX2D + 4, kTileX2D + 1, a.status,
+                        div(D2{1.f, 0.f}, alp)};
+
+  // 1: points
+  for (int g = threadIdx.x; g < np + 4; g += kThreads2D) {
+    const Src s = map_x(i0 - 2 + g, nx, a.sp);
+    HWENO_CHECK(s.kind == 2 || (s.idx >= 0 && s.idx < nx), a.status);
+    double u[M], v[M], w[M];
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      if (s.kind == 2) {
+        u[c] = imposed(a.sp, s, c);
+        v[c] = w[c] = 0.0;
+      } else {
+        const long long q = c * N + row + s.idx;
+        u[c] = static_cast<const double*>(a.U)[q];
+        v[c] = static_cast<const double*>(a.V)[q];
+        w[c] = static_cast<const double*>(a.W)[q];
+        if (s.kind == 1) {
+          if (refl2<EQ, 0>(c) < 0.f) { u[c] = -u[c]; w[c] = -w[c]; }
+          else v[c] = -v[c];
+        }
+      }
+    }
+    load_point_2d<EQ, 0>(r, g, u, v, w, gm1, alp, hp);
+  }
+  __syncthreads();
+  // 2: edges
+  for (int g = threadIdx.x; g < np + 3; g += kThreads2D) edge_pairs(r, g, 1, alp);
+  __syncthreads();
+  // 3: interfaces and limiter
+  {
+    const int j = threadIdx.x;
+    items_2d<EQ, 0>(r, j, j <= np, j + 1, j < np, j + 2, 1, alpha, dx, idx, a.sp, ls);
+  }
+  __syncthreads();
+  if (ls.nf + ls.nl > 0) {
+    listed_items<0>(r, ls.f, ls.nf, ls.l, ls.nl,
+                    [](int j, bool lim) { return lim ? j + 2 : j + 1; }, 1, tile + row_, alpha, dx,
+                    idx, a.sp);
+    __syncthreads();
+  }
+  // 4: the x parts
+  if (threadIdx.x < np) {
+    const int j = threadIdx.x, k = j + 2;
+    HWENO_CHECK(i0 + j < nx, a.status);
+    const long long q = row + i0 + j;
+    double* LX = static_cast<double*>(a.LX);
+    double* VT = static_cast<double*>(a.VT);
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      double dF, dD, dE;
+      differences_2d<EQ, 0>(r, c, k, 1, j, j + 1, dF, dD, dE);
+      LX[c * N + q] = -dF * idx;
+      LX[(M + c) * N + q] = -dD * idx2;
+      LX[(2 * M + c) * N + q] = dE * (idx * (-1.0 / 12.0));
+      VT[c * N + q] = a.sp.limiter ? r.lim(c, j) : r.N(c, k);
+    }
+  }
+}
+
+// FP32 bounds of the two wave speeds as rough_speed in 1D.
+template <int EQ>
+__device__ __forceinline__ void rough_speeds2(const double* u, float gam, float& sx, float& sy) {
+  if constexpr (EQ == HWENO_BURGERS) {
+    sx = sy = fabsf(to_float(u[0]));
+  } else {
+    const float r = to_float(u[0]), m = to_float(u[1]), n = to_float(u[2]), E = to_float(u[3]);
+    const float ir = 1.f / r, e = E - 0.5f * (m * m + n * n) * ir;
+    const float c = sqrtf(gam * (gam - 1.f) * e * ir);
+    const bool ok = e >= 0.00390625f * E;
+    sx = ok ? fabsf(m * ir) + c : __int_as_float(0x7fc00000);
+    sy = ok ? fabsf(n * ir) + c : __int_as_float(0x7fc00000);
+  }
+}
+
+template <int EQ>
+__global__ void __launch_bounds__(kThreads2D, HWENO_MINB_2D_F64)
+k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
+  constexpr int M = Dim2<EQ>::M;
+  constexpr int C = kColsF64, R = kRowsF64, L = (R + 4) * C;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ Lists2D ls;
+  __shared__ unsigned s_top[2];
+  if (a.skip_done && !(a.t[0] < a.t_end)) return;
+  const int nx = a.nx, ny = a.ny;
+  const long long N = (long long)nx * ny;
+  const int i0 = blockIdx.x * C, j0 = blockIdx.y * R;
+  const int ncol = min(C, nx - i0), nrow = min(R, ny - j0);
+  HWENO_CHECK(ncol >= 1 && nrow >= 1, a.status);
+  const double dy = a.geod[3], idy = a.geod[4], idy2 = a.geod[5];
+  const double alpha = a.alpha_in[1], gm1 = a.sp.wd[9] - 1.0;
+  if (threadIdx.x == 0) {
+    ls.nf = ls.nl = 0;
+    s_top[0] = s_top[1] = 0u;
+  }
+  // the stage's time step (stage 1: written by the x-sweep before it) and
+  // boundary time
+  const double dt = mode == MODE_RHS ? 0.0 : a.dt[0];
+  const D2 alp = scale_pair(alpha), hp = to_pair(dy);
+  const Tile2D<EQ, 1> r{reinterpret_cast<double*>(smem_raw), L, (R + 1) * C, a.status,
+                        div(D2{1.f, 0.f}, alp)};
+
+  // 1: points
+  for (int k = threadIdx.x; k < L; k += kThreads2D) {
+    const int rr = k / C, col = k % C, i = i0 + col;
+    if (col >= ncol || rr >= nrow + 4) continue;
+    const int jj = j0 - 2 + rr;
+    Src s{jj, 0, 0};
+    if (jj < 0 || jj >= ny)
+      s = map_y(jj, ny, i, a.x0, a.dx, a.y0, a.dy, __dadd_rn(a.t[0], __dmul_rn(a.stage_c, dt)),
+                a.sp);
+    HWENO_CHECK(s.kind == 2 || (s.idx >= 0 && s.idx < ny && i < nx), a.status);
+    double u[M], v[M], w[M];
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      if (s.kind == 2) {
+        u[c] = imposed(a.sp, s, c);
+        v[c] = w[c] = 0.0;
+      } else {
+        const long long q = c * N + (long long)s.idx * nx + i;
+        u[c] = static_cast<const double*>(a.U)[q];
+        v[c] = static_cast<const double*>(a.V)[q];
+        w[c] = static_cast<const double*>(a.W)[q];
+        if (s.kind == 1) {
+          if (refl2<EQ, 1>(c) < 0.f) { u[c] = -u[c]; v[c] = -v[c]; }
+          else w[c] = -w[c];
+        }
+      }
+    }
+    load_point_2d<EQ, 1>(r, k, u, w, v, gm1, alp, hp);
+  }
+  __syncthreads();
+  // 2: edges
+  for (int k = threadIdx.x; k < (R + 3) * C; k += kThreads2D)
+    if (k % C < ncol && k / C < nrow + 3) edge_pairs(r, k, C, alp);
+  __syncthreads();
+  // 3: interfaces y_{j0+r-1/2}, r = 0..nrow (lower point in loaded row r + 1),
+  // and the limiter of the points of row r (loaded row r + 2)
+  {
+    const int j = threadIdx.x, rr = j / C;
+    const bool in = j % C < ncol;
+    items_2d<EQ, 1>(r, j, in && rr <= nrow, j + C, in && rr < nrow, j + 2 * C, C, alpha, dy, idy,
+                    a.sp, ls);
+  }
+  __syncthreads();
+  if (ls.nf + ls.nl > 0) {
+    listed_items<1>(r, ls.f, ls.nf, ls.l, ls.nl,
+                    [](int j, bool lim) { return lim ? j + 2 * C : j + C; }, C,
+                    blockIdx.x + blockIdx.y, alpha, dy, idy, a.sp);
+    __syncthreads();
+  }
+  // 4: the y parts, the Runge-Kutta combination
+  const int j = threadIdx.x, rr = j / C, k = j + 2 * C;
+  const bool mine = j % C < ncol && rr < nrow;
+  const bool want_alpha = mode == MODE_STAGE1 || mode == MODE_STAGE2;
+  double un[M];
+  float fx = 0.f, fy = 0.f;
+  if (mine) {
+    HWENO_CHECK(j0 + rr < ny && i0 + j % C < nx, a.status);
+    const long long q = (long long)(j0 + rr) * nx + i0 + j % C;
+    const double* LX = static_cast<const double*>(a.LX);
+    const double* VT = static_cast<const double*>(a.VT);
+    const double b = mode == MODE_STAGE1 ? 1.0 : mode == MODE_STAGE2 ? 0.25 : 2.0 / 3.0;
+    const double a0 = mode == MODE_STAGE2 ? 0.75 : 1.0 / 3.0;
+    const double bdt = b * dt;
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      const long long qc = c * N + q;
+      double dG, dT, dX;
+      differences_2d<EQ, 1>(r, c, k, C, j, j + C, dG, dT, dX);
+      const double l1 = fma(-idy, dG, LX[qc]), l3 = fma(-idy2, dT, LX[(2 * M) * N + qc]);
+      const double l2 = fma(idy * (-1.0 / 12.0), dX, LX[M * N + qc]);
+      const double vt = VT[qc], wt = a.sp.limiter ? r.lim(c, j) : r.N(c, k);
+      if (mode == MODE_RHS) {
+        static_cast<double*>(a.L1)[qc] = l1;
+        static_cast<double*>(a.L2)[qc] = l2;
+        static_cast<double*>(a.L3)[qc] = l3;
+        if (a.Wlim) static_cast<double*>(a.Wlim)[qc] = wt;
+      } else {
+        // b (x + dt L) first, then a x0 added in one operation: one rounding
+        // of the full value
+        double x = fma(bdt, l1, b * r.U(c, k)), y = fma(bdt, l2, b * vt), z = fma(bdt, l3, b * wt);
+        if (mode == MODE_STAGE1) {
+          static_cast<double*>(a.Wt0out)[qc] = wt;
+        } else {
+          x = fma(a0, static_cast<const double*>(a.U0)[qc], x);
+          y = fma(a0, static_cast<const double*>(a.Vt0)[qc], y);
+          z = fma(a0, static_cast<const double*>(a.Wt0)[qc], z);
+        }
+        un[c] = x;
+        static_cast<double*>(a.Uout)[qc] = x;
+        static_cast<double*>(a.Vout)[qc] = y;
+        static_cast<double*>(a.Wout)[qc] = z;
+      }
+    }
+    if (want_alpha) rough_speeds2<EQ>(un, a.sp.wf[9], fx, fy);
+  }
+  // wave speeds of the new state: in FP64 only where the FP32 ones come
+  // within 2^-9 of the tile's largest (or are not usable)
+  if (want_alpha) {
+    const unsigned tx = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fx, 0.f)));
+    const unsigned ty = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fy, 0.f)));
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&s_top[0], tx);
+      atomicMax(&s_top[1], ty);
+    }
+    __syncthreads();
+    const float topx = __uint_as_float(s_top[0]) * (1.f - 0x1p-9f);
+    const float topy = __uint_as_float(s_top[1]) * (1.f - 0x1p-9f);
+    double ax = 0.0, ay = 0.0;
+    if (mine && !(fx < topx && fy < topy)) {
+      double sx, sy;
+      speeds2<EQ>(un, a.sp.wd[9], sx, sy);
+      if (!(sx <= real_max<double>()) || !(sy <= real_max<double>()))
+        atomicOr(a.status, STATUS_NONFINITE);
+      ax = fmax(ax, sx);
+      ay = fmax(ay, sy);
+    }
+    if (__any_sync(0xffffffffu, ax > 0.0 || ay > 0.0)) {
+      const unsigned long long mx = warp_max_bits(ax), my = warp_max_bits(ay);
+      if ((threadIdx.x & 31) == 0) {
+        atomicMax(&a.alpha_out[0], mx);
+        atomicMax(&a.alpha_out[1], my);
+      }
+    }
+  }
+}
+
+template <int EQ>
+cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
+  constexpr size_t bytes = Tile2D<EQ, 0>::bytes(kTileX2D + 4, kTileX2D + 1);
+  static unsigned configured = 0;  // devices whose limit is raised
+  if (const cudaError_t e = ensure_smem_limit(k_xsweep_2d_f64<EQ>, bytes, configured)) return e;
+  const dim3 grid((a.nx + kTileX2D - 1) / kTileX2D, a.ny);
+  k_xsweep_2d_f64<EQ><<<grid, kThreads2D, bytes, s>>>(a, mode);
+  return cudaGetLastError();
+}
+
+template <int EQ>
+cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
+  constexpr size_t bytes =
+      Tile2D<EQ, 1>::bytes((kRowsF64 + 4) * kColsF64, (kRowsF64 + 1) * kColsF64);
+  static unsigned configured = 0;  // devices whose limit is raised
+  if (const cudaError_t e = ensure_smem_limit(k_ysweep_2d_f64<EQ>, bytes, configured)) return e;
+  const dim3 grid((a.nx + kColsF64 - 1) / kColsF64, (a.ny + kRowsF64 - 1) / kRowsF64);
+  k_ysweep_2d_f64<EQ><<<grid, kThreads2D, bytes, s>>>(a, mode);
+  return cudaGetLastError();
+}
