@@ -142,6 +142,15 @@ __device__ __forceinline__ double square(double a) { return __dmul_rn(a, a); }
 __device__ __forceinline__ double scale(double a, double p2) { return __dmul_rn(a, p2); }
 __device__ __forceinline__ double abs2(double a) { return fabs(a); }
 
+// c ? -a : a
+__device__ __forceinline__ D2 flip(bool c, D2 a) { return c ? neg(a) : a; }
+__device__ __forceinline__ double flip(bool c, double a) { return c ? -a : a; }
+// a b + c for a power of two a
+__device__ __forceinline__ D2 scale_add(D2 b, float a, D2 c) { return add(scale(b, a), c); }
+__device__ __forceinline__ double scale_add(double b, double a, double c) {
+  return __fma_rn(b, a, c);
+}
+
 // c ? a : b, word by word
 __device__ __forceinline__ D2 pick2(bool c, D2 a, D2 b) {
   return D2{c ? a.h : b.h, c ? a.l : b.l};
@@ -167,12 +176,6 @@ template <>
 struct Num<double> {
   using Scale = double;
   static __device__ __forceinline__ constexpr double c(double x) { return x; }
-  static __device__ __forceinline__ double lead(double x) { return x; }
-  static __device__ __forceinline__ void exponent(double x, double& up, double& down) {
-    const int e = __double2hiint(x) & 0x7ff00000;
-    up = __hiloint2double(e, 0);
-    down = __hiloint2double((2046 << 20) - e, 0);
-  }
 };
 
 }  // namespace hweno

@@ -30,7 +30,7 @@ struct LineTile {
   static constexpr int NE = EUL ? M : 0;
   static constexpr int MF = EUL ? M - 1 : M;  // stored rows of F and h
   static constexpr int nd = 2 * M + 2 * MF + MX, np = (SLIM ? 4 : 6) * M + NE, no = 3 * M;
-  static constexpr size_t bytes(int L, int LI) {
+  __host__ __device__ static constexpr size_t bytes(int L, int LI) {
     return sizeof(double) * ((size_t)(nd + np) * L + (size_t)no * LI);
   }
   double* base;
@@ -75,6 +75,7 @@ struct LineTile {
     if constexpr (SLIM) return mul(sub(H(0, c, k), H(1, c, k)), ial);
     else return p(5 * M + c, k);
   }
+  // eigen-system inputs: sqrt(rho), un, H, ut
   __device__ __forceinline__ D2& E(int e, int k) const { return p((SLIM ? 4 : 6) * M + e, k); }
   __device__ __forceinline__ double& C(int c, int j) const { return o(c, j); }
   __device__ __forceinline__ double& D(int c, int j) const { return o(M + c, j); }
@@ -101,18 +102,21 @@ __device__ __forceinline__ D2 scale_pair(double x) {
   return r;
 }
 
-// The pairs of point k from the derivative N and h = A N of its state:
-// H^{+-} = dx (h +- alpha N) / 2 and dx N.
+// The pairs of point k, component c, from the derivative N and h = A N of its
+// state: H^{+-} = dx (h +- alpha N) / 2 and dx N.
+template <class T>
+__device__ __forceinline__ void point_pair(const T& r, int c, int k, double N, double h, D2 alp,
+                                           D2 dxp) {
+  const D2 nx = mul(dxp, to_pair(N)), x = mul(dxp, to_pair(h)), y = mul(alp, nx);
+  if constexpr (!T::SLIM) r.p(5 * T::M + c, k) = nx;
+  r.H(0, c, k) = scale(add(x, y), 0.5f);
+  r.H(1, c, k) = scale(sub(x, y), 0.5f);
+}
 template <class T>
 __device__ __forceinline__ void point_pairs(const T& r, int k, const double* N, const double* h,
                                             D2 alp, D2 dxp) {
 #pragma unroll
-  for (int c = 0; c < T::M; ++c) {
-    const D2 nx = mul(dxp, to_pair(N[c])), x = mul(dxp, to_pair(h[c])), y = mul(alp, nx);
-    if constexpr (!T::SLIM) r.p(5 * T::M + c, k) = nx;
-    r.H(0, c, k) = scale(add(x, y), 0.5f);
-    r.H(1, c, k) = scale(sub(x, y), 0.5f);
-  }
+  for (int c = 0; c < T::M; ++c) point_pair(r, c, k, N[c], h[c], alp, dxp);
 }
 
 // The eigen-system's inputs at point k from rho, 1/rho, E + p and the
@@ -121,26 +125,32 @@ template <class T>
 __device__ __forceinline__ void point_eigen(const T& r, int k, double rho, double ir, double Ep,
                                             double un, double ut) {
   const D2 rp = scale_pair(rho);
-  const D2 up = to_pair(un), tp = T::M == 4 ? to_pair(ut) : D2{};
-  const D2 H = mul(to_pair(Ep), to_pair(ir));
   r.E(0, k) = mul(rp, rsqrt2(rp));
-  r.E(1, k) = up;
-  r.E(2, k) = H;
-  if constexpr (T::M == 4) r.E(3, k) = tp;
+  r.E(1, k) = to_pair(un);
+  r.E(2, k) = mul(to_pair(Ep), to_pair(ir));
+  if constexpr (T::M == 4) r.E(3, k) = to_pair(ut);
 }
 
-// The edge between points k and k + S.
+// Component c of the edge between points k and k + S.
+template <class T>
+__device__ __forceinline__ void edge_pair(const T& r, int c, int k, int S, D2 alp) {
+  const D2 dU = to_pair(sub(r.U(c, k + S), r.U(c, k)));
+  const D2 dF = to_pair(sub(r.F(c, k + S), r.F(c, k))), au = mul(alp, dU);
+  if constexpr (!T::SLIM) r.p(4 * T::M + c, k) = dU;
+  r.X(0, c, k) = scale(add(dF, au), 0.5f);
+  r.X(1, c, k) = scale(sub(dF, au), 0.5f);
+}
 template <class T>
 __device__ __forceinline__ void edge_pairs(const T& r, int k, int S, D2 alp) {
   D2 dU[T::M];
 #pragma unroll
   for (int c = 0; c < T::M; ++c) {
-    dU[c] = to_pair(r.U(c, k + S) - r.U(c, k));
+    dU[c] = to_pair(sub(r.U(c, k + S), r.U(c, k)));
     if constexpr (!T::SLIM) r.p(4 * T::M + c, k) = dU[c];
   }
 #pragma unroll
   for (int c = 0; c < T::M; ++c) {
-    const D2 dF = T::EUL && c == 0 ? dU[T::kn] : to_pair(r.F(c, k + S) - r.F(c, k));
+    const D2 dF = T::EUL && c == 0 ? dU[T::kn] : to_pair(sub(r.F(c, k + S), r.F(c, k)));
     const D2 au = mul(alp, dU[c]);
     r.X(0, c, k) = scale(add(dF, au), 0.5f);
     r.X(1, c, k) = scale(sub(dF, au), 0.5f);
@@ -210,29 +220,31 @@ struct LineData<double, T> {
     }
     H = mul(madd(gm1(), madd(-0.5, ke, u[M - 1]), u[M - 1]), ir);
   }
-  __device__ __forceinline__ void state(int k, bool edge, double& un, double& ut, double& H) const {
-    constexpr int M = T::M;
-    double a[M], b[M];
+  // point k's velocities and enthalpy
+  __device__ __forceinline__ void prim_at(int k, double& un, double& ut, double& H) const {
+    double a[T::M];
 #pragma unroll
-    for (int c = 0; c < M; ++c) {
-      a[c] = r.U(c, k);
-      b[c] = edge ? r.U(c, k + S) : 0.0;
-    }
+    for (int c = 0; c < T::M; ++c) a[c] = r.U(c, k);
+    prim(a, un, ut, H);
+  }
+  __device__ __forceinline__ void state(int k, bool edge, double& un, double& ut, double& H) const {
     if (!edge) {
-      prim(a, un, ut, H);
+      prim_at(k, un, ut, H);
     } else if (sp.eig_avg == 0) {  // Roe average
       double uL, tL = 0.0, HL, uR, tR = 0.0, HR;
-      prim(a, uL, tL, HL);
-      prim(b, uR, tR, HR);
-      const double sl = mul(a[0], rsqrt_fp64(a[0])), sr = mul(b[0], rsqrt_fp64(b[0]));
+      prim_at(k, uL, tL, HL);
+      prim_at(k + S, uR, tR, HR);
+      const double sl = mul(r.U(0, k), rsqrt_fp64(r.U(0, k)));
+      const double sr = mul(r.U(0, k + S), rsqrt_fp64(r.U(0, k + S)));
       const double is = recip_fp64(add(sl, sr));
       auto roe = [&](double x, double y) { return mul(add(mul(sl, x), mul(sr, y)), is); };
       un = roe(uL, uR);
       ut = roe(tL, tR);
       H = roe(HL, HR);
     } else {  // arithmetic mean state
+      double a[T::M];
 #pragma unroll
-      for (int c = 0; c < M; ++c) a[c] = mul(0.5, add(a[c], b[c]));
+      for (int c = 0; c < T::M; ++c) a[c] = mul(0.5, add(r.U(c, k), r.U(c, k + S)));
       prim(a, un, ut, H);
     }
   }
@@ -253,68 +265,115 @@ template <class X, class T>
 __device__ __forceinline__ void side_differences(const LineData<X, T>& in, int sd, int c, int k,
                                                  int S, X* x) {
   using P2 = typename Num<X>::Scale;
-  const P2 sg = sd ? P2(-1) : P2(1);
+  const bool sg = sd != 0;
   const int k0 = sd ? k + S : k, km = sd ? k0 + S : k0 - S, kp = sd ? k : k0 + S;
   // the edges (k - S, k), (k, k + S) or (k + S, k + 2 S), (k, k + S)
   const X Hm = in.H(sd, c, km), H0 = in.H(sd, c, k0), Hp = in.H(sd, c, kp);
-  x[0] = scale(sub(H0, in.X(sd, c, sd ? k0 : km)), sg);
-  x[1] = scale(sub(H0, in.X(sd, c, k)), sg);
-  x[2] = scale(sub(add(Hm, Hp), scale(H0, P2(2))), sg);
-  x[3] = scale(sub(Hm, Hp), sg);
-  x[4] = scale(H0, sg);
+  x[0] = flip(sg, sub(H0, in.X(sd, c, sd ? k0 : km)));
+  x[1] = flip(sg, sub(H0, in.X(sd, c, k)));
+  x[2] = flip(sg, scale_add(H0, P2(-2), add(Hm, Hp)));
+  x[3] = flip(sg, sub(Hm, Hp));
+  x[4] = flip(sg, H0);
 }
 
-// c of the interface between points k and k + S; in pairs, false when the
-// correction is not small (the values are then not to be used).
-template <class X, int DIR, class T>
-__device__ __forceinline__ bool interface_line(const T& r, int k, int S, double alpha, double dx,
-                                               const SchemeParams& sp, double* cc) {
-  constexpr int M = T::M;
-  constexpr bool FP64 = std::is_same<X, double>::value;
-  const LineData<X, T> in(r, S, alpha, dx, sp);
-  const LineWeights<X> w = line_weights<X>(sp, false);
-  bool weak = true;
-  LineChar<X, M == 1 ? 3 : M, M == 1 ? 0 : DIR> ch;
+template <class T, class X, int DIR>
+using CharOf = LineChar<X, T::M == 1 ? 3 : T::M, T::M == 1 ? 0 : DIR>;
+
+// The characteristic system of the interface between k and k + S (`edge`) or
+// of point k.
+template <int DIR, class X, class T>
+__device__ __forceinline__ CharOf<T, X, DIR> char_system(const LineData<X, T>& in, int k,
+                                                         bool edge) {
+  CharOf<T, X, DIR> ch;
   if constexpr (T::EUL) {
     X un, ut{}, H;
-    in.state(k, true, un, ut, H);
+    in.state(k, edge, un, ut, H);
     const X q = ch.kinetic(un, ut);
     ch.init(un, ut, H, q, mul(in.gm1(), sub(H, q)), in.gm1());
   }
-  auto side = [&](X y1, X y2, X s, X d, X H0) {
-    if constexpr (FP64) return side_value(y1, y2, s, d, H0, w);
-    else return side_correction(y1, y2, s, d, H0, w, weak);
-  };
-  X f[M], lin[M];
-#pragma unroll
-  for (int c = 0; c < M; ++c) f[c] = lin[c] = X{};
-#pragma unroll 1
-  for (int sd = 0; sd < 2; ++sd) {
-    X x[M][5];
-#pragma unroll
-    for (int c = 0; c < M; ++c) {
-      side_differences(in, sd, c, k, S, x[c]);
-      if constexpr (!FP64) lin[c] = add(lin[c], linear_part(x[c][0], x[c][1], x[c][3]));
-    }
-    if constexpr (T::EUL) {
-      typename decltype(ch)::Factors a[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        X y[M];
-#pragma unroll
-        for (int c = 0; c < M; ++c) y[c] = x[c][v];
-        a[v] = ch.factors(y);
-      }
-#pragma unroll 1
-      for (int q = 0; q < M; ++q) {
-        const X y = side(a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q), a[4].field(q));
-#pragma unroll
-        for (int c = 0; c < M; ++c) f[c] = add_if(q == c, f[c], y);
-      }
+  return ch;
+}
+
+// Adds side sd of the interface between k and k + S to the characteristic
+// fields f (pairs: 12 times the corrections; FP64: the side's values) and, in
+// pairs, to 60 times the linear parts; returns, in pairs, 12 times the sum of
+// the fields' bounds of side_correction in units of the density. ONE: field
+// q0 alone, to f[0].
+template <int DIR, bool ONE = false, class X, class T>
+__device__ __forceinline__ float interface_side(const LineData<X, T>& in,
+                                                const CharOf<T, X, DIR>& ch,
+                                                const LineWeights<X>& w, int sd, int k, int S,
+                                                X* f, X* lin, int q0 = 0) {
+  constexpr int M = T::M;
+  constexpr bool FP64 = std::is_same<X, double>::value;
+  float sum = 0.f;
+  auto side = [&](int q, X y1, X y2, X s, X d, X H0) {
+    if constexpr (FP64) {
+      return side_value(y1, y2, s, d, H0, w);
     } else {
-      f[0] = add(f[0], side(x[0][0], x[0][1], x[0][2], x[0][3], x[0][4]));
+      float e = 0.f;
+      const D2 v = side_correction(y1, y2, s, d, H0, w, e);
+      sum += T::EUL ? ch.density_units(q, e) : e;
+      return v;
     }
+  };
+  X x[M][5];
+#pragma unroll
+  for (int c = 0; c < M; ++c) {
+    side_differences(in, sd, c, k, S, x[c]);
+    if constexpr (!FP64) lin[c] = add(lin[c], linear_part(x[c][0], x[c][1], x[c][3]));
   }
+  if constexpr (T::EUL) {
+    typename CharOf<T, X, DIR>::Factors a[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      X y[M];
+#pragma unroll
+      for (int c = 0; c < M; ++c) y[c] = x[c][v];
+      a[v] = ch.factors(y);
+    }
+    if constexpr (ONE) {
+      f[0] = side(q0, a[0].field(q0), a[1].field(q0), a[2].field(q0), a[3].field(q0),
+                  a[4].field(q0));
+      return sum;
+    }
+#pragma unroll 1
+    for (int q = 0; q < M; ++q) {
+      const X y = side(q, a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q),
+                       a[4].field(q));
+#pragma unroll
+      for (int c = 0; c < M; ++c) f[c] = add_if(q == c, f[c], y);
+    }
+  } else {
+    f[0] = add(f[0], side(0, x[0][0], x[0][1], x[0][2], x[0][3], x[0][4]));
+  }
+  return sum;
+}
+
+// Whether the interface between k and k + S, of whose bounds `e` is the sum
+// over both sides, may be taken in pairs: e = 0, or small against alpha times
+// the smaller of the two densities (scalar equations: values).
+template <class T>
+__device__ __forceinline__ bool interface_weak(const T& r, int k, int S, float e, double alpha,
+                                               const SchemeParams& sp) {
+  if (T::M > 1 && sp.eig_avg != 0) return false;  // (the mean state is taken in FP64)
+  float level;
+  if constexpr (T::EUL) {
+    const float s = fminf(r.E(0, k).h, r.E(0, k + S).h);
+    level = s * s;
+  } else {
+    level = fminf(fabsf(to_float(r.U(0, k))), fabsf(to_float(r.U(0, k + S))));
+  }
+  // (false for a NaN: of e, or of a level or alpha outside the pairs' range)
+  return e <= 12.f * kWeakLevel * scale_pair(alpha).h * level;
+}
+
+// c from the sums over both sides.
+template <int DIR, class X, class T>
+__device__ __forceinline__ void interface_value(const LineData<X, T>& in,
+                                                const CharOf<T, X, DIR>& ch, int k, double alpha,
+                                                X* f, const X* lin, double* cc) {
+  constexpr int M = T::M;
   if constexpr (T::EUL) {
     X out[M];
     ch.right(f, out);
@@ -324,10 +383,30 @@ __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double 
 #pragma unroll
   for (int c = 0; c < M; ++c) {
     // f^+_i + f^-_{i+1} = (F_i + F_{i+1}) / 2 - alpha (U_{i+1} - U_i) / 2
-    if constexpr (FP64) cc[c] = madd(-0.5 * alpha, in.dU(c, k), f[c]);
-    else cc[c] = to_double(madd(dconst(1.0 / 60.0), lin[c], mul(f[c], dconst(1.0 / 12.0))));
+    if constexpr (std::is_same<X, double>::value)
+      cc[c] = madd(-0.5 * alpha, in.dU(c, k), f[c]);
+    else
+      cc[c] = to_double(madd(dconst(1.0 / 60.0), lin[c], mul(f[c], dconst(1.0 / 12.0))));
   }
-  return weak;
+}
+
+// c of the interface between points k and k + S; in pairs, false when the
+// correction is not small (the values are then not to be used).
+template <class X, int DIR, class T>
+__device__ __forceinline__ bool interface_line(const T& r, int k, int S, double alpha, double dx,
+                                               const SchemeParams& sp, double* cc) {
+  const LineData<X, T> in(r, S, alpha, dx, sp);
+  const LineWeights<X> w = line_weights<X>(sp, false);
+  const auto ch = char_system<DIR>(in, k, true);
+  X f[T::M], lin[T::M];
+#pragma unroll
+  for (int c = 0; c < T::M; ++c) f[c] = lin[c] = X{};
+  float e = 0.f;
+#pragma unroll 1
+  for (int sd = 0; sd < 2; ++sd) e += interface_side<DIR>(in, ch, w, sd, k, S, f, lin);
+  interface_value<DIR>(in, ch, k, alpha, f, lin, cc);
+  if constexpr (std::is_same<X, double>::value) return true;
+  else return interface_weak(r, k, S, e, alpha, sp);
 }
 
 // The derivative flux dx (h-hat^+ + h-hat^-) of component c at the interface
@@ -336,11 +415,95 @@ template <class T>
 __device__ __forceinline__ double derivative_flux_fp64(const T& r, int c, int k, int S, double kU,
                                                        double kh, double kv) {
   const int m = k - S, p = k + S, q = k + 2 * S;
-  const double t0 = r.F(c, p) - r.F(c, k), t1 = r.F(c, q) - r.F(c, m);
-  const double su = (r.U(c, q) - r.U(c, p)) - (r.U(c, k) - r.U(c, m));
-  const double sh = fma(-7.0, r.h(c, k) + r.h(c, p), r.h(c, m) + r.h(c, q));
-  const double sv = fma(3.0, r.N(c, k) - r.N(c, p), r.N(c, m) - r.N(c, q));
-  return fma(1.875, t0, fma(-0.125, t1, fma(kU, su, fma(kh, sh, kv * sv))));
+  const double t0 = sub(r.F(c, p), r.F(c, k)), t1 = sub(r.F(c, q), r.F(c, m));
+  const double su = sub(sub(r.U(c, q), r.U(c, p)), sub(r.U(c, k), r.U(c, m)));
+  const double sh = madd(-7.0, add(r.h(c, k), r.h(c, p)), add(r.h(c, m), r.h(c, q)));
+  const double sv = madd(3.0, sub(r.N(c, k), r.N(c, p)), sub(r.N(c, m), r.N(c, q)));
+  return madd(1.875, t0, madd(-0.125, t1, madd(kU, su, madd(kh, sh, mul(kv, sv)))));
+}
+
+// The limiter's four differences at point k, component c.
+template <class X, class T>
+__device__ __forceinline__ void limiter_differences(const LineData<X, T>& in, int c, int k, int S,
+                                                    X* x) {
+  x[0] = in.dU(c, k - S);
+  x[1] = in.dU(c, k);
+  x[2] = in.Nx(c, k - S);
+  x[3] = in.Nx(c, k + S);
+}
+
+// The limited derivative from its characteristic fields (chars) or
+// components z: pairs, 4 times the corrections to the linear
+// dx q_0' = 3/4 (u_{i+1} - u_{i-1}) - dx (v_{i-1} + v_{i+1}) / 4; FP64, dx v~.
+template <int DIR, class X, class T>
+__device__ __forceinline__ void limiter_sum(const LineData<X, T>& in, const CharOf<T, X, DIR>& ch,
+                                            int k, int S, double idx, bool chars, X* z,
+                                            double* vt) {
+  constexpr int M = T::M;
+  const T& r = in.r;
+  if constexpr (T::EUL) {
+    if (chars) {
+      X out[M];
+      ch.right(z, out);
+#pragma unroll
+      for (int c = 0; c < M; ++c) z[c] = out[c];
+    }
+  }
+  const double k3 = mul(0.75, idx), k1 = mul(0.25, idx);
+#pragma unroll
+  for (int c = 0; c < M; ++c) {
+    if constexpr (std::is_same<X, double>::value) {
+      vt[c] = mul(idx, z[c]);
+    } else {
+      const double q0 = madd(k3, sub(r.U(c, k + S), r.U(c, k - S)),
+                             mul(-0.25, add(r.N(c, k - S), r.N(c, k + S))));
+      vt[c] = madd(k1, to_double(z[c].l), madd(k1, to_double(z[c].h), q0));
+    }
+  }
+}
+
+// Characteristic field (or component) q of the limiter at point k in pairs,
+// with the characteristic system it makes for limiter_sum.
+template <int DIR, class T>
+__device__ __forceinline__ D2 limiter_field(const LineData<D2, T>& in, CharOf<T, D2, DIR>& ch,
+                                            int k, int S, const SchemeParams& sp, int q,
+                                            float& e) {
+  constexpr int M = T::M;
+  D2 y[4];
+  if (T::EUL && sp.limiter != 2) {  // uniform
+    if constexpr (T::EUL) {
+      D2 x[M][4];
+#pragma unroll
+      for (int c = 0; c < M; ++c) limiter_differences(in, c, k, S, x[c]);
+      ch = char_system<DIR>(in, k, false);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        D2 u[M];
+#pragma unroll
+        for (int c = 0; c < M; ++c) u[c] = x[c][v];
+        y[v] = ch.factors(u).field(q);
+      }
+    }
+  } else {
+    limiter_differences(in, q, k, S, y);
+  }
+  const D2 z = limiter_correction(y[0], y[1], y[2], y[3], line_weights<D2>(sp, true), e);
+  if (T::EUL && sp.limiter != 2) e = ch.density_units(q, e);
+  return z;
+}
+
+// Whether point k's limited derivative, of whose bounds `e` is the sum, may be
+// taken in pairs: e = 0, or (characteristic fields, whose FP64 form starts
+// from projected values) small against the density.
+template <class T>
+__device__ __forceinline__ bool limiter_weak(const T& r, int k, float e, const SchemeParams& sp) {
+  if constexpr (T::EUL) {
+    if (sp.limiter != 2) {
+      const float s = r.E(0, k).h;
+      return e <= 4.f * kWeakLevel * s * s;
+    }
+  }
+  return e <= 0.f;
 }
 
 // The limited derivative at point k; in pairs, false as interface_line.
@@ -349,57 +512,50 @@ __device__ __forceinline__ bool limiter_line(const T& r, int k, int S, double dx
                                              const SchemeParams& sp, double* vt) {
   constexpr int M = T::M;
   const LineData<X, T> in(r, S, 0.0, dx, sp);
-  bool weak = true;
-  X x[4][M], z[M];
+  float sum = 0.f;
+  X x[M][4], z[M];
 #pragma unroll
-  for (int c = 0; c < M; ++c) {
-    x[0][c] = in.dU(c, k - S);
-    x[1][c] = in.dU(c, k);
-    x[2][c] = in.Nx(c, k - S);
-    x[3][c] = in.Nx(c, k + S);
-  }
+  for (int c = 0; c < M; ++c) limiter_differences(in, c, k, S, x[c]);
   const LineWeights<X> w = line_weights<X>(sp, true);
-  auto limit = [&](X q1, X q2, X Vm, X Vp) {
-    if constexpr (std::is_same<X, double>::value) return limiter_value(q1, q2, Vm, Vp, w);
-    else return limiter_correction(q1, q2, Vm, Vp, w, weak);
+  const bool chars = T::EUL && sp.limiter != 2;  // uniform
+  CharOf<T, X, DIR> ch;
+  auto limit = [&](int q, X q1, X q2, X Vm, X Vp) {
+    if constexpr (std::is_same<X, double>::value) {
+      return limiter_value(q1, q2, Vm, Vp, w);
+    } else {
+      float e = 0.f;
+      const D2 v = limiter_correction(q1, q2, Vm, Vp, w, e);
+      sum += chars ? ch.density_units(q, e) : e;
+      return v;
+    }
   };
-  if (T::EUL && sp.limiter != 2) {  // uniform
+  if (chars) {
     if constexpr (T::EUL) {
-      LineChar<X, M, DIR> ch;
-      X un, ut{}, H, f[M];
-      in.state(k, false, un, ut, H);
-      const X q = ch.kinetic(un, ut);
-      ch.init(un, ut, H, q, mul(in.gm1(), sub(H, q)), in.gm1());
-      typename decltype(ch)::Factors a[4];
+      ch = char_system<DIR>(in, k, false);
+      typename CharOf<T, X, DIR>::Factors a[4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) a[v] = ch.factors(x[v]);
+      for (int v = 0; v < 4; ++v) {
+        X y[M];
 #pragma unroll
-      for (int c = 0; c < M; ++c) f[c] = X{};
+        for (int c = 0; c < M; ++c) y[c] = x[c][v];
+        a[v] = ch.factors(y);
+      }
+#pragma unroll
+      for (int c = 0; c < M; ++c) z[c] = X{};
 #pragma unroll 1
       for (int q = 0; q < M; ++q) {
-        const X y = limit(a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q));
+        const X y = limit(q, a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q));
 #pragma unroll
-        for (int c = 0; c < M; ++c) f[c] = pick2(q == c, y, f[c]);
+        for (int c = 0; c < M; ++c) z[c] = pick2(q == c, y, z[c]);
       }
-      ch.right(f, z);
     }
   } else {
 #pragma unroll
-    for (int c = 0; c < M; ++c) z[c] = limit(x[0][c], x[1][c], x[2][c], x[3][c]);
+    for (int c = 0; c < M; ++c) z[c] = limit(c, x[c][0], x[c][1], x[c][2], x[c][3]);
   }
-  // dx q_0' = 3/4 (u_{i+1} - u_{i-1}) - dx (v_{i-1} + v_{i+1}) / 4
-  const double k3 = 0.75 * idx, k1 = 0.25 * idx;
-#pragma unroll
-  for (int c = 0; c < M; ++c) {
-    if constexpr (std::is_same<X, double>::value) {
-      vt[c] = mul(idx, z[c]);
-    } else {
-      const double q0 =
-          fma(k3, r.U(c, k + S) - r.U(c, k - S), -0.25 * (r.N(c, k - S) + r.N(c, k + S)));
-      vt[c] = fma(k1, to_double(z[c].l), fma(k1, to_double(z[c].h), q0));
-    }
-  }
-  return weak;
+  limiter_sum<DIR>(in, ch, k, S, idx, chars, z, vt);
+  if constexpr (std::is_same<X, double>::value) return true;
+  else return limiter_weak(r, k, sum, sp);
 }
 
 // ---------------------------------------------------------------------------
@@ -430,12 +586,11 @@ __device__ __forceinline__ void interface_group(const T& r, int k, int S, int j,
   const LineWeights<double> w = line_weights<double>(sp, false);
   LineChar<double, M == 1 ? 3 : M, M == 1 ? 0 : DIR> ch;
   if constexpr (T::EUL) {
-    double a[M], un, ut = 0.0, H;
+    double un, ut = 0.0, H;
     if (sp.eig_avg == 0) {  // Roe average; each side's lanes take one state
-#pragma unroll
-      for (int i = 0; i < M; ++i) a[i] = r.U(i, sd ? k + S : k);
-      in.prim(a, un, ut, H);
-      const double s = mul(a[0], rsqrt_fp64(a[0]));
+      const int ks = sd ? k + S : k;
+      in.prim_at(ks, un, ut, H);
+      const double s = mul(r.U(0, ks), rsqrt_fp64(r.U(0, ks)));
       const double so = __shfl_xor_sync(all, s, NC), is = recip_fp64(add(s, so));
       auto roe = [&](double x) {
         const double m = mul(s, x), o = __shfl_xor_sync(all, m, NC);
@@ -445,9 +600,7 @@ __device__ __forceinline__ void interface_group(const T& r, int k, int S, int j,
       H = roe(H);
       if constexpr (M == 4) ut = roe(ut);
     } else {
-#pragma unroll
-      for (int i = 0; i < M; ++i) a[i] = mul(0.5, add(r.U(i, k), r.U(i, k + S)));
-      in.prim(a, un, ut, H);
+      in.state(k, true, un, ut, H);
     }
     const double kin = ch.kinetic(un, ut);
     ch.init(un, ut, H, kin, mul(in.gm1(), sub(H, kin)), in.gm1());
@@ -495,11 +648,7 @@ __device__ __forceinline__ void limiter_group(const T& r, int k, int S, int j, b
   double z;
   if (T::EUL && sp.limiter != 2) {  // uniform
     if constexpr (T::EUL) {
-      LineChar<double, M, DIR> ch;
-      double un, ut = 0.0, H;
-      in.state(k, false, un, ut, H);
-      const double kin = ch.kinetic(un, ut);
-      ch.init(un, ut, H, kin, mul(in.gm1(), sub(H, kin)), in.gm1());
+      const auto ch = char_system<DIR>(in, k, false);
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         double y[M];
@@ -573,6 +722,125 @@ __device__ __forceinline__ void listed_items(const T& r, const unsigned short* l
       }
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// The wide form of the item phases, for launches that leave SMs idle: several
+// threads per item share its work by roles, so that the phase takes the time
+// of one role's instruction stream and every sub-partition has warps to
+// interleave. Roles: the two sides of an interface (FIELDS: one per side and
+// field), the limiter (FIELDS: one per field), the derivative flux. The
+// arithmetic of every quantity is that of interface_line and limiter_line,
+// operation for operation, so the results are the same bits.
+// ---------------------------------------------------------------------------
+template <int M, bool FIELDS>
+struct WideRoles {
+  static constexpr int sides = FIELDS ? 2 * M : 2, limiter = FIELDS ? M : 1;
+  static constexpr int count = sides + limiter + 1;
+  // exchange rows of LI pairs: sides' fields, "-" side's linear parts, the
+  // limiter's fields; then the bounds of the sides' and the limiter's fields
+  static constexpr int rows = 7 * M;
+};
+
+// The lists of a tile's items for FP64.
+template <int MAX>
+struct ItemLists {
+  int nf, nl;
+  unsigned short f[MAX], l[MAX];
+};
+
+// Phases 3 and 3b for role `role` of interface j (left point kf) and point j
+// (kl). xch: exchange rows. Every thread of the CTA calls it; C, D and lim
+// are ready after the next barrier.
+template <int DIR, bool FIELDS, class T, class L, class At>
+__device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j, bool has_f, int kf,
+                                           bool has_l, int kl, int S, double alpha, double dx,
+                                           double idx, const SchemeParams& sp, L& ls, At at,
+                                           int rot) {
+  constexpr int M = T::M;
+  using R = WideRoles<M, FIELDS>;
+  const LineData<D2, T> in(r, S, alpha, dx, sp);
+  auto row = [&](int q) -> D2& { return xch[q * r.LI + j]; };
+  CharOf<T, D2, DIR> ch;
+  D2 f[M], lin[M];
+  const int sd = FIELDS ? role / M : role, q0 = FIELDS ? role % M : 0;
+  const bool lim_role = role >= R::sides && role < R::sides + R::limiter;
+  const int lq = role - R::sides;
+  const bool limited = sp.limiter != 0, chars = T::EUL && sp.limiter != 2;
+  if (role < R::sides) {
+    if (has_f) {
+      const LineWeights<D2> w = line_weights<D2>(sp, false);
+      ch = char_system<DIR>(in, kf, true);
+#pragma unroll
+      for (int c = 0; c < M; ++c) f[c] = lin[c] = D2{0.f, 0.f};
+      row(4 * M + sd * M + q0).h = interface_side<DIR, FIELDS>(in, ch, w, sd, kf, S, f, lin, q0);
+      if constexpr (FIELDS) {
+        row(sd * M + q0) = f[0];
+      } else {
+#pragma unroll
+        for (int c = 0; c < M; ++c) row(sd * M + c) = f[c];
+      }
+      if (sd == 1 && q0 == 0)
+#pragma unroll
+        for (int c = 0; c < M; ++c) row(2 * M + c) = lin[c];
+    }
+  } else if (lim_role) {
+    if (has_l && limited) {
+      if constexpr (FIELDS) {
+        float e = 0.f;
+        row(3 * M + lq) = limiter_field<DIR>(in, ch, kl, S, sp, lq, e);
+        row(6 * M + lq).h = e;
+      } else {
+        double x[M];
+        if (!limiter_line<D2, DIR>(r, kl, S, dx, idx, sp, x))
+          ls.l[atomicAdd(&ls.nl, 1)] = (unsigned short)j;
+#pragma unroll
+        for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
+      }
+    }
+  } else if (has_f) {
+    const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
+#pragma unroll
+    for (int c = 0; c < M; ++c) r.D(c, j) = derivative_flux_fp64(r, c, kf, S, kU, kh, kv);
+  }
+  __syncthreads();
+  if (role == 0 && has_f) {
+    double cc[M];
+    float e[2] = {0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      f[c] = add(row(c), row(M + c));
+      lin[c] = add(lin[c], row(2 * M + c));
+      if (FIELDS || c == 0) {  // (in the order of the loop over fields)
+        e[0] += row(4 * M + c).h;
+        e[1] += row(5 * M + c).h;
+      }
+    }
+    interface_value<DIR>(in, ch, kf, alpha, f, lin, cc);
+    if (!interface_weak(r, kf, S, e[0] + e[1], alpha, sp))
+      ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
+#pragma unroll
+    for (int c = 0; c < M; ++c) r.C(c, j) = cc[c];
+  }
+  if constexpr (FIELDS) {
+    if (lim_role && lq == 0 && has_l && limited) {
+      D2 z[M];
+      double x[M];
+      float e = 0.f;
+#pragma unroll
+      for (int c = 0; c < M; ++c) {
+        z[c] = row(3 * M + c);
+        e += row(6 * M + c).h;
+      }
+      limiter_sum<DIR>(in, ch, kl, S, idx, chars, z, x);
+      if (!limiter_weak(r, kl, e, sp)) ls.l[atomicAdd(&ls.nl, 1)] = (unsigned short)j;
+#pragma unroll
+      for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
+    }
+  }
+  __syncthreads();
+  if (ls.nf + ls.nl > 0)  // uniform
+    listed_items<DIR>(r, ls.f, ls.nf, ls.l, ls.nl, at, S, rot, alpha, dx, idx, sp);
 }
 
 }  // namespace hweno

@@ -575,9 +575,54 @@ k_stage_1d_f64(const __grid_constant__ Args1D a, int mode, int P) {
   stage_tile_df<EQ>(a, io_of(a), mode, P, a.tile_inst[blockIdx.x], a.tile_start[blockIdx.x]);
 }
 
+template <int EQ, bool FIELDS>
+__global__ void __launch_bounds__(wide_threads<EQ>(FIELDS ? kFieldsMax : kWideMax))
+k_stage_wide_1d_f64(const __grid_constant__ Args1D a, int mode, int P) {
+  __shared__ double s_dt;
+  const int k = a.tile_inst[blockIdx.x], s = a.tile_start[blockIdx.x];
+  if (a.skip_done && !(a.t[k] < a.t_end)) return;
+  if (threadIdx.x == 0) {
+    double dt = 0.0;
+    if (mode == MODE_STAGE1) {
+      int lands = 0;
+      dt = a.dt_in ? a.dt_in[k]
+                   : time_step(a.sp, a.alpha_in[k], a.inst_hx[k], a.t[k], a.t_end, lands);
+      if (s == 0) { a.dt[k] = dt; a.lands[k] = lands; }
+    } else if (mode != MODE_RHS) {
+      dt = a.dt[k];
+    }
+    s_dt = dt;
+  }
+  __syncthreads();
+  const bool want = mode != MODE_RHS && a.alpha_out != nullptr;
+  const unsigned long long m =
+      stage_wide_df<EQ, FIELDS>(a, io_of(a), mode, P, k, s, a.alpha_in[k], s_dt, want);
+  if (want && threadIdx.x == 0) atomicMax(&a.alpha_out[k], m);
+}
+
+// The wide form is taken while there is at most one tile per SM: the tiled
+// kernel's CTAs of four warps would then leave SMs or sub-partitions idle.
+inline bool wide_fits(int P, int ntiles) { return P <= kWideMax && ntiles <= 152; }
+
+template <int EQ, bool FIELDS>
+cudaError_t stage_wide_launch(int mode, int P, const Args1D& a, int ntiles, cudaStream_t s) {
+  static unsigned configured = 0;  // devices whose limit is raised
+  if (const cudaError_t e = ensure_smem_limit(k_stage_wide_1d_f64<EQ, FIELDS>,
+                                              wide_bytes<EQ>(kWideMax), configured))
+    return e;
+  k_stage_wide_1d_f64<EQ, FIELDS>
+      <<<ntiles, wide_threads<EQ>(P), wide_bytes<EQ>(P), s>>>(a, mode, P);
+  return cudaGetLastError();
+}
+
 template <int EQ>
 cudaError_t stage_launch_f64(int variant, int mode, const Args1D& a, int ntiles, cudaStream_t s) {
   const int P = tile_points(variant);
+  if (wide_fits(P, ntiles)) {
+    if constexpr (wide_fields<EQ>(kFieldsMax))
+      if (wide_fields<EQ>(P)) return stage_wide_launch<EQ, true>(mode, P, a, ntiles, s);
+    return stage_wide_launch<EQ, false>(mode, P, a, ntiles, s);
+  }
   const size_t bytes = Tile1D<EQ>::bytes(P + 4, P + 1);
   static unsigned configured = 0;  // devices whose limit is raised
   if (const cudaError_t e = ensure_smem_limit(
@@ -1354,29 +1399,138 @@ k_step_cluster_split_1d(const __grid_constant__ Args1D a, const __grid_constant_
   }
 }
 
-// Launch on clusters of C CTAs; returns cudaErrorNotSupported (nothing
-// launched) when the device cannot hold such a cluster.
-template <int EQ, class Real, bool SPLIT>
-cudaError_t step_cluster_try(const Args1D& a, const FusedArgs& f, int C, cudaStream_t s) {
-  constexpr size_t tile =
-      SPLIT ? SplitLayout<EQ, Real>::bytes : Layout1D<EQ, Real, kThreads1D, 1>::bytes;
-  constexpr size_t bytes = tile > kClusterSmem ? tile : kClusterSmem;
-  auto kern = SPLIT ? k_step_cluster_split_1d<EQ, Real> : k_step_cluster_1d<EQ, Real>;
-  static unsigned configured = 0;  // devices whose limit is raised
-  if (const cudaError_t e = ensure_smem_limit(kern, bytes, configured)) return e;
-  static unsigned nonportable = 0;  // devices allowed clusters above 8
+// FP64: the same kernel structure around the wide form of a stage, with the
+// smallest of three tile sizes (28, 60, 124 points) for which the instance
+// fits 16 CTAs: the fewer points a CTA has, the less its warps compete.
+template <int EQ, bool FIELDS>
+__global__ void __launch_bounds__(wide_threads<EQ>(FIELDS ? kFieldsMax : kWideMax))
+k_step_cluster_f64(const __grid_constant__ Args1D a, const __grid_constant__ FusedArgs f, int P) {
+  namespace cg = cooperative_groups;
+  constexpr int M = Dim1<EQ>::M;
+  __shared__ unsigned long long s_own;  // this CTA's tile: alpha of U^n
+  __shared__ double part[4];  // shares: alpha of U^n and of the three stage outputs
+  __shared__ double s_alpha, s_dt;
+  __shared__ int s_lands;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks();
+  const int rank = (int)cl.block_rank();
+  const int k = blockIdx.x / C;
+  const int n = a.inst_n[k];
+  const int s = rank * P;
+  const bool mine = s < n;
+  if (threadIdx.x < 4) part[threadIdx.x] = 0.0;
+  if (threadIdx.x == 0) s_own = 0ull;
+  double t = a.t[k];  // rank 0 writes t[k] only after the first step's barriers
+  __syncthreads();
+  // the cluster's maximum of share q (after a cluster barrier), to every thread
+  auto cluster_alpha = [&](int q) -> double {
+    if (threadIdx.x < 32) {
+      const double v = (int)threadIdx.x < C ? cl.map_shared_rank(part, (int)threadIdx.x)[q] : 0.0;
+      const unsigned long long m = warp_max_bits(v);
+      if (threadIdx.x == 0) s_alpha = __longlong_as_double((long long)m);
+    }
+    __syncthreads();
+    return s_alpha;
+  };
+  {  // alpha(U^n) of this tile's points
+    double amax = 0.0;
+    if (mine && t < a.t_end) {
+      const double* U = static_cast<const double*>(a.U) + a.inst_off[k] * M;
+      const int e = min(s + P, n);
+      for (int j = s + threadIdx.x; j < e; j += blockDim.x) {
+        double u[M];
+#pragma unroll
+        for (int c = 0; c < M; ++c) u[c] = U[(long long)c * n + j];
+        amax = fmax(amax, wave_speed<EQ>(u, a.sp.wd[9], a.sp.wd[10]));
+      }
+    }
+    const unsigned long long m = warp_max_bits(amax);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_own, m);
+    __syncthreads();
+    if (threadIdx.x == 0) part[0] = __longlong_as_double((long long)s_own);
+  }
+  cl.sync();
+  double alpha = cluster_alpha(0);
+#pragma unroll 1
+  for (int step = 0; step < f.steps; ++step) {
+    const bool live = t < a.t_end;  // the same in every CTA
+    const bool has = live && mine;
+    double dt = 0.0;
+    int lands = 0;
+    if (live) {
+      if (threadIdx.x == 0) {
+        s_dt = a.dt_in ? a.dt_in[k] : time_step(a.sp, alpha, a.inst_hx[k], t, a.t_end, s_lands);
+        if (a.dt_in) s_lands = 0;
+      }
+      __syncthreads();
+      dt = s_dt;
+      lands = s_lands;
+    }
+    const bool more = step + 1 < f.steps;  // stage 3 also gives alpha of U^{n+1}
+    double al[3] = {alpha, 0.0, 0.0};
+#pragma unroll 1
+    for (int stage = 0; stage < 3; ++stage) {
+      const double in = stage == 0 ? al[0] : stage == 1 ? al[1] : al[2];
+      const bool want = stage < 2 || more;
+      if (has) {
+        const unsigned long long m =
+            stage_wide_df<EQ, FIELDS>(a, step_io(a, f, stage, nullptr, nullptr), MODE_STAGE1 + stage, P, k,
+                              s, in, dt, want);
+        if (want && threadIdx.x == 0) part[stage + 1] = __longlong_as_double((long long)m);
+      }
+      cl.sync();
+      if (want) {
+        const double v = cluster_alpha(stage + 1);
+        if (stage == 0) al[1] = v;
+        else if (stage == 1) al[2] = v;
+        else alpha = v;
+      }
+    }
+    if (live) {
+      const double tn = lands ? a.t_end : t + dt;
+      if (rank == 0 && threadIdx.x == 0) {
+        const_cast<double*>(a.t)[k] = tn;
+        a.dt[k] = dt;
+        a.lands[k] = lands;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          f.alpha[q * f.batch + k] = (unsigned long long)__double_as_longlong(al[q]);
+        if (!(al[0] <= DBL_MAX)) atomicOr(a.status, STATUS_NONFINITE);
+        if (f.pu) atomicAdd(f.pu, (unsigned long long)n);
+        if (f.dt_used) f.dt_used[k] = dt;
+        if (!more && tn < a.t_end) atomicAdd(f.active, 1);
+      }
+      t = tn;
+    } else if (rank == 0 && threadIdx.x == 0 && f.dt_used) {
+      f.dt_used[k] = 0.0;  // finished: nothing moves
+    }
+  }
+}
+
+// Launch `kern` on clusters of C CTAs of `threads` threads; returns
+// cudaErrorNotSupported (nothing launched) when the device cannot hold such a
+// cluster. `st`: what is known of this kernel and CTA size, per device.
+struct ClusterState {
+  unsigned configured = 0;   // devices whose shared-memory limit is raised
+  unsigned nonportable = 0;  // devices allowed clusters above 8
+  signed char fits[32][kSplitMax + 1] = {};  // per cluster size: 0 unknown, 1 yes, -1 no
+};
+template <class K, class... Args>
+cudaError_t cluster_launch(K* kern, ClusterState& st, int C, int batch, int threads, size_t bytes,
+                           cudaStream_t s, const Args&... args) {
+  if (const cudaError_t e = ensure_smem_limit(kern, bytes, st.configured)) return e;
   int dev = 0;
   if (const cudaError_t e = cudaGetDevice(&dev)) return e;
   const unsigned bit = dev < 32 ? 1u << dev : 0u;
-  if (C > 8 && !(nonportable & bit)) {
+  if (C > 8 && !(st.nonportable & bit)) {
     if (const cudaError_t e =
             cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))
       return e;
-    nonportable |= bit;
+    st.nonportable |= bit;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(f.batch * C));
-  cfg.blockDim = dim3(kThreads1D);
+  cfg.gridDim = dim3((unsigned)(batch * C));
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = bytes;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -1387,8 +1541,7 @@ cudaError_t step_cluster_try(const Args1D& a, const FusedArgs& f, int C, cudaStr
   cfg.attrs = at;
   cfg.numAttrs = 1;
   // whether a cluster of this size fits, once per device and size
-  static signed char fits[32][kSplitMax + 1] = {};  // 0 unknown, 1 yes, -1 no
-  signed char& ok = fits[dev < 32 ? dev : 0][C];
+  signed char& ok = st.fits[dev < 32 ? dev : 0][C];
   if (ok == 0) {
     int clusters = 0;
     const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
@@ -1396,14 +1549,52 @@ cudaError_t step_cluster_try(const Args1D& a, const FusedArgs& f, int C, cudaStr
     ok = clusters > 0 ? 1 : -1;
   }
   if (ok < 0) return cudaErrorNotSupported;
-  return cudaLaunchKernelEx(&cfg, kern, a, f);
+  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// The cluster step: for instances of at most kSplitMax * kSplitTile points
-// the latency form (28-point tiles, the work of a point over four warps) when
-// the device holds such clusters, else 124-point tiles.
+template <int EQ, class Real, bool SPLIT>
+cudaError_t step_cluster_try(const Args1D& a, const FusedArgs& f, int C, cudaStream_t s) {
+  constexpr size_t tile =
+      SPLIT ? SplitLayout<EQ, Real>::bytes : Layout1D<EQ, Real, kThreads1D, 1>::bytes;
+  constexpr size_t bytes = tile > kClusterSmem ? tile : kClusterSmem;
+  auto kern = SPLIT ? k_step_cluster_split_1d<EQ, Real> : k_step_cluster_1d<EQ, Real>;
+  static ClusterState st;
+  return cluster_launch(kern, st, C, f.batch, kThreads1D, bytes, s, a, f);
+}
+
+template <int EQ, int P>
+cudaError_t step_cluster_f64_try(const Args1D& a, const FusedArgs& f, int max_n, cudaStream_t s) {
+  const int C = (max_n + P - 1) / P;
+  if (C > (P == kTile1D ? kClusterMax : kSplitMax)) return cudaErrorNotSupported;
+  constexpr size_t tile = wide_bytes<EQ>(P);
+  constexpr size_t bytes = tile > kClusterSmem ? tile : kClusterSmem;
+  static ClusterState st;
+  return cluster_launch(k_step_cluster_f64<EQ, wide_fields<EQ>(P)>, st, C, f.batch,
+                        wide_threads<EQ>(P), bytes, s, a, f, P);
+}
+
+// The cluster step. FP32, and Euler in FP64: for instances of at most
+// kSplitMax * kSplitTile points the latency form (28-point tiles, the work of
+// a point over four warps) when the device holds such clusters. Else FP32
+// takes 124-point tiles and FP64 the wide form (28-point tiles for the scalar
+// equations). Measured, FP64, us per step, latency form / wide form: Burgers
+// N = 60..440 18.5 / 14, Euler Riemann problem 51 / 47.5 but blast waves,
+// with FP64 items in most tiles, 51 / 60; 124-point tiled cluster / wide form
+// at N = 460..992: Burgers 35 / 15, Euler 108 / 52 to 74.
 template <int EQ, class Real>
 cudaError_t step_cluster_launch(const Args1D& a, const FusedArgs& f, int max_n, cudaStream_t s) {
+  if constexpr (std::is_same<Real, double>::value) {
+    cudaError_t e = cudaErrorNotSupported;
+    if (EQ == HWENO_EULER) {
+      const int Cs = (max_n + kSplitTile - 1) / kSplitTile;
+      if (Cs <= kSplitMax) e = step_cluster_try<EQ, Real, true>(a, f, Cs, s);
+    } else {
+      e = step_cluster_f64_try<EQ, kSplitTile>(a, f, max_n, s);
+    }
+    if (e == cudaErrorNotSupported) e = step_cluster_f64_try<EQ, 60>(a, f, max_n, s);
+    if (e == cudaErrorNotSupported) e = step_cluster_f64_try<EQ, kTile1D>(a, f, max_n, s);
+    return e;
+  } else {
   const int Cs = (max_n + kSplitTile - 1) / kSplitTile;
   if (Cs <= kSplitMax) {
     const cudaError_t e = step_cluster_try<EQ, Real, true>(a, f, Cs, s);
@@ -1411,6 +1602,7 @@ cudaError_t step_cluster_launch(const Args1D& a, const FusedArgs& f, int max_n, 
   }
   const int C = (max_n + kTile1D - 1) / kTile1D;
   return step_cluster_try<EQ, Real, false>(a, f, C, s);
+  }
 }
 
 template <class Real>

@@ -6,8 +6,11 @@
 // What bounds them: an all-FP64 stage (x- and y-sweep) needs about 2 200 FP64
 // instructions per point at 65 to 77 cycles per warp and sub-partition; here
 // about 400 remain, next to about 17 000 FP32 instructions. Measured: double
-// Mach 1920 x 480, 13.2 -> 4.09 ms per step (FP64 pipe 86% -> 60% busy); 256^2,
-// 1.06 -> 0.37 ms per step; Burgers rhs 321 x 203, 95 -> 50 us.
+// Mach 1920 x 480, 13.2 -> 3.91 ms per step (FP64 pipe 86% -> 60% busy); 256^2,
+// 1.06 -> 0.37 ms per step; Burgers rhs 321 x 203, 95 -> 50 us. Error against
+// 128-bit arithmetic relative to the all-FP64 sweeps (2-norms): U 0.8-1.0,
+// V, W 0.66-1.0, L^1 0.1-1.0 (Burgers on 48 x 60, the coarsest grid: 1.25),
+// L^2, L^3 0.45-0.55, v~, w~ 0.01-0.6.
 //
 // Tiles: the x-sweep takes row segments of 124 points. The y-sweep takes
 // blocks of 4 columns x 31 rows: 35 rows loaded for 31 (16 columns x 7 rows
@@ -20,14 +23,11 @@ constexpr int kColsF64 = 4, kRowsF64 = kThreads2D / kColsF64 - 1;
 template <int EQ, int DIR>
 using Tile2D = LineTile<Dim2<EQ>::M, DIR, EQ == HWENO_EULER, Dim2<EQ>::M, true>;
 
-struct Lists2D {  // items evaluated in FP64
-  int nf, nl;
-  unsigned short f[kThreads2D], l[kThreads2D];
-};
+using Lists2D = ItemLists<kThreads2D>;
 
 // Phase 1, loaded point k: state u, the derivatives v along and w across the
 // line; stores the flux, the two Jacobian-vector products and the pairs.
-template <int EQ, int DIR>
+template <int EQ, int DIR, bool WIDE>
 __device__ __forceinline__ void load_point_2d(const Tile2D<EQ, DIR>& r, int k, const double* u,
                                               const double* v, const double* w, double gm1,
                                               D2 alp, D2 hp) {
@@ -50,7 +50,16 @@ __device__ __forceinline__ void load_point_2d(const Tile2D<EQ, DIR>& r, int k, c
   }
   if constexpr (EQ == HWENO_EULER)
     point_eigen(r, k, u[0], q.ir, q.Ep, DIR == 0 ? q.u : q.v, DIR == 0 ? q.v : q.u);
-  point_pairs(r, k, v, h, alp, hp);
+  if constexpr (!WIDE) point_pairs(r, k, v, h, alp, hp);
+}
+
+// The wide form of the sweeps (wide_items), for grids with at most one tile
+// per SM: four threads per point (roles), in phases 2 and 4 one component each.
+// Measured, two steps: density wave 48^2 370 -> 274 us, 100 x 60 379 -> 286 us.
+constexpr int kWideThreads2D = 4 * kThreads2D;
+template <int EQ, int DIR>
+constexpr size_t xch_bytes(int LI) {
+  return sizeof(D2) * WideRoles<Dim2<EQ>::M, false>::rows * LI;
 }
 
 // Phase 3 of one thread: interface j (left point kf) and limiter point j
@@ -62,8 +71,7 @@ __device__ __forceinline__ void items_2d(const Tile2D<EQ, DIR>& r, int j, bool h
   constexpr int M = Dim2<EQ>::M;
   double x[M];
   if (has_f) {
-    // (the mean state's eigenvectors are taken in FP64)
-    if (!((M == 1 || sp.eig_avg == 0) && interface_line<D2, DIR>(r, kf, S, alpha, dx, sp, x)))
+    if (!interface_line<D2, DIR>(r, kf, S, alpha, dx, sp, x))
       ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
     const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
 #pragma unroll
@@ -86,16 +94,16 @@ template <int EQ, int DIR>
 __device__ __forceinline__ void differences_2d(const Tile2D<EQ, DIR>& r, int c, int k, int S,
                                                int ja, int jb, double& dF, double& dD,
                                                double& dE) {
-  dF = fma(0.5, r.F(c, k + S) - r.F(c, k - S), r.C(c, jb) - r.C(c, ja));
-  dD = r.D(c, jb) - r.D(c, ja);
-  dE = fma(8.0, r.extra(c, k + S) - r.extra(c, k - S),
-           r.extra(c, k - 2 * S) - r.extra(c, k + 2 * S));
+  dF = madd(0.5, sub(r.F(c, k + S), r.F(c, k - S)), sub(r.C(c, jb), r.C(c, ja)));
+  dD = sub(r.D(c, jb), r.D(c, ja));
+  dE = madd(8.0, sub(r.extra(c, k + S), r.extra(c, k - S)),
+            sub(r.extra(c, k - 2 * S), r.extra(c, k + 2 * S)));
 }
 
-template <int EQ>
-__global__ void __launch_bounds__(kThreads2D, HWENO_MINB_2D_F64)
+template <int EQ, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kWideThreads2D : kThreads2D, WIDE ? 1 : HWENO_MINB_2D_F64)
 k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
-  constexpr int M = Dim2<EQ>::M;
+  constexpr int M = Dim2<EQ>::M, NT = WIDE ? kWideThreads2D : kThreads2D;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Lists2D ls;
   if (a.skip_done && !(a.t[0] < a.t_end)) return;
@@ -131,7 +139,7 @@ k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
                         div(D2{1.f, 0.f}, alp)};
 
   // 1: points
-  for (int g = threadIdx.x; g < np + 4; g += kThreads2D) {
+  for (int g = threadIdx.x; g < np + 4; g += NT) {
     const Src s = map_x(i0 - 2 + g, nx, a.sp);
     HWENO_CHECK(s.kind == 2 || (s.idx >= 0 && s.idx < nx), a.status);
     double u[M], v[M], w[M];
@@ -151,38 +159,47 @@ k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
         }
       }
     }
-    load_point_2d<EQ, 0>(r, g, u, v, w, gm1, alp, hp);
+    load_point_2d<EQ, 0, WIDE>(r, g, u, v, w, gm1, alp, hp);
   }
   __syncthreads();
-  // 2: edges
-  for (int g = threadIdx.x; g < np + 3; g += kThreads2D) edge_pairs(r, g, 1, alp);
-  __syncthreads();
-  // 3: interfaces and limiter
-  {
-    const int j = threadIdx.x;
-    items_2d<EQ, 0>(r, j, j <= np, j + 1, j < np, j + 2, 1, alpha, dx, idx, a.sp, ls);
-  }
-  __syncthreads();
-  if (ls.nf + ls.nl > 0) {
-    listed_items<0>(r, ls.f, ls.nf, ls.l, ls.nl,
-                    [](int j, bool lim) { return lim ? j + 2 : j + 1; }, 1, tile + row_, alpha, dx,
-                    idx, a.sp);
+  const int role = threadIdx.x / kThreads2D, j = threadIdx.x % kThreads2D;
+  auto at = [](int i, bool lim) { return lim ? i + 2 : i + 1; };
+  if constexpr (WIDE) {
+    // 2: pairs of points and edges
+    if (role < M && j < np + 4) point_pair(r, role, j, r.N(role, j), r.h(role, j), alp, hp);
+    if (role < M && j < np + 3) edge_pair(r, role, j, 1, alp);
     __syncthreads();
+    // 3: interfaces and limiter
+    wide_items<0, false>(r, reinterpret_cast<D2*>(smem_raw + Tile2D<EQ, 0>::bytes(r.L, r.LI)), role,
+                         j, j <= np, j + 1, j < np, j + 2, 1, alpha, dx, idx, a.sp, ls, at, 0);
+    __syncthreads();
+  } else {
+    // 2: edges
+    for (int g = threadIdx.x; g < np + 3; g += NT) edge_pairs(r, g, 1, alp);
+    __syncthreads();
+    // 3: interfaces and limiter
+    items_2d<EQ, 0>(r, j, j <= np, j + 1, j < np, j + 2, 1, alpha, dx, idx, a.sp, ls);
+    __syncthreads();
+    if (ls.nf + ls.nl > 0) {
+      listed_items<0>(r, ls.f, ls.nf, ls.l, ls.nl, at, 1, tile + row_, alpha, dx, idx, a.sp);
+      __syncthreads();
+    }
   }
   // 4: the x parts
-  if (threadIdx.x < np) {
-    const int j = threadIdx.x, k = j + 2;
+  if (j < np && role < M) {
+    const int k = j + 2;
     HWENO_CHECK(i0 + j < nx, a.status);
     const long long q = row + i0 + j;
     double* LX = static_cast<double*>(a.LX);
     double* VT = static_cast<double*>(a.VT);
 #pragma unroll
-    for (int c = 0; c < M; ++c) {
+    for (int cc = 0; cc < (WIDE ? 1 : M); ++cc) {
+      const int c = WIDE ? role : cc;
       double dF, dD, dE;
       differences_2d<EQ, 0>(r, c, k, 1, j, j + 1, dF, dD, dE);
-      LX[c * N + q] = -dF * idx;
-      LX[(M + c) * N + q] = -dD * idx2;
-      LX[(2 * M + c) * N + q] = dE * (idx * (-1.0 / 12.0));
+      LX[c * N + q] = mul(-dF, idx);
+      LX[(M + c) * N + q] = mul(-dD, idx2);
+      LX[(2 * M + c) * N + q] = mul(dE, mul(idx, -1.0 / 12.0));
       VT[c * N + q] = a.sp.limiter ? r.lim(c, j) : r.N(c, k);
     }
   }
@@ -203,10 +220,10 @@ __device__ __forceinline__ void rough_speeds2(const double* u, float gam, float&
   }
 }
 
-template <int EQ>
-__global__ void __launch_bounds__(kThreads2D, HWENO_MINB_2D_F64)
+template <int EQ, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kWideThreads2D : kThreads2D, WIDE ? 1 : HWENO_MINB_2D_F64)
 k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
-  constexpr int M = Dim2<EQ>::M;
+  constexpr int M = Dim2<EQ>::M, NT = WIDE ? kWideThreads2D : kThreads2D;
   constexpr int C = kColsF64, R = kRowsF64, L = (R + 4) * C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Lists2D ls;
@@ -231,7 +248,7 @@ k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
                         div(D2{1.f, 0.f}, alp)};
 
   // 1: points
-  for (int k = threadIdx.x; k < L; k += kThreads2D) {
+  for (int k = threadIdx.x; k < L; k += NT) {
     const int rr = k / C, col = k % C, i = i0 + col;
     if (col >= ncol || rr >= nrow + 4) continue;
     const int jj = j0 - 2 + rr;
@@ -257,49 +274,58 @@ k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
         }
       }
     }
-    load_point_2d<EQ, 1>(r, k, u, w, v, gm1, alp, hp);
+    load_point_2d<EQ, 1, WIDE>(r, k, u, w, v, gm1, alp, hp);
   }
-  __syncthreads();
-  // 2: edges
-  for (int k = threadIdx.x; k < (R + 3) * C; k += kThreads2D)
-    if (k % C < ncol && k / C < nrow + 3) edge_pairs(r, k, C, alp);
   __syncthreads();
   // 3: interfaces y_{j0+r-1/2}, r = 0..nrow (lower point in loaded row r + 1),
   // and the limiter of the points of row r (loaded row r + 2)
-  {
-    const int j = threadIdx.x, rr = j / C;
-    const bool in = j % C < ncol;
-    items_2d<EQ, 1>(r, j, in && rr <= nrow, j + C, in && rr < nrow, j + 2 * C, C, alpha, dy, idy,
-                    a.sp, ls);
-  }
-  __syncthreads();
-  if (ls.nf + ls.nl > 0) {
-    listed_items<1>(r, ls.f, ls.nf, ls.l, ls.nl,
-                    [](int j, bool lim) { return lim ? j + 2 * C : j + C; }, C,
-                    blockIdx.x + blockIdx.y, alpha, dy, idy, a.sp);
+  const int role = threadIdx.x / kThreads2D, j = threadIdx.x % kThreads2D, rr = j / C;
+  const bool in = j % C < ncol, has_f = in && rr <= nrow, mine = in && rr < nrow;
+  auto at = [](int i, bool lim) { return lim ? i + 2 * C : i + C; };
+  if constexpr (WIDE) {
+    if (role < M)
+      for (int k = j; k < L; k += kThreads2D) {
+        if (k % C >= ncol) continue;
+        if (k / C < nrow + 4) point_pair(r, role, k, r.N(role, k), r.h(role, k), alp, hp);
+        if (k / C < nrow + 3) edge_pair(r, role, k, C, alp);
+      }
     __syncthreads();
+    wide_items<1, false>(r, reinterpret_cast<D2*>(smem_raw + Tile2D<EQ, 1>::bytes(r.L, r.LI)), role,
+                         j, has_f, j + C, mine, j + 2 * C, C, alpha, dy, idy, a.sp, ls, at, 0);
+    __syncthreads();
+  } else {
+    for (int k = threadIdx.x; k < (R + 3) * C; k += NT)
+      if (k % C < ncol && k / C < nrow + 3) edge_pairs(r, k, C, alp);
+    __syncthreads();
+    items_2d<EQ, 1>(r, j, has_f, j + C, mine, j + 2 * C, C, alpha, dy, idy, a.sp, ls);
+    __syncthreads();
+    if (ls.nf + ls.nl > 0) {
+      listed_items<1>(r, ls.f, ls.nf, ls.l, ls.nl, at, C, blockIdx.x + blockIdx.y, alpha, dy, idy,
+                      a.sp);
+      __syncthreads();
+    }
   }
   // 4: the y parts, the Runge-Kutta combination
-  const int j = threadIdx.x, rr = j / C, k = j + 2 * C;
-  const bool mine = j % C < ncol && rr < nrow;
+  const int k = j + 2 * C;
   const bool want_alpha = mode == MODE_STAGE1 || mode == MODE_STAGE2;
   double un[M];
   float fx = 0.f, fy = 0.f;
-  if (mine) {
+  if (mine && role < M) {
     HWENO_CHECK(j0 + rr < ny && i0 + j % C < nx, a.status);
     const long long q = (long long)(j0 + rr) * nx + i0 + j % C;
     const double* LX = static_cast<const double*>(a.LX);
     const double* VT = static_cast<const double*>(a.VT);
     const double b = mode == MODE_STAGE1 ? 1.0 : mode == MODE_STAGE2 ? 0.25 : 2.0 / 3.0;
     const double a0 = mode == MODE_STAGE2 ? 0.75 : 1.0 / 3.0;
-    const double bdt = b * dt;
+    const double bdt = mul(b, dt);
 #pragma unroll
-    for (int c = 0; c < M; ++c) {
+    for (int cc = 0; cc < (WIDE ? 1 : M); ++cc) {
+      const int c = WIDE ? role : cc;
       const long long qc = c * N + q;
       double dG, dT, dX;
       differences_2d<EQ, 1>(r, c, k, C, j, j + C, dG, dT, dX);
-      const double l1 = fma(-idy, dG, LX[qc]), l3 = fma(-idy2, dT, LX[(2 * M) * N + qc]);
-      const double l2 = fma(idy * (-1.0 / 12.0), dX, LX[M * N + qc]);
+      const double l1 = madd(-idy, dG, LX[qc]), l3 = madd(-idy2, dT, LX[(2 * M) * N + qc]);
+      const double l2 = madd(mul(idy, -1.0 / 12.0), dX, LX[M * N + qc]);
       const double vt = VT[qc], wt = a.sp.limiter ? r.lim(c, j) : r.N(c, k);
       if (mode == MODE_RHS) {
         static_cast<double*>(a.L1)[qc] = l1;
@@ -309,22 +335,40 @@ k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
       } else {
         // b (x + dt L) first, then a x0 added in one operation: one rounding
         // of the full value
-        double x = fma(bdt, l1, b * r.U(c, k)), y = fma(bdt, l2, b * vt), z = fma(bdt, l3, b * wt);
-        if (mode == MODE_STAGE1) {
+        double x = r.U(c, k), y = vt, z = wt;
+        if (mode == MODE_STAGE1) {  // b = 1, a = 0
+          x = madd(bdt, l1, x);
+          y = madd(bdt, l2, y);
+          z = madd(bdt, l3, z);
           static_cast<double*>(a.Wt0out)[qc] = wt;
         } else {
-          x = fma(a0, static_cast<const double*>(a.U0)[qc], x);
-          y = fma(a0, static_cast<const double*>(a.Vt0)[qc], y);
-          z = fma(a0, static_cast<const double*>(a.Wt0)[qc], z);
+          x = madd(bdt, l1, mul(b, x));
+          y = madd(bdt, l2, mul(b, y));
+          z = madd(bdt, l3, mul(b, z));
+          x = madd(a0, static_cast<const double*>(a.U0)[qc], x);
+          y = madd(a0, static_cast<const double*>(a.Vt0)[qc], y);
+          z = madd(a0, static_cast<const double*>(a.Wt0)[qc], z);
         }
-        un[c] = x;
+        un[cc] = x;
+        if constexpr (WIDE) reinterpret_cast<double&>(r.H(0, c, k)) = x;  // (not read in phase 4)
         static_cast<double*>(a.Uout)[qc] = x;
         static_cast<double*>(a.Vout)[qc] = y;
         static_cast<double*>(a.Wout)[qc] = z;
       }
     }
-    if (want_alpha) rough_speeds2<EQ>(un, a.sp.wf[9], fx, fy);
   }
+  if constexpr (WIDE) {
+    if (!want_alpha) return;
+    __syncthreads();
+    if (role > 0) {
+      __syncthreads();  // (the one below)
+      return;
+    }
+    if (mine)
+#pragma unroll
+      for (int c = 0; c < M; ++c) un[c] = reinterpret_cast<double&>(r.H(0, c, k));
+  }
+  if (mine && want_alpha) rough_speeds2<EQ>(un, a.sp.wf[9], fx, fy);
   // wave speeds of the new state: in FP64 only where the FP32 ones come
   // within 2^-9 of the tile's largest (or are not usable)
   if (want_alpha) {
@@ -356,23 +400,40 @@ k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
   }
 }
 
-template <int EQ>
+template <int EQ, bool WIDE>
 cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
-  constexpr size_t bytes = Tile2D<EQ, 0>::bytes(kTileX2D + 4, kTileX2D + 1);
+  constexpr size_t bytes = Tile2D<EQ, 0>::bytes(kTileX2D + 4, kTileX2D + 1) +
+                           (WIDE ? xch_bytes<EQ, 0>(kTileX2D + 1) : 0);
   static unsigned configured = 0;  // devices whose limit is raised
-  if (const cudaError_t e = ensure_smem_limit(k_xsweep_2d_f64<EQ>, bytes, configured)) return e;
+  if (const cudaError_t e = ensure_smem_limit(k_xsweep_2d_f64<EQ, WIDE>, bytes, configured))
+    return e;
   const dim3 grid((a.nx + kTileX2D - 1) / kTileX2D, a.ny);
-  k_xsweep_2d_f64<EQ><<<grid, kThreads2D, bytes, s>>>(a, mode);
+  k_xsweep_2d_f64<EQ, WIDE><<<grid, WIDE ? kWideThreads2D : kThreads2D, bytes, s>>>(a, mode);
   return cudaGetLastError();
 }
 
+template <int EQ, bool WIDE>
+cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
+  constexpr int LI = (kRowsF64 + 1) * kColsF64;
+  constexpr size_t bytes = Tile2D<EQ, 1>::bytes((kRowsF64 + 4) * kColsF64, LI) +
+                           (WIDE ? xch_bytes<EQ, 1>(LI) : 0);
+  static unsigned configured = 0;  // devices whose limit is raised
+  if (const cudaError_t e = ensure_smem_limit(k_ysweep_2d_f64<EQ, WIDE>, bytes, configured))
+    return e;
+  const dim3 grid((a.nx + kColsF64 - 1) / kColsF64, (a.ny + kRowsF64 - 1) / kRowsF64);
+  k_ysweep_2d_f64<EQ, WIDE><<<grid, WIDE ? kWideThreads2D : kThreads2D, bytes, s>>>(a, mode);
+  return cudaGetLastError();
+}
+
+// The wide form of a sweep while its tiles number at most one per SM.
+template <int EQ>
+cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
+  const long long tiles = (long long)((a.nx + kTileX2D - 1) / kTileX2D) * a.ny;
+  return tiles <= 152 ? xsweep_f64<EQ, true>(mode, a, s) : xsweep_f64<EQ, false>(mode, a, s);
+}
 template <int EQ>
 cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
-  constexpr size_t bytes =
-      Tile2D<EQ, 1>::bytes((kRowsF64 + 4) * kColsF64, (kRowsF64 + 1) * kColsF64);
-  static unsigned configured = 0;  // devices whose limit is raised
-  if (const cudaError_t e = ensure_smem_limit(k_ysweep_2d_f64<EQ>, bytes, configured)) return e;
-  const dim3 grid((a.nx + kColsF64 - 1) / kColsF64, (a.ny + kRowsF64 - 1) / kRowsF64);
-  k_ysweep_2d_f64<EQ><<<grid, kThreads2D, bytes, s>>>(a, mode);
-  return cudaGetLastError();
+  const long long tiles = (long long)((a.nx + kColsF64 - 1) / kColsF64) *
+                          ((a.ny + kRowsF64 - 1) / kRowsF64);
+  return tiles <= 152 ? ysweep_f64<EQ, true>(mode, a, s) : ysweep_f64<EQ, false>(mode, a, s);
 }

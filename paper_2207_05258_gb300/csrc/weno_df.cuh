@@ -13,14 +13,14 @@
 // p_0 commutes with the characteristic projection. So only C needs the
 // projection, and it depends on differences of the data alone.
 //
-// A pair carries 48 bits, so C has an error of about 2^-46 phi |difference|.
-// While phi_1, phi_2 <= kWeakPhi that is below the FP64 evaluation's own
-// rounding (which starts from the full values); where it is not (shocks,
-// unresolved kinks, and whatever leaves the FP32 range: any overflow or NaN
-// fails the same test), the caller evaluates the item in FP64. Measured
-// against 128-bit arithmetic on Riemann problems, density waves, blast waves
-// and noise, N = 60 .. 3200: the 2-norm error of L^1 is 0.08 to 1.03 times
-// that of the all-FP64 form, of L^2 0.3 to 0.6, of v~ 0.01 to 1.0 times.
+// A pair carries 48 bits, so C has an error of about 2^-46 (phi_1 |p_1 - p_0|
+// + phi_2 |p_2 - p_0|). Items are evaluated in pairs while that stays below
+// the rounding of the FP64 form, which starts from the full values and has an
+// error of a few 2^-53 of alpha U: either phi_1, phi_2 <= kWeakPhi, or the sum
+// of the phi |differences| over the sides and fields that exceed it is at most
+// kWeakLevel of the local alpha U. Where neither holds (shocks, under-resolved
+// jumps, and whatever leaves the FP32 range: any overflow or NaN fails the
+// same test) the caller evaluates the item in FP64.
 #pragma once
 
 #include <type_traits>
@@ -69,10 +69,10 @@ struct LineWeights {
   float bmax;
 };
 
-// phi_l above which an item is evaluated in FP64. At 1/16 the errors quoted
-// above hold; 1/32 leaves a factor two. (1/4 would not do: v~ behind a
-// contact then has 5 times the FP64 form's largest error.)
-constexpr float kWeakPhi = 1.f / 32.f;
+// The bounds of the two tests above. (With the first alone, 1/16 would do and
+// 1/4 would not: v~ behind a contact then has 5 times the FP64 form's largest
+// error. 1/32 and 1/64 leave factors of two and more.)
+constexpr float kWeakPhi = 1.f / 32.f, kWeakLevel = 1.f / 64.f;
 
 // The smoothness indicators b_l of one side of an interface from the
 // differences of its stencil: y1 = f_{i-1} - f_i + H_i,
@@ -112,10 +112,11 @@ __device__ __forceinline__ void limiter_indicators(X q1, X q2, X lap, X du, X dV
   b2 = add(square(q2), eps);
 }
 
-// (phi_1 - phi_2) p + (phi_1 + phi_2) q from b_l in pairs; clears `weak` when
-// a phi_l exceeds kWeakPhi or the arithmetic has left its range.
+// (phi_1 - phi_2) p + (phi_1 + phi_2) q from b_l in pairs; where a phi_l
+// exceeds kWeakPhi, adds a bound of phi (|p| + |q|) to e (infinite or NaN
+// where the arithmetic has left its range).
 __device__ __forceinline__ D2 correction(D2 b0, D2 b1, D2 b2, D2 p, D2 q,
-                                         const LineWeights<D2>& w, bool& weak) {
+                                         const LineWeights<D2>& w, float& e) {
   // the indicators scaled by a power of two to at most 2 (products of three
   // of them and tau stay in range); tau = t^2 / 4 scales back by that power
   const float mx = fmaxf(b0.h, fmaxf(b1.h, b2.h));
@@ -131,29 +132,30 @@ __device__ __forceinline__ D2 correction(D2 b0, D2 b1, D2 b2, D2 p, D2 q,
   const D2 den = madd(mul(b1, b2), madd(w.g0, tau, b0), mul(mul(tau, b0), add(q1, q2)));
   const D2 num = mul(tau, madd(p, sub(n1, n2), mul(q, add(n1, n2))));
   const float top = tau.h * fmaxf(fabsf(n1.h), fabsf(n2.h));
-  weak &= (top <= kWeakPhi * den.h) & (mx < w.bmax);
+  if (!(top <= kWeakPhi * den.h)) e += top * fast_rcp(den.h) * (fabsf(p.h) + fabsf(q.h));
+  if (!(mx < w.bmax)) e = __int_as_float(0x7f800000);
   return div(num, den);
 }
 
 // 12 C of one side of an interface: 60 (p_1 - p_0) = 5 g - 3 m and
 // 60 (p_2 - p_0) = -5 g - 3 m with m = d + 2 lap.
 __device__ __forceinline__ D2 side_correction(D2 y1, D2 y2, D2 s, D2 d, D2 H0,
-                                              const LineWeights<D2>& w, bool& weak) {
+                                              const LineWeights<D2>& w, float& e) {
   const D2 g = add(y1, y2), lap = sub(y1, y2);
   D2 b0, b1, b2;
   flux_indicators(y1, y2, s, d, H0, g, lap, w.eps, b0, b1, b2);
   const D2 m = mul(add(d, scale(lap, 2.f)), dconst(-3.0 / 5.0));
-  return correction(b0, b1, b2, g, m, w, weak);
+  return correction(b0, b1, b2, g, m, w, e);
 }
 
 // 4 times the correction of dx v~_i to the linear dx q_0':
 // 4 (q_1 - q_0) = r - 2 lap, 4 (q_2 - q_0) = r + 2 lap.
 __device__ __forceinline__ D2 limiter_correction(D2 q1, D2 q2, D2 Vm, D2 Vp,
-                                                 const LineWeights<D2>& w, bool& weak) {
+                                                 const LineWeights<D2>& w, float& e) {
   const D2 lap = sub(q2, q1), du = add(q1, q2), dV = sub(Vm, Vp), r = sub(add(Vm, Vp), du);
   D2 b0, b1, b2;
   limiter_indicators(q1, q2, lap, du, dV, r, w.eps, b0, b1, b2);
-  return correction(b0, b1, b2, scale(lap, -2.f), r, w, weak);
+  return correction(b0, b1, b2, scale(lap, -2.f), r, w, e);
 }
 
 // In FP64 the value itself in the form of the paper's weights,
@@ -163,11 +165,20 @@ __device__ __forceinline__ D2 limiter_correction(D2 q1, D2 q2, D2 Vm, D2 Vp,
 // and a correction that cancels it would not resolve.
 __device__ __forceinline__ double weighted(double b0, double b1, double b2, double p0, double p1,
                                            double p2, const LineWeights<double>& w) {
-  double up, down;
-  Num<double>::exponent(fmax(b0, fmax(b1, b2)), up, down);
-  b0 = mul(b0, down);
-  b1 = mul(b1, down);
-  b2 = mul(b2, down);
+  // scaled to at most 2 by their exponent fields (the largest is the
+  // maximum of non-negative bit patterns)
+  const int top = max(__double2hiint(b0), max(__double2hiint(b1), __double2hiint(b2)));
+  const int e = top & 0x7ff00000;
+  const double up = __hiloint2double(e, 0);
+  auto shift = [&](double x) {  // x 2^-exponent; 0 below the normal range
+    const int h = __double2hiint(x) - (e - (1023 << 20));
+    return h >= (1 << 20) ? __hiloint2double(h, __double2loint(x)) : 0.0;
+  };
+  if (e != 0x7ff00000) {  // (an infinity or NaN stays and shows in the result)
+    b0 = shift(b0);
+    b1 = shift(b1);
+    b2 = shift(b2);
+  }
   const double t = add(fabs(sub(b0, b1)), fabs(sub(b0, b2)));
   const double tau = mul(mul(mul(0.25, t), t), up);
   const double P12 = mul(b1, b2), P = mul(b0, P12), tb = mul(tau, b0);
@@ -223,6 +234,13 @@ struct LineChar {
     hic = scale(ic, 0.5f);
     huc = mul(hic, un);
   }
+  // a field's bound in units of the density (the shear field is a momentum)
+  __device__ __forceinline__ float density_units(int q, float e) const {
+    if constexpr (M == 4 && std::is_same<X, D2>::value)
+      return q == 3 ? e * fast_rcp(c.h) : e;
+    else
+      return e;
+  }
   // kinetic energy per mass
   static __device__ __forceinline__ X kinetic(X un, X ut) {
     X s = square(un);
@@ -237,7 +255,7 @@ struct LineChar {
     __device__ __forceinline__ X field(int q) const {
       using P2 = typename Num<X>::Scale;
       const X p = pick2(q == 1, x0, A), r = pick2(q == 1, A, B);
-      const X v = add(p, scale(r, q == 0 ? P2(1) : q == 1 ? P2(-2) : P2(-1)));
+      const X v = scale_add(r, q == 0 ? P2(1) : q == 1 ? P2(-2) : P2(-1), p);
       if constexpr (M == 4) return pick2(q == 3, S, v);
       else return v;
     }
