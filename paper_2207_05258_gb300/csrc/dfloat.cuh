@@ -85,7 +85,8 @@ __device__ __forceinline__ D2 div(D2 n, D2 d) {
   // n - q d, exact in the leading words
   float m = __fmaf_rn(-q, d.h, n.h);
   m = __fadd_rn(m, __fmaf_rn(-q, d.l, n.l));
-  return renorm(q, __fmul_rn(m, r));
+  const float h = __fmaf_rn(m, r, q);  // renorm(q, m r)
+  return D2{h, __fmaf_rn(m, r, -__fadd_rn(h, -q))};
 }
 // 1 / sqrt(x): the hardware approximation and one Newton step in pairs
 __device__ __forceinline__ D2 rsqrt2(D2 x) {
@@ -157,6 +158,78 @@ __device__ __forceinline__ D2 pick2(bool c, D2 a, D2 b) {
 }
 __device__ __forceinline__ double pick2(bool c, double a, double b) { return c ? a : b; }
 
+// Two pairs in the lanes of packed FP32 instructions (fma / add / mul .f32x2,
+// which take 2 cycles for both lanes, negated operands included): half the
+// instructions to issue and to fetch. Each lane rounds as the scalar form.
+struct Q2 {
+  float2 h, l;
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ Q2 both(D2 a, D2 b) {
+  return Q2{make_float2(a.h, b.h), make_float2(a.l, b.l)};
+}
+__device__ __forceinline__ Q2 both(D2 a) { return both(a, a); }
+__device__ __forceinline__ D2 first(Q2 a) { return D2{a.h.x, a.l.x}; }
+__device__ __forceinline__ D2 second(Q2 a) { return D2{a.h.y, a.l.y}; }
+__device__ __forceinline__ Q2 renorm(float2 s, float2 e) {
+  const float2 h = __fadd2_rn(s, e);
+  return Q2{h, __fadd2_rn(e, neg2(__fadd2_rn(h, neg2(s))))};
+}
+__device__ __forceinline__ Q2 neg(Q2 a) { return Q2{neg2(a.h), neg2(a.l)}; }
+__device__ __forceinline__ Q2 add(Q2 a, Q2 b) {
+  const float2 s = __fadd2_rn(a.h, b.h);
+  const float2 t = __fadd2_rn(s, neg2(a.h));
+  const float2 e = __fadd2_rn(__fadd2_rn(a.h, neg2(__fadd2_rn(s, neg2(t)))),
+                              __fadd2_rn(b.h, neg2(t)));
+  return renorm(s, __fadd2_rn(e, __fadd2_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Q2 sub(Q2 a, Q2 b) { return add(a, neg(b)); }
+__device__ __forceinline__ Q2 mul(Q2 a, Q2 b) {
+  const float2 p = __fmul2_rn(a.h, b.h);
+  float2 e = __ffma2_rn(a.h, b.h, neg2(p));
+  e = __ffma2_rn(a.h, b.l, e);
+  e = __ffma2_rn(a.l, b.h, e);
+  return renorm(p, e);
+}
+__device__ __forceinline__ Q2 mul(Q2 a, float c) {
+  const float2 p = __fmul2_rn(a.h, dup(c));
+  return renorm(p, __ffma2_rn(a.l, dup(c), __ffma2_rn(a.h, dup(c), neg2(p))));
+}
+__device__ __forceinline__ Q2 square(Q2 a) {
+  const float2 p = __fmul2_rn(a.h, a.h);
+  return renorm(p, __ffma2_rn(__fadd2_rn(a.h, a.h), a.l, __ffma2_rn(a.h, a.h, neg2(p))));
+}
+__device__ __forceinline__ Q2 scale(Q2 a, float2 p2) {
+  return Q2{__fmul2_rn(a.h, p2), __fmul2_rn(a.l, p2)};
+}
+__device__ __forceinline__ Q2 scale(Q2 a, float p2) { return scale(a, dup(p2)); }
+__device__ __forceinline__ Q2 scale_add(Q2 b, float a, Q2 c) { return add(scale(b, a), c); }
+__device__ __forceinline__ Q2 abs2(Q2 a) { return both(abs2(first(a)), abs2(second(a))); }
+__device__ __forceinline__ Q2 madd(Q2 a, Q2 b, Q2 c) {
+  const float2 p = __fmul2_rn(a.h, b.h);
+  float2 e = __ffma2_rn(a.h, b.h, neg2(p));
+  e = __ffma2_rn(a.h, b.l, e);
+  e = __ffma2_rn(a.l, b.h, e);
+  const float2 s = __fadd2_rn(p, c.h);
+  const float2 t = __fadd2_rn(s, neg2(p));
+  const float2 r = __fadd2_rn(__fadd2_rn(p, neg2(__fadd2_rn(s, neg2(t)))),
+                              __fadd2_rn(c.h, neg2(t)));
+  return renorm(s, __fadd2_rn(r, __fadd2_rn(e, c.l)));
+}
+__device__ __forceinline__ Q2 div(Q2 n, Q2 d) {
+  const float2 r = make_float2(fast_rcp(d.h.x), fast_rcp(d.h.y));
+  const float2 q = __fmul2_rn(n.h, r);
+  float2 m = __ffma2_rn(neg2(q), d.h, n.h);
+  m = __fadd2_rn(m, __ffma2_rn(neg2(q), d.l, n.l));
+  const float2 h = __ffma2_rn(m, r, q);
+  return Q2{h, __ffma2_rn(m, r, neg2(__fadd2_rn(h, neg2(q))))};
+}
+
+__device__ __forceinline__ Q2 pick2(bool c, Q2 a, Q2 b) {
+  return both(pick2(c, first(a), first(b)), pick2(c, second(a), second(b)));
+}
+
 // What generic code needs to know of a number type X (D2 or double).
 template <class X>
 struct Num;
@@ -171,6 +244,11 @@ struct Num<D2> {
     up = __uint_as_float(e);
     down = __uint_as_float((254u << 23) - e);
   }
+};
+template <>
+struct Num<Q2> {
+  using Scale = float;
+  static __device__ __forceinline__ Q2 c(double x) { return both(dconst(x)); }
 };
 template <>
 struct Num<double> {

@@ -12,7 +12,13 @@
 #include "internal.h"
 #include "weno_df.cuh"
 
+#ifndef HWENO_UNROLL_FIELDS
+#define HWENO_UNROLL_FIELDS 1
+#endif
+
 namespace hweno {
+
+constexpr int kUnrollFields = HWENO_UNROLL_FIELDS;
 
 // Shared memory of a tile of L loaded points (flat index k; the neighbours
 // of k along the line are k - S and k + S) and LI interfaces or updated
@@ -64,15 +70,15 @@ struct LineTile {
     else return d(2 * M + MF + c, k);
   }
   __device__ __forceinline__ double& extra(int r, int k) const { return d(2 * M + 2 * MF + r, k); }
-  // split pairs of side sd (0: H^+, P; 1: H^-, M)
+  // split pairs of side sd (0: H^+, P; 1: -H^-, -M)
   __device__ __forceinline__ D2& H(int sd, int c, int k) const { return p(sd * M + c, k); }
   __device__ __forceinline__ D2& X(int sd, int c, int k) const { return p((2 + sd) * M + c, k); }
   __device__ __forceinline__ D2 dU(int c, int k) const {
-    if constexpr (SLIM) return mul(sub(X(0, c, k), X(1, c, k)), ial);
+    if constexpr (SLIM) return mul(add(X(0, c, k), X(1, c, k)), ial);
     else return p(4 * M + c, k);
   }
   __device__ __forceinline__ D2 Nx(int c, int k) const {
-    if constexpr (SLIM) return mul(sub(H(0, c, k), H(1, c, k)), ial);
+    if constexpr (SLIM) return mul(add(H(0, c, k), H(1, c, k)), ial);
     else return p(5 * M + c, k);
   }
   // eigen-system inputs: sqrt(rho), un, H, ut
@@ -110,7 +116,7 @@ __device__ __forceinline__ void point_pair(const T& r, int c, int k, double N, d
   const D2 nx = mul(dxp, to_pair(N)), x = mul(dxp, to_pair(h)), y = mul(alp, nx);
   if constexpr (!T::SLIM) r.p(5 * T::M + c, k) = nx;
   r.H(0, c, k) = scale(add(x, y), 0.5f);
-  r.H(1, c, k) = scale(sub(x, y), 0.5f);
+  r.H(1, c, k) = scale(sub(y, x), 0.5f);
 }
 template <class T>
 __device__ __forceinline__ void point_pairs(const T& r, int k, const double* N, const double* h,
@@ -138,7 +144,7 @@ __device__ __forceinline__ void edge_pair(const T& r, int c, int k, int S, D2 al
   const D2 dF = to_pair(sub(r.F(c, k + S), r.F(c, k))), au = mul(alp, dU);
   if constexpr (!T::SLIM) r.p(4 * T::M + c, k) = dU;
   r.X(0, c, k) = scale(add(dF, au), 0.5f);
-  r.X(1, c, k) = scale(sub(dF, au), 0.5f);
+  r.X(1, c, k) = scale(sub(au, dF), 0.5f);
 }
 template <class T>
 __device__ __forceinline__ void edge_pairs(const T& r, int k, int S, D2 alp) {
@@ -153,7 +159,7 @@ __device__ __forceinline__ void edge_pairs(const T& r, int k, int S, D2 alp) {
     const D2 dF = T::EUL && c == 0 ? dU[T::kn] : to_pair(sub(r.F(c, k + S), r.F(c, k)));
     const D2 au = mul(alp, dU[c]);
     r.X(0, c, k) = scale(add(dF, au), 0.5f);
-    r.X(1, c, k) = scale(sub(dF, au), 0.5f);
+    r.X(1, c, k) = scale(sub(au, dF), 0.5f);
   }
 }
 
@@ -199,10 +205,11 @@ struct LineData<double, T> {
                                       const SchemeParams& sp_)
       : r(r_), S(S_), alpha(al), dx(d), sp(sp_) {}
   __device__ __forceinline__ double H(int sd, int c, int k) const {
-    return mul(0.5 * dx, madd(sd ? -alpha : alpha, r.N(c, k), r.h(c, k)));
+    return mul(0.5 * dx, madd(alpha, r.N(c, k), sd ? -r.h(c, k) : r.h(c, k)));
   }
   __device__ __forceinline__ double X(int sd, int c, int k) const {
-    return mul(0.5, madd(sd ? -alpha : alpha, dU(c, k), sub(r.F(c, k + S), r.F(c, k))));
+    const double dF = sub(r.F(c, k + S), r.F(c, k));
+    return mul(0.5, madd(alpha, dU(c, k), sd ? -dF : dF));
   }
   __device__ __forceinline__ double dU(int c, int k) const {
     return sub(r.U(c, k + S), r.U(c, k));
@@ -259,21 +266,32 @@ __device__ __forceinline__ X add_if(bool c, X a, X y) {
 // The stencil differences of side sd of the interface between k and k + S,
 // component c (the arguments of side_correction): the "+" side is about point
 // k, the "-" side about k + S. The latter reverses the stencil and negates H;
-// with M the difference of f^- along an edge, all five quantities are the "+"
-// side's expressions in M and H^- times -1.
+// with -H^- and -M for H^+ and P (M the difference of f^- along an edge) its
+// expressions are those of the "+" side.
 template <class X, class T>
 __device__ __forceinline__ void side_differences(const LineData<X, T>& in, int sd, int c, int k,
                                                  int S, X* x) {
   using P2 = typename Num<X>::Scale;
-  const bool sg = sd != 0;
   const int k0 = sd ? k + S : k, km = sd ? k0 + S : k0 - S, kp = sd ? k : k0 + S;
   // the edges (k - S, k), (k, k + S) or (k + S, k + 2 S), (k, k + S)
   const X Hm = in.H(sd, c, km), H0 = in.H(sd, c, k0), Hp = in.H(sd, c, kp);
-  x[0] = flip(sg, sub(H0, in.X(sd, c, sd ? k0 : km)));
-  x[1] = flip(sg, sub(H0, in.X(sd, c, k)));
-  x[2] = flip(sg, scale_add(H0, P2(-2), add(Hm, Hp)));
-  x[3] = flip(sg, sub(Hm, Hp));
-  x[4] = flip(sg, H0);
+  x[0] = sub(H0, in.X(sd, c, sd ? k0 : km));
+  x[1] = sub(H0, in.X(sd, c, k));
+  x[2] = scale_add(H0, P2(-2), add(Hm, Hp));
+  x[3] = sub(Hm, Hp);
+  x[4] = H0;
+}
+// Both sides packed.
+template <class T>
+__device__ __forceinline__ void sides_differences(const LineData<D2, T>& in, int c, int k, int S,
+                                                  Q2* x) {
+  auto at = [&](int a, int b) { return both(in.H(0, c, a), in.H(1, c, b)); };
+  const Q2 Hm = at(k - S, k + 2 * S), H0 = at(k, k + S), Hp = at(k + S, k);
+  x[0] = sub(H0, both(in.X(0, c, k - S), in.X(1, c, k + S)));
+  x[1] = sub(H0, both(in.X(0, c, k), in.X(1, c, k)));
+  x[2] = scale_add(H0, -2.f, add(Hm, Hp));
+  x[3] = sub(Hm, Hp);
+  x[4] = H0;
 }
 
 template <class T, class X, int DIR>
@@ -390,6 +408,54 @@ __device__ __forceinline__ void interface_value(const LineData<X, T>& in,
   }
 }
 
+// Both sides as interface_side, packed: the same operations on the two lanes.
+template <int DIR, class T>
+__device__ __forceinline__ float interface_sides(const LineData<D2, T>& in,
+                                                 const CharOf<T, D2, DIR>& ch,
+                                                 const LineWeights<D2>& w_, int k, int S, D2* f,
+                                                 D2* lin) {
+  constexpr int M = T::M;
+  const LineWeights<Q2> w{both(w_.g0), both(w_.g1), both(w_.g2), both(w_.eps), w_.bmax};
+  float2 sum = make_float2(0.f, 0.f);
+  auto sides = [&](int q, Q2 y1, Q2 y2, Q2 s, Q2 d, Q2 H0) {
+    float2 e = make_float2(0.f, 0.f);
+    const Q2 v = side_correction(y1, y2, s, d, H0, w, e);
+    sum.x += T::EUL ? ch.density_units(q, e.x) : e.x;
+    sum.y += T::EUL ? ch.density_units(q, e.y) : e.y;
+    return add(first(v), second(v));
+  };
+  Q2 x[M][5];
+#pragma unroll
+  for (int c = 0; c < M; ++c) {
+    sides_differences(in, c, k, S, x[c]);
+    const Q2 l = linear_part(x[c][0], x[c][1], x[c][3]);
+    lin[c] = add(first(l), second(l));
+  }
+  if constexpr (T::EUL) {
+    const auto chq = ch.packed();
+    typename LineChar<Q2, M, DIR>::Factors a[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      Q2 y[M];
+#pragma unroll
+      for (int c = 0; c < M; ++c) y[c] = x[c][v];
+      a[v] = chq.factors(y);
+    }
+#pragma unroll
+    for (int c = 0; c < M; ++c) f[c] = D2{0.f, 0.f};
+#pragma unroll kUnrollFields
+    for (int q = 0; q < M; ++q) {
+      const D2 y = sides(q, a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q),
+                         a[4].field(q));
+#pragma unroll
+      for (int c = 0; c < M; ++c) f[c] = pick2(q == c, y, f[c]);
+    }
+  } else {
+    f[0] = sides(0, x[0][0], x[0][1], x[0][2], x[0][3], x[0][4]);
+  }
+  return sum.x + sum.y;
+}
+
 // c of the interface between points k and k + S; in pairs, false when the
 // correction is not small (the values are then not to be used).
 template <class X, int DIR, class T>
@@ -399,14 +465,18 @@ __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double 
   const LineWeights<X> w = line_weights<X>(sp, false);
   const auto ch = char_system<DIR>(in, k, true);
   X f[T::M], lin[T::M];
+  if constexpr (std::is_same<X, double>::value) {
 #pragma unroll
-  for (int c = 0; c < T::M; ++c) f[c] = lin[c] = X{};
-  float e = 0.f;
+    for (int c = 0; c < T::M; ++c) f[c] = lin[c] = X{};
 #pragma unroll 1
-  for (int sd = 0; sd < 2; ++sd) e += interface_side<DIR>(in, ch, w, sd, k, S, f, lin);
-  interface_value<DIR>(in, ch, k, alpha, f, lin, cc);
-  if constexpr (std::is_same<X, double>::value) return true;
-  else return interface_weak(r, k, S, e, alpha, sp);
+    for (int sd = 0; sd < 2; ++sd) interface_side<DIR>(in, ch, w, sd, k, S, f, lin);
+    interface_value<DIR>(in, ch, k, alpha, f, lin, cc);
+    return true;
+  } else {
+    const float e = interface_sides<DIR>(in, ch, w, k, S, f, lin);
+    interface_value<DIR>(in, ch, k, alpha, f, lin, cc);
+    return interface_weak(r, k, S, e, alpha, sp);
+  }
 }
 
 // The derivative flux dx (h-hat^+ + h-hat^-) of component c at the interface
@@ -542,11 +612,27 @@ __device__ __forceinline__ bool limiter_line(const T& r, int k, int S, double dx
       }
 #pragma unroll
       for (int c = 0; c < M; ++c) z[c] = X{};
+      if constexpr (std::is_same<X, double>::value) {
 #pragma unroll 1
-      for (int q = 0; q < M; ++q) {
-        const X y = limit(q, a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q));
+        for (int q = 0; q < M; ++q) {
+          const X y = limit(q, a[0].field(q), a[1].field(q), a[2].field(q), a[3].field(q));
 #pragma unroll
-        for (int c = 0; c < M; ++c) z[c] = pick2(q == c, y, z[c]);
+          for (int c = 0; c < M; ++c) z[c] = pick2(q == c, y, z[c]);
+        }
+      } else {  // two fields packed (three fields: the last one twice)
+        const LineWeights<Q2> wq{both(w.g0), both(w.g1), both(w.g2), both(w.eps), w.bmax};
+#pragma unroll kUnrollFields
+        for (int h = 0; h < 2; ++h) {
+          const int qa = 2 * h, qb = M == 3 && h == 1 ? 2 : qa + 1;
+          auto two = [&](int v) { return both(a[v].field(qa), a[v].field(qb)); };
+          float2 e = make_float2(0.f, 0.f);
+          const Q2 y = limiter_correction(two(0), two(1), two(2), two(3), wq, e);
+          sum += ch.density_units(qa, e.x);
+          if (qb != qa) sum += ch.density_units(qb, e.y);
+#pragma unroll
+          for (int c = 0; c < M; ++c)
+            z[c] = pick2(c == qa, first(y), pick2(c == qb, second(y), z[c]));
+        }
       }
     }
   } else {

@@ -112,48 +112,75 @@ __device__ __forceinline__ void limiter_indicators(X q1, X q2, X lap, X du, X dV
   b2 = add(square(q2), eps);
 }
 
+// A word of a pair and of two packed pairs: what correction() does lane by
+// lane.
+__device__ __forceinline__ void to_unit(float mx, float& up, float& down) {
+  Num<D2>::exponent(mx, up, down);
+}
+__device__ __forceinline__ void to_unit(float2 mx, float2& up, float2& down) {
+  to_unit(mx.x, up.x, down.x);
+  to_unit(mx.y, up.y, down.y);
+}
+__device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(a, fmaxf(b, c)); }
+__device__ __forceinline__ float2 max3(float2 a, float2 b, float2 c) {
+  return make_float2(max3(a.x, b.x, c.x), max3(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float quarter(float a) { return 0.25f * a; }
+__device__ __forceinline__ float2 quarter(float2 a) { return __fmul2_rn(a, dup(0.25f)); }
+__device__ __forceinline__ void bound(float& e, float tau, float n1, float n2, float den, float p,
+                                      float q, float mx, float bmax) {
+  const float top = tau * fmaxf(fabsf(n1), fabsf(n2));
+  if (!(top <= kWeakPhi * den)) e += top * fast_rcp(den) * (fabsf(p) + fabsf(q));
+  if (!(mx < bmax)) e = __int_as_float(0x7f800000);
+}
+__device__ __forceinline__ void bound(float2& e, float2 tau, float2 n1, float2 n2, float2 den,
+                                      float2 p, float2 q, float2 mx, float bmax) {
+  bound(e.x, tau.x, n1.x, n2.x, den.x, p.x, q.x, mx.x, bmax);
+  bound(e.y, tau.y, n1.y, n2.y, den.y, p.y, q.y, mx.y, bmax);
+}
+
 // (phi_1 - phi_2) p + (phi_1 + phi_2) q from b_l in pairs; where a phi_l
 // exceeds kWeakPhi, adds a bound of phi (|p| + |q|) to e (infinite or NaN
-// where the arithmetic has left its range).
-__device__ __forceinline__ D2 correction(D2 b0, D2 b1, D2 b2, D2 p, D2 q,
-                                         const LineWeights<D2>& w, float& e) {
+// where the arithmetic has left its range). X: D2, or Q2 with e per lane.
+template <class X, class E>
+__device__ __forceinline__ X correction(X b0, X b1, X b2, X p, X q, const LineWeights<X>& w, E& e) {
   // the indicators scaled by a power of two to at most 2 (products of three
   // of them and tau stay in range); tau = t^2 / 4 scales back by that power
-  const float mx = fmaxf(b0.h, fmaxf(b1.h, b2.h));
-  float up, down;
-  Num<D2>::exponent(mx, up, down);
+  const E mx = max3(b0.h, b1.h, b2.h);
+  E up, down;
+  to_unit(mx, up, down);
   b0 = scale(b0, down);
   b1 = scale(b1, down);
   b2 = scale(b2, down);
-  const D2 e1 = sub(b0, b1), e2 = sub(b0, b2);
-  const D2 tau = scale(square(add(abs2(e1), abs2(e2))), 0.25f * up);
-  const D2 q1 = mul(w.g1, b2), q2 = mul(w.g2, b1);
-  const D2 n1 = mul(q1, e1), n2 = mul(q2, e2);
-  const D2 den = madd(mul(b1, b2), madd(w.g0, tau, b0), mul(mul(tau, b0), add(q1, q2)));
-  const D2 num = mul(tau, madd(p, sub(n1, n2), mul(q, add(n1, n2))));
-  const float top = tau.h * fmaxf(fabsf(n1.h), fabsf(n2.h));
-  if (!(top <= kWeakPhi * den.h)) e += top * fast_rcp(den.h) * (fabsf(p.h) + fabsf(q.h));
-  if (!(mx < w.bmax)) e = __int_as_float(0x7f800000);
+  const X e1 = sub(b0, b1), e2 = sub(b0, b2);
+  const X tau = scale(square(add(abs2(e1), abs2(e2))), quarter(up));
+  const X q1 = mul(w.g1, b2), q2 = mul(w.g2, b1);
+  const X n1 = mul(q1, e1), n2 = mul(q2, e2);
+  const X den = madd(mul(b1, b2), madd(w.g0, tau, b0), mul(mul(tau, b0), add(q1, q2)));
+  const X num = mul(tau, madd(p, sub(n1, n2), mul(q, add(n1, n2))));
+  bound(e, tau.h, n1.h, n2.h, den.h, p.h, q.h, mx, w.bmax);
   return div(num, den);
 }
 
-// 12 C of one side of an interface: 60 (p_1 - p_0) = 5 g - 3 m and
-// 60 (p_2 - p_0) = -5 g - 3 m with m = d + 2 lap.
-__device__ __forceinline__ D2 side_correction(D2 y1, D2 y2, D2 s, D2 d, D2 H0,
-                                              const LineWeights<D2>& w, float& e) {
-  const D2 g = add(y1, y2), lap = sub(y1, y2);
-  D2 b0, b1, b2;
+// 12 C of one side of an interface (Q2: of both): 60 (p_1 - p_0) = 5 g - 3 m
+// and 60 (p_2 - p_0) = -5 g - 3 m with m = d + 2 lap.
+template <class X, class E>
+__device__ __forceinline__ X side_correction(X y1, X y2, X s, X d, X H0, const LineWeights<X>& w,
+                                             E& e) {
+  const X g = add(y1, y2), lap = sub(y1, y2);
+  X b0, b1, b2;
   flux_indicators(y1, y2, s, d, H0, g, lap, w.eps, b0, b1, b2);
-  const D2 m = mul(add(d, scale(lap, 2.f)), dconst(-3.0 / 5.0));
+  const X m = mul(add(d, scale(lap, 2.f)), Num<X>::c(-3.0 / 5.0));
   return correction(b0, b1, b2, g, m, w, e);
 }
 
 // 4 times the correction of dx v~_i to the linear dx q_0':
 // 4 (q_1 - q_0) = r - 2 lap, 4 (q_2 - q_0) = r + 2 lap.
-__device__ __forceinline__ D2 limiter_correction(D2 q1, D2 q2, D2 Vm, D2 Vp,
-                                                 const LineWeights<D2>& w, float& e) {
-  const D2 lap = sub(q2, q1), du = add(q1, q2), dV = sub(Vm, Vp), r = sub(add(Vm, Vp), du);
-  D2 b0, b1, b2;
+template <class X, class E>
+__device__ __forceinline__ X limiter_correction(X q1, X q2, X Vm, X Vp, const LineWeights<X>& w,
+                                                E& e) {
+  const X lap = sub(q2, q1), du = add(q1, q2), dV = sub(Vm, Vp), r = sub(add(Vm, Vp), du);
+  X b0, b1, b2;
   limiter_indicators(q1, q2, lap, du, dV, r, w.eps, b0, b1, b2);
   return correction(b0, b1, b2, scale(lap, -2.f), r, w, e);
 }
@@ -234,6 +261,22 @@ struct LineChar {
     hic = scale(ic, 0.5f);
     huc = mul(hic, un);
   }
+  // what factors() needs, in both lanes
+  __device__ __forceinline__ LineChar<Q2, M, DIR> packed() const {
+    LineChar<Q2, M, DIR> r;
+    if constexpr (std::is_same<X, D2>::value) {
+      r.b = both(b);
+      r.bq = both(bq);
+      r.bu = both(bu);
+      r.hic = both(hic);
+      r.huc = both(huc);
+      if constexpr (M == 4) {
+        r.bt = both(bt);
+        r.ut = both(ut);
+      }
+    }
+    return r;
+  }
   // a field's bound in units of the density (the shear field is a momentum)
   __device__ __forceinline__ float density_units(int q, float e) const {
     if constexpr (M == 4 && std::is_same<X, D2>::value)
@@ -285,7 +328,8 @@ struct LineChar {
 
 // 60 times an interface's linear part relative to (F_i + F_{i+1}) / 2, one
 // component: the sum of 11 y1 + 19 y2 + 3 d over the two sides.
-__device__ __forceinline__ D2 linear_part(D2 y1, D2 y2, D2 d) {
+template <class X>
+__device__ __forceinline__ X linear_part(X y1, X y2, X d) {
   return add(mul(y1, 11.f), add(mul(y2, 19.f), mul(d, 3.f)));
 }
 
