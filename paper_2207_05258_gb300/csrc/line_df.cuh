@@ -386,11 +386,39 @@ __device__ __forceinline__ bool interface_weak(const T& r, int k, int S, float e
   return e <= 12.f * kWeakLevel * scale_pair(alpha).h * level;
 }
 
-// c from the sums over both sides.
+// The linear part in pairs has an error of 2^-48 of the differences it is made
+// of, that in FP64 one of F's rounding. 2D scalar equations take it in FP64
+// where a difference exceeds 2^-3 of F (coarse grids, sonic points: error of
+// L^1 against the plain FP64 form at 48 x 60 1.25 -> 0.46); in 1D and for
+// Euler the pairs' was the smaller error at every size.
+template <class T>
+__device__ __forceinline__ bool fine_grid(const LineData<D2, T>& in, int k, int S) {
+  if constexpr (T::EUL || !T::SLIM) return true;
+  const float top = fmaxf(fmaxf(fabsf(in.H(0, 0, k).h), fabsf(in.H(1, 0, k + S).h)),
+                          fmaxf(fabsf(in.X(0, 0, k).h), fabsf(in.X(1, 0, k).h)));
+  const float F = fmaxf(fabsf(to_float(in.r.F(0, k))), fabsf(to_float(in.r.F(0, k + S))));
+  return top <= 0x1p-3f * F;
+}
+// The linear part of the scalar c in FP64.
+template <class T>
+__device__ __forceinline__ double linear_part_fp64(const T& r, int k, int S, double alpha,
+                                                   double dx) {
+  const int m = k - S, p = k + S, q = k + 2 * S;
+  const double h = madd(33.0, sub(r.h(0, k), r.h(0, p)), mul(3.0, sub(r.h(0, m), r.h(0, q))));
+  const double N = madd(27.0, add(r.N(0, k), r.N(0, p)), mul(3.0, add(r.N(0, m), r.N(0, q))));
+  const double F = sub(sub(r.F(0, q), r.F(0, p)), sub(r.F(0, k), r.F(0, m)));
+  const double U = madd(27.0, sub(r.U(0, p), r.U(0, k)), mul(11.0, sub(r.U(0, q), r.U(0, m))));
+  const double x = madd(11.0, F, mul(alpha, madd(dx, N, -U)));
+  return mul(1.0 / 120.0, madd(dx, h, x));
+}
+
+// c from the sums over both sides (lin64: the scalar linear part, where
+// fine_grid is false).
 template <int DIR, class X, class T>
 __device__ __forceinline__ void interface_value(const LineData<X, T>& in,
-                                                const CharOf<T, X, DIR>& ch, int k, double alpha,
-                                                X* f, const X* lin, double* cc) {
+                                                const CharOf<T, X, DIR>& ch, int k, int S,
+                                                double alpha, X* f, const X* lin, double lin64,
+                                                double* cc) {
   constexpr int M = T::M;
   if constexpr (T::EUL) {
     X out[M];
@@ -406,6 +434,34 @@ __device__ __forceinline__ void interface_value(const LineData<X, T>& in,
     else
       cc[c] = to_double(madd(dconst(1.0 / 60.0), lin[c], mul(f[c], dconst(1.0 / 12.0))));
   }
+  if constexpr (!T::EUL && std::is_same<X, D2>::value)
+    if (!fine_grid(in, k, S)) cc[0] = add(lin64, to_double(mul(f[0], dconst(1.0 / 12.0))));
+}
+
+// The derivative flux dx (h-hat^+ + h-hat^-) of component c at the interface
+// between k and k + S: both sides' p_0' of Sec. 2.1 in terms of F, U, h, N.
+template <class T>
+__device__ __forceinline__ double derivative_flux_fp64(const T& r, int c, int k, int S,
+                                                       double alpha, double dx) {
+  const double kU = mul(0.125, alpha), kh = mul(dx, 1.0 / 24.0), kv = mul(alpha, kh);
+  const int m = k - S, p = k + S, q = k + 2 * S;
+  const double t0 = sub(r.F(c, p), r.F(c, k)), t1 = sub(r.F(c, q), r.F(c, m));
+  const double su = sub(sub(r.U(c, q), r.U(c, p)), sub(r.U(c, k), r.U(c, m)));
+  const double sh = madd(-7.0, add(r.h(c, k), r.h(c, p)), add(r.h(c, m), r.h(c, q)));
+  const double sv = madd(3.0, sub(r.N(c, k), r.N(c, p)), sub(r.N(c, m), r.N(c, q)));
+  return madd(1.875, t0, madd(-0.125, t1, madd(kU, su, madd(kh, sh, mul(kv, sv)))));
+}
+
+// The same from both sides' differences: Euler in pairs (45 fewer FP64
+// instructions per point and stage of 1D: batch of Riemann problems 7.52 ->
+// 6.74 ms); scalar equations in FP64, where the pairs' error was up to twice
+// that on grids of less than 100 points.
+template <class T>
+__device__ __forceinline__ double derivative_flux(const LineData<D2, T>& in, const Q2* x, int c,
+                                                  int k, int S, double alpha, double dx) {
+  if constexpr (!T::EUL) return derivative_flux_fp64(in.r, c, k, S, alpha, dx);
+  const Q2 d = derivative_part(x[0], x[1], x[2], x[3], x[4]);
+  return to_double(scale(sub(first(d), second(d)), 0.25f));
 }
 
 // Both sides as interface_side, packed: the same operations on the two lanes.
@@ -413,7 +469,7 @@ template <int DIR, class T>
 __device__ __forceinline__ float interface_sides(const LineData<D2, T>& in,
                                                  const CharOf<T, D2, DIR>& ch,
                                                  const LineWeights<D2>& w_, int k, int S, D2* f,
-                                                 D2* lin) {
+                                                 D2* lin, double alpha, double dx, double* dd) {
   constexpr int M = T::M;
   const LineWeights<Q2> w{both(w_.g0), both(w_.g1), both(w_.g2), both(w_.eps), w_.bmax};
   float2 sum = make_float2(0.f, 0.f);
@@ -430,6 +486,7 @@ __device__ __forceinline__ float interface_sides(const LineData<D2, T>& in,
     sides_differences(in, c, k, S, x[c]);
     const Q2 l = linear_part(x[c][0], x[c][1], x[c][3]);
     lin[c] = add(first(l), second(l));
+    dd[c] = derivative_flux(in, x[c], c, k, S, alpha, dx);
   }
   if constexpr (T::EUL) {
     const auto chq = ch.packed();
@@ -456,11 +513,13 @@ __device__ __forceinline__ float interface_sides(const LineData<D2, T>& in,
   return sum.x + sum.y;
 }
 
-// c of the interface between points k and k + S; in pairs, false when the
-// correction is not small (the values are then not to be used).
+// c (to cc) and, in pairs, the derivative flux (to dd) of the interface between
+// points k and k + S; in pairs, false when the correction is not small (the
+// values are then not to be used).
 template <class X, int DIR, class T>
 __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double alpha, double dx,
-                                               const SchemeParams& sp, double* cc) {
+                                               const SchemeParams& sp, double* cc,
+                                               double* dd = nullptr) {
   const LineData<X, T> in(r, S, alpha, dx, sp);
   const LineWeights<X> w = line_weights<X>(sp, false);
   const auto ch = char_system<DIR>(in, k, true);
@@ -470,26 +529,15 @@ __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double 
     for (int c = 0; c < T::M; ++c) f[c] = lin[c] = X{};
 #pragma unroll 1
     for (int sd = 0; sd < 2; ++sd) interface_side<DIR>(in, ch, w, sd, k, S, f, lin);
-    interface_value<DIR>(in, ch, k, alpha, f, lin, cc);
+    interface_value<DIR>(in, ch, k, S, alpha, f, lin, 0.0, cc);
     return true;
   } else {
-    const float e = interface_sides<DIR>(in, ch, w, k, S, f, lin);
-    interface_value<DIR>(in, ch, k, alpha, f, lin, cc);
+    const float e = interface_sides<DIR>(in, ch, w, k, S, f, lin, alpha, dx, dd);
+    double lin64 = 0.0;
+    if (!fine_grid(in, k, S)) lin64 = linear_part_fp64(r, k, S, alpha, dx);
+    interface_value<DIR>(in, ch, k, S, alpha, f, lin, lin64, cc);
     return interface_weak(r, k, S, e, alpha, sp);
   }
-}
-
-// The derivative flux dx (h-hat^+ + h-hat^-) of component c at the interface
-// between k and k + S: both sides' p_0' of Sec. 2.1 in terms of F, U, h, N.
-template <class T>
-__device__ __forceinline__ double derivative_flux_fp64(const T& r, int c, int k, int S, double kU,
-                                                       double kh, double kv) {
-  const int m = k - S, p = k + S, q = k + 2 * S;
-  const double t0 = sub(r.F(c, p), r.F(c, k)), t1 = sub(r.F(c, q), r.F(c, m));
-  const double su = sub(sub(r.U(c, q), r.U(c, p)), sub(r.U(c, k), r.U(c, m)));
-  const double sh = madd(-7.0, add(r.h(c, k), r.h(c, p)), add(r.h(c, m), r.h(c, q)));
-  const double sv = madd(3.0, sub(r.N(c, k), r.N(c, p)), sub(r.N(c, m), r.N(c, q)));
-  return madd(1.875, t0, madd(-0.125, t1, madd(kU, su, madd(kh, sh, mul(kv, sv)))));
 }
 
 // The limiter's four differences at point k, component c.
@@ -778,8 +826,16 @@ __device__ __forceinline__ void listed_items(const T& r, const unsigned short* l
   const bool few_f = nf <= 3 * gf * nw, few_l = nl <= 3 * gl * nw;
   const int uf = few_f ? (nf + gf - 1) / gf : (nf + 31) / 32;
   const int ul = few_l ? (nl + gl - 1) / gl : (nl + 31) / 32;
-  for (int u = (warp + rot) % nw; u < uf + ul; u += nw) {
-    if (u < uf) {
+  // Euler: the listed interfaces' derivative fluxes, a component per lane
+  const int ud = T::EUL ? (nf * M + 31) / 32 : 0;
+  for (int u = (warp + rot) % nw; u < uf + ul + ud; u += nw) {
+    if (u >= uf + ul) {
+      const int i = (u - uf - ul) * 32 + lane;
+      if (i < nf * M) {
+        const int j = list_f[i / M];
+        r.D(i % M, j) = derivative_flux_fp64(r, i % M, at(j, false), S, alpha, dx);
+      }
+    } else if (u < uf) {
       if (few_f) {
         const int i = u * gf + lane / G::kInterface;
         const bool live = i < nf;
@@ -885,9 +941,13 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
       }
     }
   } else if (has_f) {
-    const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
-#pragma unroll
-    for (int c = 0; c < M; ++c) r.D(c, j) = derivative_flux_fp64(r, c, kf, S, kU, kh, kv);
+#pragma unroll 1  // (code to fetch)
+    for (int c = 0; c < M; ++c) {
+      Q2 x[5];
+      sides_differences(in, c, kf, S, x);
+      r.D(c, j) = derivative_flux(in, x, c, kf, S, alpha, dx);
+    }
+    if (!fine_grid(in, kf, S)) r.C(0, j) = linear_part_fp64(r, kf, S, alpha, dx);
   }
   __syncthreads();
   if (role == 0 && has_f) {
@@ -902,7 +962,7 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
         e[1] += row(5 * M + c).h;
       }
     }
-    interface_value<DIR>(in, ch, kf, alpha, f, lin, cc);
+    interface_value<DIR>(in, ch, kf, S, alpha, f, lin, r.C(0, j), cc);
     if (!interface_weak(r, kf, S, e[0] + e[1], alpha, sp))
       ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
 #pragma unroll

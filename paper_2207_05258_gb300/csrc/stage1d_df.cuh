@@ -217,14 +217,13 @@ __device__ __forceinline__ void stage_tile_df(const Args1D& a, const StageIO& io
   // and the limited derivatives of points j = 0..np-1 (loaded index j + 2)
   const bool limited = a.sp.limiter != 0;
   for (int j = threadIdx.x; j <= np; j += nt) {
-    double x[M];
-    if (!interface_line<D2, 0>(r, j + 1, 1, alpha, dx, a.sp, x))
+    double x[M], d[M];
+    if (!interface_line<D2, 0>(r, j + 1, 1, alpha, dx, a.sp, x, d))
       s_f[atomicAdd(&s_nf, 1)] = (unsigned short)j;
-    const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
 #pragma unroll
     for (int c = 0; c < M; ++c) {
       r.C(c, j) = x[c];
-      r.D(c, j) = derivative_flux_fp64(r, c, j + 1, 1, kU, kh, kv);
+      r.D(c, j) = d[c];
     }
     if (j < np && limited) {
       if (!limiter_line<D2, 0>(r, j + 2, 1, dx, idx, a.sp, x))

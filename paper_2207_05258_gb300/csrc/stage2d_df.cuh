@@ -71,13 +71,13 @@ __device__ __forceinline__ void items_2d(const Tile2D<EQ, DIR>& r, int j, bool h
   constexpr int M = Dim2<EQ>::M;
   double x[M];
   if (has_f) {
-    if (!interface_line<D2, DIR>(r, kf, S, alpha, dx, sp, x))
+    double d[M];
+    if (!interface_line<D2, DIR>(r, kf, S, alpha, dx, sp, x, d))
       ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
-    const double kU = 0.125 * alpha, kh = dx * (1.0 / 24.0), kv = alpha * kh;
 #pragma unroll
     for (int c = 0; c < M; ++c) {
       r.C(c, j) = x[c];
-      r.D(c, j) = derivative_flux_fp64(r, c, kf, S, kU, kh, kv);
+      r.D(c, j) = d[c];
     }
   }
   if (has_l && sp.limiter != 0) {

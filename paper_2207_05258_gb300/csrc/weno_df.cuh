@@ -333,6 +333,13 @@ __device__ __forceinline__ X linear_part(X y1, X y2, X d) {
   return add(mul(y1, 11.f), add(mul(y2, 19.f), mul(d, 3.f)));
 }
 
+// 4 times one side's dx p_0' (Sec. 2.1, the derivative flux), one component;
+// the "-" side's with its reversed and negated rows is minus its share.
+template <class X>
+__device__ __forceinline__ X derivative_part(X y1, X y2, X s, X d, X H0) {
+  return add(scale(H0, 4.f), add(add(y1, d), madd(Num<X>::c(-2.0 / 3.0), s, mul(y2, -7.f))));
+}
+
 // Maximum over the warp of non-negative doubles (their bits order as
 // unsigned integers), by integer reductions: a double maximum costs FP64
 // compares. The result is valid in every lane.

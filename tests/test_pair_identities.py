@@ -99,3 +99,38 @@ def test_derivative_flux():
             + dx / 24 * (h[0] + h[3] - 7 * (h[1] + h[2]))
             + al * dx / 24 * (v[0] - v[3] + 3 * (v[1] - v[2])))
     assert expand(both - form) == 0
+
+
+def test_derivative_flux():
+    """One side's dx p_0' from its differences, and the sum over both sides
+    with the "-" side's rows reversed and negated, against the form in F, U, h,
+    N that the FP64 path evaluates."""
+    dx, al = symbols("dx alpha")
+    F, U, h, N = (symbols(f"{q}m {q}k {q}p {q}q") for q in "FUhN")
+    t0, t1 = F[2] - F[1], F[3] - F[0]
+    su = (U[3] - U[2]) - (U[1] - U[0])
+    sh = (h[0] + h[3]) - 7 * (h[1] + h[2])
+    sv = 3 * (N[1] - N[2]) + N[0] - N[3]
+    ref = (R(15, 8) * t0 - t1 / 8 + al / 8 * su + dx / 24 * (sh + al * sv))
+
+    def side(sg, linear=False):  # rows of the "+" side, of the "-" side negated and reversed
+        order = [0, 1, 2] if sg > 0 else [3, 2, 1]
+        f = [(F[i] + sg * al * U[i]) / 2 for i in order]
+        H = [sg * dx * (h[i] + sg * al * N[i]) / 2 for i in order]
+        y1, y2 = f[1] - f[0], f[2] - f[1]  # edge rows (reversal and negation cancel)
+        y1, y2 = H[1] - y1, H[1] - y2
+        s, d = H[0] + H[2] - 2 * H[1], H[0] - H[2]
+        if linear:
+            return 11 * y1 + 19 * y2 + 3 * d
+        return H[1] + (y1 + d - 7 * y2) / 4 - s / 6
+
+    assert expand(side(1) - side(-1) - ref) == 0
+
+    # the linear part of c: in FP64, and from the sides' differences
+    lin = (11 * ((F[3] - F[2]) - (F[1] - F[0]))
+           + al * (dx * (27 * (N[1] + N[2]) + 3 * (N[0] + N[3]))
+                   - 27 * (U[2] - U[1]) - 11 * (U[3] - U[0]))
+           + dx * (33 * (h[1] - h[2]) + 3 * (h[0] - h[3]))) / 120
+    assert expand((side(1, True) + side(-1, True)) / 60 - lin) == 0
+    with open(SRC) as fh:
+        assert constants("derivative_part") == [R(-2, 3)] and "madd(Num<X>::c" in fh.read()
