@@ -55,7 +55,7 @@ __device__ __forceinline__ void euler_fh(const T* u, const T* v, double gm1, T* 
 // through euler_fh.
 __device__ __forceinline__ void point_vjp(const double* u, const double* v, const double* gF,
                                           const double* gH, double gm1, double* gu, double* gv) {
-  const double ir = 1.0 / u[0], vel = u[1] * ir;
+  const double ir = recip_fp64(u[0]), vel = u[1] * ir;
   const double p = gm1 * (u[2] - 0.5 * u[1] * vel), Ep = u[2] + p;
   const double dvel = (v[1] - vel * v[0]) * ir;
   const double dp = gm1 * (v[2] - vel * v[1] + 0.5 * vel * vel * v[0]);
@@ -89,7 +89,7 @@ __device__ __forceinline__ void point_vjp(const double* u, const double* v, cons
 // pullback (gu, gH) of sum gL.L + gR.R.
 __device__ __forceinline__ void eigen_at(double u, double H, double gm1, Eigen<double, 3>& e) {
   const double c2 = gm1 * (H - 0.5 * u * u);
-  const double c = ::sqrt(c2), ic = 1.0 / c;
+  const double ic = rsqrt_fp64(c2), c = c2 * ic;
   euler_eigen<double, 3>(0, u, 0.0, H, c, ic, gm1, e);
 }
 
@@ -98,7 +98,7 @@ __device__ __forceinline__ void eigen_at(double u, double H, double gm1, Eigen<d
 __device__ __forceinline__ void eigen_vjp(double u, double H, double gm1, const double (*gL)[3],
                                           const double (*gR)[3], double& gu, double& gH) {
   const double q = 0.5 * u * u;
-  const double c = ::sqrt(gm1 * (H - q)), ic = 1.0 / c;
+  const double c2 = gm1 * (H - q), ic = rsqrt_fp64(c2), c = c2 * ic;
   const double b1 = gm1 * ic * ic;
   const double sL1 = gL[0][1] + gL[2][1];
   const double a_b2 = 0.5 * (gL[0][0] + gL[2][0]) - gL[1][0];
@@ -126,14 +126,14 @@ __device__ __forceinline__ void eigen_vjp(double u, double H, double gm1, const 
 // Velocity and total enthalpy of a conserved state, H = gamma E / rho -
 // (gamma - 1) vel^2 / 2, and the pullback of (gvel, gH) onto (rho, m, E).
 __device__ __forceinline__ void vel_enthalpy(const double* u, double gm1, double& vel, double& H) {
-  const double ir = 1.0 / u[0];
+  const double ir = recip_fp64(u[0]);
   vel = u[1] * ir;
   H = (gm1 + 1.0) * u[2] * ir - 0.5 * gm1 * vel * vel;
 }
 
 __device__ __forceinline__ void vel_enthalpy_vjp(const double* u, double gm1, double gvel,
                                                  double gH, double* gu) {
-  const double ir = 1.0 / u[0], vel = u[1] * ir;
+  const double ir = recip_fp64(u[0]), vel = u[1] * ir;
   const double gv = gvel - gH * gm1 * vel;  // H depends on vel
   gu[0] += -gv * vel * ir - gH * (gm1 + 1.0) * u[2] * ir * ir;
   gu[1] += gv * ir;
@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(NT, 2) k_adjoint_euler_1d(const __grid_constan
     // characteristic nonlinear fluxes
     const double uL[3] = {su[0][jf + 1], su[1][jf + 1], su[2][jf + 1]};
     const double uR[3] = {su[0][jf + 2], su[1][jf + 2], su[2][jf + 2]};
-    const double sL = ::sqrt(uL[0]), sR = ::sqrt(uR[0]), iS = 1.0 / (sL + sR);
+    const double sL = uL[0] * rsqrt_fp64(uL[0]), sR = uR[0] * rsqrt_fp64(uR[0]);
+    const double iS = recip_fp64(sL + sR);
     double velL, HL, velR, HR;
     vel_enthalpy(uL, gm1, velL, HL);
     vel_enthalpy(uR, gm1, velR, HR);
@@ -301,8 +302,8 @@ __global__ void __launch_bounds__(NT, 2) k_adjoint_euler_1d(const __grid_constan
     double gUL[3] = {0, 0, 0}, gUR[3] = {0, 0, 0};
     const double gsL = (gub * (velL - ub) + gHb * (HL - Hb)) * iS;
     const double gsR = (gub * (velR - ub) + gHb * (HR - Hb)) * iS;
-    gUL[0] += 0.5 * gsL / sL;
-    gUR[0] += 0.5 * gsR / sR;
+    gUL[0] += 0.5 * gsL * recip_fp64(sL);
+    gUR[0] += 0.5 * gsR * recip_fp64(sR);
     vel_enthalpy_vjp(uL, gm1, gub * sL * iS, gHb * sL * iS, gUL);
     vel_enthalpy_vjp(uR, gm1, gub * sR * iS, gHb * sR * iS, gUR);
     // per slot, in place: gF, gH (through the point fluxes) and the direct

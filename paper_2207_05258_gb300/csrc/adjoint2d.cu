@@ -61,7 +61,7 @@ struct AdjLayout2D {
 // (u, v, H) of a conserved 2D Euler state, H = gamma E / rho - (gamma - 1)
 // (u^2 + v^2) / 2, and the pullback of (gu, gv, gH) onto (rho, m, n, E).
 __device__ __forceinline__ void velh2(const double* U, double gm1, double& u, double& v, double& H) {
-  const double ir = 1.0 / U[0];
+  const double ir = recip_fp64(U[0]);
   u = U[1] * ir;
   v = U[2] * ir;
   H = (gm1 + 1.0) * U[3] * ir - 0.5 * gm1 * (u * u + v * v);
@@ -69,7 +69,7 @@ __device__ __forceinline__ void velh2(const double* U, double gm1, double& u, do
 
 __device__ __forceinline__ void velh2_vjp(const double* U, double gm1, double gu, double gv,
                                           double gH, double* g) {
-  const double ir = 1.0 / U[0], u = U[1] * ir, v = U[2] * ir;
+  const double ir = recip_fp64(U[0]), u = U[1] * ir, v = U[2] * ir;
   const double gu2 = gu - gH * gm1 * u, gv2 = gv - gH * gm1 * v;
   g[0] += -(gu2 * u + gv2 * v) * ir - gH * (gm1 + 1.0) * U[3] * ir * ir;
   g[1] += gu2 * ir;
@@ -81,7 +81,7 @@ __device__ __forceinline__ void velh2_vjp(const double* U, double gm1, double gu
 template <int DIR>
 __device__ __forceinline__ void eigen2(double u, double v, double H, double gm1,
                                        Eigen<double, 4>& e) {
-  const double c = ::sqrt(gm1 * (H - 0.5 * (u * u + v * v))), ic = 1.0 / c;
+  const double c2 = gm1 * (H - 0.5 * (u * u + v * v)), ic = rsqrt_fp64(c2), c = c2 * ic;
   euler_eigen<double, 4>(DIR, u, v, H, c, ic, gm1, e);
 }
 
@@ -97,7 +97,7 @@ __device__ __forceinline__ void eigen2_vjp(double u, double v, double H, double 
   auto gR = [&](int r, int k) { return gLR[(16 + r * 4 + k) * NH]; };
   const double un = DIR == 0 ? u : v, ut = DIR == 0 ? v : u;
   const double q = 0.5 * (u * u + v * v);
-  const double c = ::sqrt(gm1 * (H - q)), ic = 1.0 / c;
+  const double c2 = gm1 * (H - q), ic = rsqrt_fp64(c2), c = c2 * ic;
   const double b1 = gm1 * ic * ic;
   // cotangents of the intermediate scalars, read off the entries
   const double sLn = gL(0, kn) + gL(3, kn), sLt = gL(0, kt) + gL(3, kt);
@@ -138,7 +138,7 @@ __device__ __forceinline__ void point2_vjp_u(const double* U, const double* N, c
     gu[0] += gF[0] * U[0] + gH[0] * N[0] + gE[0] * T[0];
   } else {
     constexpr int a = DIR == 0 ? 1 : 2;  // momentum along DIR
-    const double ir = 1.0 / U[0], u = U[1] * ir, v = U[2] * ir;
+    const double ir = recip_fp64(U[0]), u = U[1] * ir, v = U[2] * ir;
     const double p = gm1 * (U[3] - 0.5 * (U[1] * u + U[2] * v)), Ep = U[3] + p;
     const double un = DIR == 0 ? u : v;
     double aU[4] = {0.0, 0.0, 0.0, 0.0};
@@ -194,7 +194,7 @@ __device__ __forceinline__ void jac2_t(const double* U, const double* g, double 
     out[0] += U[0] * g[0];
   } else {
     constexpr int a = DIR == 0 ? 1 : 2;
-    const double ir = 1.0 / U[0], u = U[1] * ir, v = U[2] * ir;
+    const double ir = recip_fp64(U[0]), u = U[1] * ir, v = U[2] * ir;
     const double p = gm1 * (U[3] - 0.5 * (U[1] * u + U[2] * v)), Ep = U[3] + p;
     const double un = DIR == 0 ? u : v;
     const double adu = g[1] * U[a] + (DIR == 0 ? g[3] * Ep : 0.0);
@@ -389,8 +389,8 @@ __global__ void __launch_bounds__(NT, 256 / NT) k_adjoint_sweep_2d(const __grid_
         acc(kk + sd, fH + c, sd ? gm[3 + kk] : gp[3 + kk]);
       }
       // central flux (Eq. mixed): -1/12, 7/12, 7/12, -1/12
-      acc(2 * sd, 4 * M + c, (sd ? 7.0 : -1.0) * mc / 12.0);
-      acc(2 * sd + 1, 4 * M + c, (sd ? -1.0 : 7.0) * mc / 12.0);
+      acc(2 * sd, 4 * M + c, (sd ? 7.0 / 12.0 : -1.0 / 12.0) * mc);
+      acc(2 * sd + 1, 4 * M + c, (sd ? -1.0 / 12.0 : 7.0 / 12.0) * mc);
     }
     const double (*SF)[NL] = sd ? sFm : sFp;
     const double (*SH)[NL] = sd ? sHm : sHp;
@@ -409,7 +409,8 @@ __global__ void __launch_bounds__(NT, 256 / NT) k_adjoint_sweep_2d(const __grid_
       for (int c = 0; c < 4; ++c) { UL[c] = su[c][jf + 1]; UR[c] = su[c][jf + 2]; }
       velh2(UL, gm1, uL, vL, HL);
       velh2(UR, gm1, uR, vR, HR);
-      sL = ::sqrt(UL[0]); sR = ::sqrt(UR[0]); iS = 1.0 / (sL + sR);
+      sL = UL[0] * rsqrt_fp64(UL[0]); sR = UR[0] * rsqrt_fp64(UR[0]);
+      iS = recip_fp64(sL + sR);
       ub = (sL * uL + sR * uR) * iS; vb = (sL * vL + sR * vR) * iS;
       Hb = (sL * HL + sR * HR) * iS;
       Eigen<double, 4> e;
@@ -471,8 +472,8 @@ __global__ void __launch_bounds__(NT, 256 / NT) k_adjoint_sweep_2d(const __grid_
       // Roe average -> the two states (slots 1 and 2, direct u cotangents)
       const double gsL = (g3[0] * (uL - ub) + g3[1] * (vL - vb) + g3[2] * (HL - Hb)) * iS;
       const double gsR = (g3[0] * (uR - ub) + g3[1] * (vR - vb) + g3[2] * (HR - Hb)) * iS;
-      gUL[0] = 0.5 * gsL / sL;
-      gUR[0] = 0.5 * gsR / sR;
+      gUL[0] = 0.5 * gsL * recip_fp64(sL);
+      gUR[0] = 0.5 * gsR * recip_fp64(sR);
       velh2_vjp(UL, gm1, g3[0] * sL * iS, g3[1] * sL * iS, g3[2] * sL * iS, gUL);
       velh2_vjp(UR, gm1, g3[0] * sR * iS, g3[1] * sR * iS, g3[2] * sR * iS, gUR);
     }

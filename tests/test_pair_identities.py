@@ -134,3 +134,34 @@ def test_derivative_flux():
     assert expand((side(1, True) + side(-1, True)) / 60 - lin) == 0
     with open(SRC) as fh:
         assert constants("derivative_part") == [R(-2, 3)] and "madd(Num<X>::c" in fh.read()
+
+
+def test_weights_over_common_denominator():
+    """The reverse mode's form: v = sum of phi_l p_l is the paper's combination,
+    and the cotangents of the b_l are its derivatives (b_0 above the others, so
+    that tau = (b_0 - (b_1 + b_2) / 2)^2; exact at rational points)."""
+    b0, b1, b2, p0, p1, p2 = symbols("b0 b1 b2 p0 p1 p2")
+    g1, g2 = R(1, 7), R(2, 5)
+    g0 = 1 - g1 - g2
+    e1, e2 = b0 - b1, b0 - b2
+    ht = (e1 + e2) / 2
+    tau = ht ** 2
+    o = [g * (1 + tau / b) for g, b in ((g0, b0), (g1, b1), (g2, b2))]
+    paper = (o[0] * (p0 - g1 * p1 - g2 * p2) / g0 + o[1] * p1 + o[2] * p2) / sum(o)
+    q1, q2 = g1 * b2, g2 * b1
+    n1, n2, b12, bt = q1 * e1, q2 * e2, b1 * b2, b0 + tau
+    m = 1 / (b12 * (b0 + g0 * tau) + tau * b0 * (q1 + q2))
+    f0, f1, f2 = b12 * bt * m, tau * m * n1, tau * m * n2
+    P1, P2, P = p1 - p0, p2 - p0, p1 - p2
+    r0, r1, r2 = -(f1 * P1 + f2 * P2), f0 * P1 + f2 * P, f0 * P2 - f1 * P
+    gt = ht * m * (r0 * b12 + r1 * n1 + r2 * n2)
+    k = m * r0 * bt - m * tau * (g1 * r1 + g2 * r2)
+    grads = {b0: m * r0 * b12 + m * tau * (r1 * q1 + r2 * q2) + 2 * gt,
+             b1: b2 * k + g2 * m * tau * b0 * r2 - gt,
+             b2: b1 * k + g1 * m * tau * b0 * r1 - gt}
+    for vals in ((9, 2, 3, 1, 4, -2), (5, 4, 1, -3, R(1, 2), 7)):
+        at = dict(zip((b0, b1, b2, p0, p1, p2), vals))
+        assert (paper - (f0 * p0 + f1 * p1 + f2 * p2)).subs(at) == 0
+        assert (f0 + f1 + f2).subs(at) == 1
+        for b, g in grads.items():
+            assert (paper.diff(b) - g).subs(at) == 0
