@@ -141,7 +141,6 @@ __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, 
 __device__ __forceinline__ double madd(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ double square(double a) { return __dmul_rn(a, a); }
 __device__ __forceinline__ double scale(double a, double p2) { return __dmul_rn(a, p2); }
-__device__ __forceinline__ double abs2(double a) { return fabs(a); }
 
 // c ? -a : a
 __device__ __forceinline__ D2 flip(bool c, D2 a) { return c ? neg(a) : a; }

@@ -29,6 +29,24 @@ constexpr double FZ2 = 4405.0 / 112.0, FL = 1421461.0 / 1321500.0, FY = 13.0 / 3
 constexpr double L1 = -120.0 / 3169.0, L2 = 527690.0 / 262907.0;
 constexpr double LZ1 = 3169.0 / 1280.0, LU = 781.0 / 3169.0;
 constexpr double LZ2 = 262907.0 / 6720.0, LL = 1421461.0 / 1314535.0;
+// beta_0 of the reconstruction as H_i^2 + E2^2 + E3^2 + A4^2 + K11 a5^2, E2 =
+// E2d d + E2l lap, E3 = E3s s + E3d g, A4 = A4d d + A4l lap, a5 = s/4 + 3/4 g
+// (square roots times the exact coefficients, to 20 digits; E3h: E3's
+// coefficient of H_i over s + 2 H_i and g - 2 H_i). The factorised
+// coefficients above are those of the same quadratic form.
+constexpr double K11 = 21520059541.0 / 1377684.0;
+constexpr double E2d = 0.52842290755678754049, E2l = 2.0976788148466414486;
+constexpr double E3s = -1.6032089149031235916, E3h = -12.661835579599691806,
+                 E3d = -7.9341267047029694945;
+constexpr double A4d = -6.2490900436484649542, A4l = -12.498180087296929908;
+constexpr bool same(double x, double y) { return x - y < 1e-10 && y - x < 1e-10; }
+static_assert(same(2.0 * E3s + E3h, 2.0 * E3d), "E3 is free of H_i");
+static_assert(same(FZ1, E3s * E3s + K11 / 16.0), "s s");
+static_assert(same(FZ1 * F1, E3s * E3d + K11 * 3.0 / 16.0), "s g");
+static_assert(same(FZ1 * F1 * F1 + FG, E3d * E3d + K11 * 9.0 / 16.0), "g g");
+static_assert(same(FZ2, E2d * E2d + A4d * A4d), "d d");
+static_assert(same(FZ2 * F2, E2d * E2l + A4d * A4l), "d lap");
+static_assert(same(FZ2 * F2 * F2 + FL, E2l * E2l + A4l * A4l), "lap lap");
 }  // namespace adj
 
 // Source of point p of an instance with n points (maybe a ghost): kind 0

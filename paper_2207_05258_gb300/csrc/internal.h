@@ -217,8 +217,8 @@ struct Args1D {
 // this)); chosen by measurement: the all-FP64 kernels are FP64-pipe bound at
 // any occupancy (1..4 CTAs gave the same throughput); the 1D FP64 kernel,
 // most of whose instructions are FP32, needs warps to hide their latency (4
-// CTAs, 128 registers: 2048-instance Riemann batch 4.41 ms per step against
-// 6.88 with 2 CTAs of 184); the FP32 ones gain from more warps (1D: 8 CTAs,
+// CTAs, 128 registers: Riemann batch 7.5 ms against 8.7 with 3 CTAs of 168; 2D
+// sweeps 3.59 against 3.69); the FP32 ones gain from more warps (1D: 8 CTAs,
 // 64 registers, +12%; 2D: 5 CTAs).
 #ifndef HWENO_MINB_1D_F64
 #define HWENO_MINB_1D_F64 4
@@ -228,9 +228,6 @@ struct Args1D {
 #endif
 #ifndef HWENO_MINB_2D_F64
 #define HWENO_MINB_2D_F64 4
-#endif
-#ifndef HWENO_MINB_X_F64
-#define HWENO_MINB_X_F64 1
 #endif
 #ifndef HWENO_MINB_X_F32
 #define HWENO_MINB_X_F32 5

@@ -32,7 +32,6 @@
 template <int EQ>
 using Tile1D = LineTile<Dim1<EQ>::M, 0, EQ == HWENO_EULER>;
 
-constexpr int kMaxPPT1D = 2;  // points per thread of any tile variant
 constexpr int kMaxTile1D = 508;
 
 template <int EQ, int NT, int PPT>

@@ -239,22 +239,17 @@ __device__ __forceinline__ void tile_point(const Args1D& a, const Real* U, const
     split_pm(F[c], u[c], H[c], v[c], ha, hda, hdx, sFp[c][g], sFm[c][g], sHp[c][g], sHm[c][g]);
 }
 
-// The limited derivative v~ at loaded point g (Sec. 2.2): v unchanged with
-// the limiter off, component-wise, or (Euler) on the characteristic fields
-// of the eigenvectors at U_g.
-// Factored characteristic projections (Char1) in the tiled stage and
-// persistent kernels in FP64 and in the FP32 persistent kernel; the FP32
-// tiled kernel, capped at 64 registers, and the 124-point cluster step keep
-// the rows of L applied one by one (the factored form's larger live set
+// Factored characteristic projections (Char1) in the persistent kernel; the
+// FP32 tiled kernel, capped at 64 registers, and the 124-point cluster step
+// keep the rows of L applied one by one (the factored form's larger live set
 // spills there).
-template <class Real>
-constexpr bool kFactored = std::is_same<Real, double>::value;
 #ifndef HWENO_FAC_RUN_F32
 #define HWENO_FAC_RUN_F32 1
 #endif
-template <class Real>
-constexpr bool kFactoredRun = kFactored<Real> || HWENO_FAC_RUN_F32;
 
+// The limited derivative v~ at loaded point g (Sec. 2.2): v unchanged with
+// the limiter off, component-wise, or (Euler) on the characteristic fields
+// of the eigenvectors at U_g.
 template <int EQ, class Real, class TV, bool FAC = true>
 __device__ __forceinline__ void limited_point(const Args1D& a, int g, Real idx, Real gm1,
                                               const Weights<Real>& w, const TV& sU,
@@ -636,7 +631,7 @@ cudaError_t stage_launch_f64(int variant, int mode, const Args1D& a, int ntiles,
 template <int EQ, class Real, int MODE, int NT, int PPT>
 __global__ void __launch_bounds__(NT, (MinBlocks1D<Real, NT>::value))
 k_stage_1d(const __grid_constant__ Args1D a) {
-  stage_tile<EQ, Real, MODE, NT, PPT, kFactored<Real>>(a, io_of(a), a.tile_inst[blockIdx.x],
+  stage_tile<EQ, Real, MODE, NT, PPT>(a, io_of(a), a.tile_inst[blockIdx.x],
                                       a.tile_start[blockIdx.x]);
 }
 
@@ -779,7 +774,7 @@ k_run_1d(const __grid_constant__ Args1D a, const __grid_constant__ PersistArgs p
     if constexpr (std::is_same<Real, double>::value)
       stage_tile_df<EQ>(a, io, MODE_STAGE1 + stage, p.tile, k, s);
     else
-      stage_any<EQ, Real, NT, PPT, kFactoredRun<Real>>(a, io, MODE_STAGE1 + stage, k, s);
+      stage_any<EQ, Real, NT, PPT, HWENO_FAC_RUN_F32>(a, io, MODE_STAGE1 + stage, k, s);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
@@ -1557,9 +1552,12 @@ cudaError_t step_cluster_try(const Args1D& a, const FusedArgs& f, int C, cudaStr
   constexpr size_t tile =
       SPLIT ? SplitLayout<EQ, Real>::bytes : Layout1D<EQ, Real, kThreads1D, 1>::bytes;
   constexpr size_t bytes = tile > kClusterSmem ? tile : kClusterSmem;
-  auto kern = SPLIT ? k_step_cluster_split_1d<EQ, Real> : k_step_cluster_1d<EQ, Real>;
   static ClusterState st;
-  return cluster_launch(kern, st, C, f.batch, kThreads1D, bytes, s, a, f);
+  if constexpr (SPLIT)
+    return cluster_launch(k_step_cluster_split_1d<EQ, Real>, st, C, f.batch, kThreads1D, bytes, s, a,
+                          f);
+  else
+    return cluster_launch(k_step_cluster_1d<EQ, Real>, st, C, f.batch, kThreads1D, bytes, s, a, f);
 }
 
 template <int EQ, int P>
@@ -1585,7 +1583,7 @@ template <int EQ, class Real>
 cudaError_t step_cluster_launch(const Args1D& a, const FusedArgs& f, int max_n, cudaStream_t s) {
   if constexpr (std::is_same<Real, double>::value) {
     cudaError_t e = cudaErrorNotSupported;
-    if (EQ == HWENO_EULER) {
+    if constexpr (EQ == HWENO_EULER) {
       const int Cs = (max_n + kSplitTile - 1) / kSplitTile;
       if (Cs <= kSplitMax) e = step_cluster_try<EQ, Real, true>(a, f, Cs, s);
     } else {
@@ -1595,13 +1593,13 @@ cudaError_t step_cluster_launch(const Args1D& a, const FusedArgs& f, int max_n, 
     if (e == cudaErrorNotSupported) e = step_cluster_f64_try<EQ, kTile1D>(a, f, max_n, s);
     return e;
   } else {
-  const int Cs = (max_n + kSplitTile - 1) / kSplitTile;
-  if (Cs <= kSplitMax) {
-    const cudaError_t e = step_cluster_try<EQ, Real, true>(a, f, Cs, s);
-    if (e != cudaErrorNotSupported) return e;
-  }
-  const int C = (max_n + kTile1D - 1) / kTile1D;
-  return step_cluster_try<EQ, Real, false>(a, f, C, s);
+    const int Cs = (max_n + kSplitTile - 1) / kSplitTile;
+    if (Cs <= kSplitMax) {
+      const cudaError_t e = step_cluster_try<EQ, Real, true>(a, f, Cs, s);
+      if (e != cudaErrorNotSupported) return e;
+    }
+    const int C = (max_n + kTile1D - 1) / kTile1D;
+    return step_cluster_try<EQ, Real, false>(a, f, C, s);
   }
 }
 
