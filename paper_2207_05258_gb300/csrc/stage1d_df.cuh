@@ -4,26 +4,27 @@
 // What bounds it: the FP64 pipe takes one warp instruction per 65 to 77
 // cycles and sub-partition, and an all-FP64 stage needs about 830 per point
 // (Euler; it ran the pipe at 86%). Here FP64 keeps what the result's last
-// bits depend on (fluxes, the differences of F and U, the linear derivative
-// flux, the linear limited derivative, the Runge-Kutta update), about 150
-// per point; the corrections relative to it are taken in pairs of FP32
-// numbers (weno_df.cuh), about 7 300 FP32 instructions per point, which issue
-// next to the FP64 pipe. Interfaces and points whose correction is not small
+// bits depend on (fluxes, the differences of F and U, the linear limited
+// derivative, the Runge-Kutta update; scalar equations: the derivative flux),
+// about 130 per point; the rest is taken in pairs of FP32 numbers
+// (weno_df.cuh), about 7 000 other instructions per point, which issue next to
+// the FP64 pipe. Interfaces and points whose correction is not small
 // (a percent or so in flows with shocks) go on a list and are evaluated in
-// FP64. Measured, 2048 Riemann problems (2.5 M points): 12.8 -> 4.0 ms per step
-// (FP64 pipe 55% busy, issue slots 49%); Buckley-Leverett, 246 k points:
-// 0.40 -> 0.14 ms. Error against 128-bit arithmetic relative to the all-FP64
-// form (2-norms; Riemann problems, density waves, blast waves, N = 60..800):
-// U 0.6-1.2, V 0.2-0.8, L^1 0.1-0.4, L^2 0.04-0.8, v~ 0.02-1. The loops over
-// sides and fields stay rolled: unrolled, the straight code outruns the
-// instruction caches (6.9 ms per step).
+// FP64. Measured, 2048 Riemann problems (2.5 M points): 12.8 -> 3.37 ms per
+// step (FP64 pipe 48% busy, issue slots 40%; stalls per issue: no instruction
+// 3.3, fixed latency 1.7, shared memory 1.1); Buckley-Leverett, 246 k points:
+// 0.40 -> 0.14 ms (FP64 pipe 74%). Error against 128-bit arithmetic relative to
+// the all-FP64 form (2-norms; Riemann problems, density waves, blast waves,
+// N = 60..800): U 0.6-1.0, V 0.3-0.95, L^1 0.1-0.4, L^2 0.04-0.8, v~ 0.02-1.
+// The loops over fields stay rolled: unrolled, the straight code outruns the
+// instruction caches (6.9 ms per step when the sides were unrolled too).
 //
 // Phases, with a barrier after each:
 //   1 points      load with ghosts; F, h = f'(u) v in FP64; H^{+-} = dx h^{+-},
 //                 dx v and the eigen-system's inputs as pairs
 //   2 edges       differences of F and U (FP64, then pairs)
 //   3 interfaces  c = f-hat - (F_i + F_{i+1})/2 and the limited derivative
-//     and points  from pairs; the derivative flux in FP64
+//     and points  from pairs; the derivative flux
 //   3b            the list, in FP64
 //   4 points      flux differences, update, wave speed
 // The tile shape (threads, points per thread) and the stage are run-time
