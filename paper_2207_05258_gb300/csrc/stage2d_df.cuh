@@ -13,18 +13,31 @@
 // arithmetic relative to the all-FP64 sweeps (2-norms): U 0.8-0.95, V, W
 // 0.66-1.0, L^1 0.1-0.5, L^2, L^3 0.45-0.55, v~, w~ 0.01-0.6.
 //
-// Tiles: the x-sweep takes row segments of 124 points. The y-sweep takes
-// blocks of 4 columns x 31 rows: 35 rows loaded for 31 (16 columns x 7 rows
+// Tiles (128 threads; Shape2D for large grids): the x-sweep takes row segments
+// of 124 points. The y-sweep takes blocks of 4 columns x 31 rows: 35 rows loaded for 31 (16 columns x 7 rows
 // load 11 for 7, and the point phase is FP64 work), while the 4 columns are
 // one 32-byte sector of a row. Both give 128 interfaces, one per thread, and
 // 51 to 55 KB of shared memory, four CTAs per SM.
 
-constexpr int kColsF64 = 4, kRowsF64 = kThreads2D / kColsF64 - 1;
+// Large grids take CTAs of 256 threads (252 points; 8 columns x 31 rows), two
+// per SM: the warps of a sub-partition that belong to one CTA run the same
+// code at about the same time and share its fetch (double Mach 1920 x 480
+// 3.43 -> 3.12 ms per step; 256^2, with fewer than four waves of them, 0.335
+// -> 0.346).
+constexpr int kThreadsF64 = 256;
+template <int NT>
+struct Shape2D {  // NT: 128, 256, or kWideThreads2D (tiles of 128)
+  static constexpr bool WIDE = NT > kThreadsF64;
+  static constexpr int T = NT == kThreadsF64 ? NT : kThreads2D;  // threads of a tile
+  static constexpr int TX = T - 4;                               // x-sweep points
+  static constexpr int C = T / 32, R = 31;                       // y-sweep columns, rows
+  static constexpr int min_ctas = WIDE ? 1 : HWENO_MINB_2D_F64 * kThreads2D / T;
+};
 
 template <int EQ, int DIR>
 using Tile2D = LineTile<Dim2<EQ>::M, DIR, EQ == HWENO_EULER, Dim2<EQ>::M, true>;
 
-using Lists2D = ItemLists<kThreads2D>;
+using Lists2D = ItemLists<kThreadsF64>;
 
 // Phase 1, loaded point k: state u, the derivatives v along and w across the
 // line; stores the flux, the two Jacobian-vector products and the pairs.
@@ -101,10 +114,12 @@ __device__ __forceinline__ void differences_2d(const Tile2D<EQ, DIR>& r, int c, 
             sub(r.extra(c, k - 2 * S), r.extra(c, k + 2 * S)));
 }
 
-template <int EQ, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? kWideThreads2D : kThreads2D, WIDE ? 1 : HWENO_MINB_2D_F64)
+template <int EQ, int NT>
+__global__ void __launch_bounds__(NT, Shape2D<NT>::min_ctas)
 k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
-  constexpr int M = Dim2<EQ>::M, NT = WIDE ? kWideThreads2D : kThreads2D;
+  constexpr int M = Dim2<EQ>::M, T = Shape2D<NT>::T;
+  constexpr int TX = Shape2D<NT>::TX;
+  constexpr bool WIDE = Shape2D<NT>::WIDE;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Lists2D ls;
   if (a.skip_done && !(a.t[0] < a.t_end)) return;
@@ -115,13 +130,13 @@ k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
   int tile = blockIdx.x, row_ = blockIdx.y;
   {
     const int T = gridDim.x, F = T - 1;
-    if (F > 0 && nx % kTileX2D != 0) {
+    if (F > 0 && nx % TX != 0) {
       const long long b = (long long)blockIdx.y * T + blockIdx.x, full = (long long)a.ny * F;
       if (b < full) { tile = (int)(b % F); row_ = (int)(b / F); }
       else { tile = F; row_ = (int)(b - full); }
     }
   }
-  const int i0 = tile * kTileX2D, np = min(kTileX2D, nx - i0);
+  const int i0 = tile * TX, np = min(TX, nx - i0);
   HWENO_CHECK(np >= 1 && row_ >= 0 && row_ < a.ny, a.status);
   const long long row = (long long)row_ * nx;
   const double dx = a.geod[0], idx = a.geod[1], idx2 = a.geod[2];
@@ -136,7 +151,7 @@ k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
     }
   }
   const D2 alp = scale_pair(alpha), hp = to_pair(dx);
-  const Tile2D<EQ, 0> r{reinterpret_cast<double*>(smem_raw), kTileX2D + 4, kTileX2D + 1, a.status,
+  const Tile2D<EQ, 0> r{reinterpret_cast<double*>(smem_raw), TX + 4, TX + 1, a.status,
                         div(D2{1.f, 0.f}, alp)};
 
   // 1: points
@@ -163,7 +178,7 @@ k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
     load_point_2d<EQ, 0, WIDE>(r, g, u, v, w, gm1, alp, hp);
   }
   __syncthreads();
-  const int role = threadIdx.x / kThreads2D, j = threadIdx.x % kThreads2D;
+  const int role = threadIdx.x / T, j = threadIdx.x % T;
   auto at = [](int i, bool lim) { return lim ? i + 2 : i + 1; };
   if constexpr (WIDE) {
     // 2: pairs of points and edges
@@ -221,11 +236,12 @@ __device__ __forceinline__ void rough_speeds2(const double* u, float gam, float&
   }
 }
 
-template <int EQ, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? kWideThreads2D : kThreads2D, WIDE ? 1 : HWENO_MINB_2D_F64)
+template <int EQ, int NT>
+__global__ void __launch_bounds__(NT, Shape2D<NT>::min_ctas)
 k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
-  constexpr int M = Dim2<EQ>::M, NT = WIDE ? kWideThreads2D : kThreads2D;
-  constexpr int C = kColsF64, R = kRowsF64, L = (R + 4) * C;
+  constexpr int M = Dim2<EQ>::M, T = Shape2D<NT>::T;
+  constexpr bool WIDE = Shape2D<NT>::WIDE;
+  constexpr int C = Shape2D<NT>::C, R = Shape2D<NT>::R, L = (R + 4) * C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Lists2D ls;
   __shared__ unsigned s_top[2];
@@ -280,12 +296,12 @@ k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
   __syncthreads();
   // 3: interfaces y_{j0+r-1/2}, r = 0..nrow (lower point in loaded row r + 1),
   // and the limiter of the points of row r (loaded row r + 2)
-  const int role = threadIdx.x / kThreads2D, j = threadIdx.x % kThreads2D, rr = j / C;
+  const int role = threadIdx.x / T, j = threadIdx.x % T, rr = j / C;
   const bool in = j % C < ncol, has_f = in && rr <= nrow, mine = in && rr < nrow;
   auto at = [](int i, bool lim) { return lim ? i + 2 * C : i + C; };
   if constexpr (WIDE) {
     if (role < M)
-      for (int k = j; k < L; k += kThreads2D) {
+      for (int k = j; k < L; k += T) {
         if (k % C >= ncol) continue;
         if (k / C < nrow + 4) point_pair(r, role, k, r.N(role, k), r.h(role, k), alp, hp);
         if (k / C < nrow + 3) edge_pair(r, role, k, C, alp);
@@ -401,40 +417,50 @@ k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
   }
 }
 
-template <int EQ, bool WIDE>
+template <int EQ, int NT>
 cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
-  constexpr size_t bytes = Tile2D<EQ, 0>::bytes(kTileX2D + 4, kTileX2D + 1) +
-                           (WIDE ? xch_bytes<EQ, 0>(kTileX2D + 1) : 0);
+  constexpr int TX = Shape2D<NT>::TX;
+  constexpr size_t bytes = Tile2D<EQ, 0>::bytes(TX + 4, TX + 1) +
+                           (Shape2D<NT>::WIDE ? xch_bytes<EQ, 0>(TX + 1) : 0);
   static unsigned configured = 0;  // devices whose limit is raised
-  if (const cudaError_t e = ensure_smem_limit(k_xsweep_2d_f64<EQ, WIDE>, bytes, configured))
-    return e;
-  const dim3 grid((a.nx + kTileX2D - 1) / kTileX2D, a.ny);
-  k_xsweep_2d_f64<EQ, WIDE><<<grid, WIDE ? kWideThreads2D : kThreads2D, bytes, s>>>(a, mode);
+  if (const cudaError_t e = ensure_smem_limit(k_xsweep_2d_f64<EQ, NT>, bytes, configured)) return e;
+  const dim3 grid((a.nx + TX - 1) / TX, a.ny);
+  k_xsweep_2d_f64<EQ, NT><<<grid, NT, bytes, s>>>(a, mode);
   return cudaGetLastError();
 }
 
-template <int EQ, bool WIDE>
+template <int EQ, int NT>
 cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
-  constexpr int LI = (kRowsF64 + 1) * kColsF64;
-  constexpr size_t bytes = Tile2D<EQ, 1>::bytes((kRowsF64 + 4) * kColsF64, LI) +
-                           (WIDE ? xch_bytes<EQ, 1>(LI) : 0);
+  constexpr int C = Shape2D<NT>::C, R = Shape2D<NT>::R, LI = (R + 1) * C;
+  constexpr size_t bytes = Tile2D<EQ, 1>::bytes((R + 4) * C, LI) +
+                           (Shape2D<NT>::WIDE ? xch_bytes<EQ, 1>(LI) : 0);
   static unsigned configured = 0;  // devices whose limit is raised
-  if (const cudaError_t e = ensure_smem_limit(k_ysweep_2d_f64<EQ, WIDE>, bytes, configured))
-    return e;
-  const dim3 grid((a.nx + kColsF64 - 1) / kColsF64, (a.ny + kRowsF64 - 1) / kRowsF64);
-  k_ysweep_2d_f64<EQ, WIDE><<<grid, WIDE ? kWideThreads2D : kThreads2D, bytes, s>>>(a, mode);
+  if (const cudaError_t e = ensure_smem_limit(k_ysweep_2d_f64<EQ, NT>, bytes, configured)) return e;
+  const dim3 grid((a.nx + C - 1) / C, (a.ny + R - 1) / R);
+  k_ysweep_2d_f64<EQ, NT><<<grid, NT, bytes, s>>>(a, mode);
   return cudaGetLastError();
 }
 
-// The wide form of a sweep while its tiles number at most one per SM.
+// The wide form of a sweep while its tiles number at most one per SM; CTAs of
+// 256 threads from four waves (of 2 x 152) of them, unless their wider tiles
+// cover more than 5% more threads; else CTAs of 128.
+inline bool large_tiles(long long tiles, long long tiles256) {
+  return tiles256 >= 4 * 304 && 40 * tiles256 <= 21 * tiles;
+}
 template <int EQ>
 cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
-  const long long tiles = (long long)((a.nx + kTileX2D - 1) / kTileX2D) * a.ny;
-  return tiles <= 152 ? xsweep_f64<EQ, true>(mode, a, s) : xsweep_f64<EQ, false>(mode, a, s);
+  auto tiles = [&](int TX) { return (long long)((a.nx + TX - 1) / TX) * a.ny; };
+  const long long n = tiles(Shape2D<kThreads2D>::TX);
+  if (n <= 152) return xsweep_f64<EQ, kWideThreads2D>(mode, a, s);
+  return large_tiles(n, tiles(Shape2D<kThreadsF64>::TX)) ? xsweep_f64<EQ, kThreadsF64>(mode, a, s)
+                                                         : xsweep_f64<EQ, kThreads2D>(mode, a, s);
 }
 template <int EQ>
 cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
-  const long long tiles = (long long)((a.nx + kColsF64 - 1) / kColsF64) *
-                          ((a.ny + kRowsF64 - 1) / kRowsF64);
-  return tiles <= 152 ? ysweep_f64<EQ, true>(mode, a, s) : ysweep_f64<EQ, false>(mode, a, s);
+  constexpr int R = Shape2D<kThreads2D>::R;
+  auto tiles = [&](int C) { return (long long)((a.nx + C - 1) / C) * ((a.ny + R - 1) / R); };
+  const long long n = tiles(Shape2D<kThreads2D>::C);
+  if (n <= 152) return ysweep_f64<EQ, kWideThreads2D>(mode, a, s);
+  return large_tiles(n, tiles(Shape2D<kThreadsF64>::C)) ? ysweep_f64<EQ, kThreadsF64>(mode, a, s)
+                                                        : ysweep_f64<EQ, kThreads2D>(mode, a, s);
 }
