@@ -145,7 +145,8 @@ typedef struct hweno_options {
                       1 arithmetic mean */
   int tile_variant; /* 1D tile shape 0 .. HWENO_TILE_VARIANTS - 1 (see
                        hweno_autotune; results do not depend on it); ignored
-                       in 2D */
+                       in 2D. 0, the default: 128 threads, 124 points; large
+                       FP64 Euler batches 256 threads, 252 points */
   int fused_small;  /* 1D: 1 = when every instance has at most
                        HWENO_FUSED_MAX_POINTS points, hweno_step runs the whole
                        step (wave speed, three stages, time update) in one

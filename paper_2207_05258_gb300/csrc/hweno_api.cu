@@ -305,6 +305,21 @@ int use_variant(hweno_ctx* c, int v) {
   return HWENO_OK;
 }
 
+// The tile shape that stands for option value v: FP64 Euler batches of at
+// least four waves of 252-point tiles (256 threads, two CTAs per SM) take
+// those for the default 124 points, unless they cover more than 5% more
+// threads: warps of one CTA on a sub-partition share their instruction fetch
+// (Riemann batch of 1.28 M points 1.65 -> 1.52 ms per plain step). Results do not
+// depend on the shape.
+int default_tile(const hweno_ctx* c, int v) {
+  constexpr int large = 2;
+  static_assert(kVariants1D[large].threads == 256 && kVariants1D[large].ppt == 1, "252 points");
+  const long long n = c->vt_ntiles[0], n256 = c->vt_ntiles[large];
+  const bool take = v == 0 && !c->fp32 && c->eq == HWENO_EULER && n256 >= 4 * 304 &&
+                    40 * n256 <= 21 * n;
+  return take ? large : v;
+}
+
 // Size classes of a 1D batch: the distinct instance sizes when there are at
 // most HWENO_MAX_SIZE_CLASSES of them, else octaves of the size (log2
 // buckets above the smallest instance, the last bucket open-ended).
@@ -916,7 +931,7 @@ int hweno_create(hweno_ctx** out, int equation, const hweno_grid* grid, double g
   c->d_inst_tiles = c->d_vt_tiles[0];
   c->ntiles0 = c->ntiles = c->vt_ntiles[0];
   select_hx(c);
-  if (c->dim == 1 && (rc = use_variant(c, 0)) != HWENO_OK) {
+  if (c->dim == 1 && (rc = use_variant(c, default_tile(c, 0))) != HWENO_OK) {
     free_all(c);
     delete c;
     return rc;
@@ -932,7 +947,8 @@ int hweno_set_options(hweno_ctx* c, const hweno_options* o) {
   const hweno_options old = c->opt;
   c->opt = *o;
   int rc = HWENO_OK;
-  if (c->dim == 1 && o->tile_variant != c->variant) rc = use_variant(c, o->tile_variant);
+  if (c->dim == 1 && o->tile_variant != old.tile_variant)
+    rc = use_variant(c, default_tile(c, o->tile_variant));
   if (rc != HWENO_OK) c->opt = old;
   select_hx(c);
   // a graph recorded by hweno_run holds the old scheme parameters
@@ -1424,9 +1440,12 @@ int hweno_totals(hweno_ctx* c, const void* U, double* totals, void* stream) {
   if (!c) return HWENO_EINVAL;
   if (!U || !totals) return fail(c, HWENO_EINVAL, "null array");
   const double cell = c->dim == 2 ? ((c->x1 - c->x0) / c->nx[0]) * ((c->y1 - c->y0) / c->ny) : 0.0;
-  const int ntot = c->dim == 1 ? c->ntiles : c->ntiles_tot;
-  const cudaError_t e = launch_totals(c->m, c->fp32, c->dim, U, ntot, c->tile, c->d_tile_inst,
-                                      c->d_tile_start, c->d_inst_n, c->d_inst_off, c->batch,
+  // 1D: the option's tile table (not default_tile's), which sets the order of the sum
+  const int v = c->dim == 1 ? c->opt.tile_variant : 0;
+  const int ntot = c->dim == 1 ? c->vt_ntiles[v] : c->ntiles_tot;
+  const cudaError_t e = launch_totals(c->m, c->fp32, c->dim, U, ntot,
+                                      c->dim == 1 ? tile_points(v) : c->tile, c->d_vt_inst[v],
+                                      c->d_vt_start[v], c->d_inst_n, c->d_inst_off, c->batch,
                                       c->nx[0], c->ny, cell, c->dim == 1 ? c->d_inst_dx : nullptr,
                                       c->d_partial, totals, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(c, e, "totals");
