@@ -8,7 +8,7 @@
 // about 340 remain (FP64 pipe 42% and 53% busy on the double Mach grid), next
 // to about 18 500 others, whose fetch and latency take the rest of the time
 // (stalls per issue: no instruction 3.1 and 1.8, fixed latency 1.7 and 1.9).
-// Measured per step: double Mach 1920 x 480 13.2 -> 3.43 ms; 256^2 1.06 ->
+// Measured per step: double Mach 1920 x 480 13.2 -> 3.12 ms; 256^2 1.06 ->
 // 0.34 ms; Burgers rhs 321 x 203, 95 -> 50 us. Error against 128-bit
 // arithmetic relative to the all-FP64 sweeps (2-norms): U 0.8-0.95, V, W
 // 0.66-1.0, L^1 0.1-0.5, L^2, L^3 0.45-0.55, v~, w~ 0.01-0.6.
