@@ -41,24 +41,6 @@ struct Layout1D<EQ, double, NT, PPT> {
   static constexpr size_t bytes = Tile1D<EQ>::bytes(P + 4, P + 1);
 };
 
-// A value no speed of the state `u` exceeds by more than 2^-11 relative, in
-// FP32 (NaN where FP32 cannot tell: p below 2^-8 E, where the subtraction
-// costs too many bits, and anything outside the float range).
-template <int EQ>
-__device__ __forceinline__ float rough_speed(const double* u, float gam) {
-  if constexpr (EQ == HWENO_BURGERS) {
-    return fabsf(to_float(u[0]));
-  } else if constexpr (EQ == HWENO_BUCKLEY) {
-    const float x = to_float(u[0]), y = 1.f - x, D = 4.f * x * x + y * y;
-    return fabsf(8.f * x * y) / (D * D);
-  } else {
-    const float r = to_float(u[0]), m = to_float(u[1]), E = to_float(u[2]);
-    const float ir = 1.f / r, vel = m * ir, e = E - 0.5f * m * vel;
-    const float s = fabsf(vel) + sqrtf(gam * (gam - 1.f) * e * ir);
-    return e >= 0.00390625f * E ? s : __int_as_float(0x7fc00000);
-  }
-}
-
 // Phase 1, point g of the tile that starts at s (the pairs of H and dx N are
 // left to the caller: N in v, h in h).
 template <int EQ, class T>

@@ -29,6 +29,7 @@
 #include "hweno_math.cuh"
 #include "internal.h"
 #include "line_df.cuh"
+#include "rough_speed.cuh"
 
 namespace hweno {
 namespace {

@@ -221,21 +221,6 @@ k_xsweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
   }
 }
 
-// FP32 bounds of the two wave speeds as rough_speed in 1D.
-template <int EQ>
-__device__ __forceinline__ void rough_speeds2(const double* u, float gam, float& sx, float& sy) {
-  if constexpr (EQ == HWENO_BURGERS) {
-    sx = sy = fabsf(to_float(u[0]));
-  } else {
-    const float r = to_float(u[0]), m = to_float(u[1]), n = to_float(u[2]), E = to_float(u[3]);
-    const float ir = 1.f / r, e = E - 0.5f * (m * m + n * n) * ir;
-    const float c = sqrtf(gam * (gam - 1.f) * e * ir);
-    const bool ok = e >= 0.00390625f * E;
-    sx = ok ? fabsf(m * ir) + c : __int_as_float(0x7fc00000);
-    sy = ok ? fabsf(n * ir) + c : __int_as_float(0x7fc00000);
-  }
-}
-
 template <int EQ, int NT>
 __global__ void __launch_bounds__(NT, Shape2D<NT>::min_ctas)
 k_ysweep_2d_f64(const __grid_constant__ Args2D a, int mode) {
