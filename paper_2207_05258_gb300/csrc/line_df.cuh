@@ -383,17 +383,56 @@ __device__ __forceinline__ bool interface_weak(const T& r, int k, int S, float e
     level = fminf(fabsf(to_float(r.U(0, k))), fabsf(to_float(r.U(0, k + S))));
   }
   // (false for a NaN: of e, or of a level or alpha outside the pairs' range)
-  return e <= 12.f * kWeakLevel * scale_pair(alpha).h * level;
+  return e <= 12.f * (T::EUL ? kWeakLevel : kWeakScalar) * scale_pair(alpha).h * level;
 }
 
+// Leading words: the largest of component c at the edges and points that the
+// interface between k and k + S takes its differences from.
+template <class T>
+__device__ __forceinline__ float difference_top(const LineData<D2, T>& in, int c, int k, int S) {
+  auto top = [](D2 a, D2 b) { return fmaxf(fabsf(a.h), fabsf(b.h)); };
+  return fmaxf(top(in.H(0, c, k), in.H(1, c, k + S)),
+               fmaxf(top(in.X(0, c, k), in.X(1, c, k)), top(in.X(0, c, k - S), in.X(1, c, k + S))));
+}
+// The largest of a vector's components in units of the density: momenta over
+// sqrt(H), the energy over H (an enthalpy near the point).
+template <class T>
+__device__ __forceinline__ float in_density(const float* x, float H) {
+  float m = fabsf(x[T::kn]);
+  if constexpr (T::M == 4) m = fmaxf(m, fabsf(x[3 - T::kn]));
+  return fmaxf(fabsf(x[0]), fmaxf(m * rsqrtf(H), fabsf(x[T::M - 1]) * fast_rcp(H)));
+}
+
+// Whether the interface between k and k + S is to be tried in pairs; decided
+// before any of the work. Euler: its linear part and derivative flux in pairs
+// have an error of 2^-48 of the differences, below that of the FP64 form while
+// these are at most kFine of alpha U (1/16: up to 1.08 of it, 1/32: 0.6).
+// Scalar equations take the linear part in FP64 where it matters (fine_grid).
+// False for data outside the pairs' range.
+constexpr float kFine = 1.f / 20.f;
+template <class T>
+__device__ __forceinline__ bool interface_fine(const LineData<D2, T>& in, int k, int S,
+                                               double alpha) {
+  const float al = scale_pair(alpha).h;
+  if constexpr (T::EUL) {
+    const float s = fminf(in.r.E(0, k).h, in.r.E(0, k + S).h);
+    float x[T::M];
+#pragma unroll
+    for (int c = 0; c < T::M; ++c) x[c] = difference_top(in, c, k, S);
+    const float H = fminf(in.r.E(2, k).h, in.r.E(2, k + S).h);
+    // (one comparison per operand: fmaxf would drop a NaN)
+    return x[0] <= kFine * al * s * s && in_density<T>(x, H) <= kFine * al * s * s;
+  } else {
+    return true;
+  }
+}
 // The linear part in pairs has an error of 2^-48 of the differences it is made
-// of, that in FP64 one of F's rounding. 2D scalar equations take it in FP64
-// where a difference exceeds 2^-3 of F (coarse grids, sonic points: error of
-// L^1 against the plain FP64 form at 48 x 60 1.25 -> 0.46); in 1D and for
-// Euler the pairs' was the smaller error at every size.
+// of, that in FP64 one of F's rounding. The scalar equations take it in FP64
+// where a difference exceeds 2^-3 of F (coarse grids, sonic points; error of
+// L^1 over the plain FP64 form's: wave of 15 points 4.2 -> 0.4).
 template <class T>
 __device__ __forceinline__ bool fine_grid(const LineData<D2, T>& in, int k, int S) {
-  if constexpr (T::EUL || !T::SLIM) return true;
+  if constexpr (T::EUL) return true;
   const float top = fmaxf(fmaxf(fabsf(in.H(0, 0, k).h), fabsf(in.H(1, 0, k + S).h)),
                           fmaxf(fabsf(in.X(0, 0, k).h), fabsf(in.X(1, 0, k).h)));
   const float F = fmaxf(fabsf(to_float(in.r.F(0, k))), fabsf(to_float(in.r.F(0, k + S))));
@@ -521,6 +560,16 @@ __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double 
                                                const SchemeParams& sp, double* cc,
                                                double* dd = nullptr) {
   const LineData<X, T> in(r, S, alpha, dx, sp);
+  if constexpr (!std::is_same<X, double>::value) {
+    if (!interface_fine(in, k, S, alpha)) {
+#pragma unroll
+      for (int c = 0; c < T::M; ++c) {
+        cc[c] = 0.0;
+        dd[c] = T::EUL ? 0.0 : derivative_flux_fp64(r, c, k, S, alpha, dx);
+      }
+      return false;
+    }
+  }
   const LineWeights<X> w = line_weights<X>(sp, false);
   const auto ch = char_system<DIR>(in, k, true);
   X f[T::M], lin[T::M];
@@ -618,7 +667,7 @@ __device__ __forceinline__ bool limiter_weak(const T& r, int k, float e, const S
   if constexpr (T::EUL) {
     if (sp.limiter != 2) {
       const float s = r.E(0, k).h;
-      return e <= 4.f * kWeakLevel * s * s;
+      return e <= 4.f * kWeakLimiter * s * s;
     }
   }
   return e <= 0.f;
@@ -909,8 +958,10 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
   const bool lim_role = role >= R::sides && role < R::sides + R::limiter;
   const int lq = role - R::sides;
   const bool limited = sp.limiter != 0, chars = T::EUL && sp.limiter != 2;
+  // interfaces that are tried in pairs (every role finds the same)
+  const bool try_f = has_f && interface_fine(in, kf, S, alpha);
   if (role < R::sides) {
-    if (has_f) {
+    if (try_f) {
       const LineWeights<D2> w = line_weights<D2>(sp, false);
       ch = char_system<DIR>(in, kf, true);
 #pragma unroll
@@ -940,7 +991,7 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
         for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
       }
     }
-  } else if (has_f) {
+  } else if (T::EUL ? try_f : has_f) {
 #pragma unroll 1  // (code to fetch)
     for (int c = 0; c < M; ++c) {
       Q2 x[5];
@@ -950,7 +1001,8 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
     if (!fine_grid(in, kf, S)) r.C(0, j) = linear_part_fp64(r, kf, S, alpha, dx);
   }
   __syncthreads();
-  if (role == 0 && has_f) {
+  if (role == 0 && has_f && !try_f) ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
+  if (role == 0 && try_f) {
     double cc[M];
     float e[2] = {0.f, 0.f};
 #pragma unroll

@@ -13,14 +13,14 @@
 // p_0 commutes with the characteristic projection. So only C needs the
 // projection, and it depends on differences of the data alone.
 //
-// A pair carries 48 bits, so C has an error of about 2^-46 (phi_1 |p_1 - p_0|
-// + phi_2 |p_2 - p_0|). Items are evaluated in pairs while that stays below
-// the rounding of the FP64 form, which starts from the full values and has an
-// error of a few 2^-53 of alpha U: either phi_1, phi_2 <= kWeakPhi, or the sum
-// of the phi |differences| over the sides and fields that exceed it is at most
-// kWeakLevel of the local alpha U. Where neither holds (shocks, under-resolved
-// jumps, and whatever leaves the FP32 range: any overflow or NaN fails the
-// same test) the caller evaluates the item in FP64.
+// A pair carries 48 bits: C has an error of about 2^-46 (phi_1 |p_1 - p_0| +
+// phi_2 |p_2 - p_0|), and where the linear part is taken in pairs that has one
+// of 2^-48 of the differences. The FP64 form starts from the full values and
+// has an error of a few 2^-53 of alpha U. Items are evaluated in pairs while
+// their error stays below that: kWeakPhi, kWeakLevel and the like here, kFine
+// and fine_grid in line_df.cuh. Where they fail (shocks, under-resolved jumps
+// and waves, noise, and whatever leaves the FP32 range: any overflow or NaN
+// fails the same tests) the caller evaluates the item in FP64.
 #pragma once
 
 #include <type_traits>
@@ -69,10 +69,19 @@ struct LineWeights {
   float bmax;
 };
 
-// The bounds of the two tests above. (With the first alone, 1/16 would do and
-// 1/4 would not: v~ behind a contact then has 5 times the FP64 form's largest
-// error. 1/32 and 1/64 leave factors of two and more.)
-constexpr float kWeakPhi = 1.f / 32.f, kWeakLevel = 1.f / 64.f;
+// An item is weak while every phi is at most kWeakPhi or the sum of phi
+// |differences| over the sides and fields that exceed it is at most a fraction
+// of the local alpha U: kWeakLevel (Euler interfaces), kWeakScalar (interfaces
+// of the scalar equations, whose differences may be as large as their values),
+// kWeakLimiter of U (limiter on characteristic fields; on components, whose
+// FP64 form starts from differences, the first test alone). Error of L^1, L^2
+// and v~ over the FP64 form's (2-norms, waves of 5 to 800 points, noise of
+// 1e-8 to 0.3, jumps, steep profiles; tests/test_host_pairs.py): at most 1.
+// With kWeakPhi = 1/32, one level of 1/64 for all and no bound on the
+// differences it reached 26 (noise about zero), 8 (waves of 7 points) and 24
+// (v~ of a wave of 15 points).
+constexpr float kWeakPhi = 1.f / 256.f, kWeakLevel = 1.f / 64.f, kWeakScalar = 1.f / 1024.f,
+                kWeakLimiter = 1.f / 4096.f;
 
 // The smoothness indicators b_l of one side of an interface from the
 // differences of its stencil: y1 = f_{i-1} - f_i + H_i,
@@ -127,16 +136,18 @@ __device__ __forceinline__ float2 max3(float2 a, float2 b, float2 c) {
 }
 __device__ __forceinline__ float quarter(float a) { return 0.25f * a; }
 __device__ __forceinline__ float2 quarter(float2 a) { return __fmul2_rn(a, dup(0.25f)); }
-__device__ __forceinline__ void bound(float& e, float tau, float n1, float n2, float den, float p,
-                                      float q, float mx, float bmax) {
-  const float top = tau * fmaxf(fabsf(n1), fabsf(n2));
+// Adds to e a bound of phi (|p| + |q|) where phi exceeds kWeakPhi, phi taken
+// with b_0 for b_0 - b_l: what the difference's own error is a fraction of.
+__device__ __forceinline__ void bound(float& e, float tau, float q1, float q2, float b0, float den,
+                                      float p, float q, float mx, float bmax) {
+  const float top = tau * (fmaxf(q1, q2) * b0);
   if (!(top <= kWeakPhi * den)) e += top * fast_rcp(den) * (fabsf(p) + fabsf(q));
   if (!(mx < bmax)) e = __int_as_float(0x7f800000);
 }
-__device__ __forceinline__ void bound(float2& e, float2 tau, float2 n1, float2 n2, float2 den,
-                                      float2 p, float2 q, float2 mx, float bmax) {
-  bound(e.x, tau.x, n1.x, n2.x, den.x, p.x, q.x, mx.x, bmax);
-  bound(e.y, tau.y, n1.y, n2.y, den.y, p.y, q.y, mx.y, bmax);
+__device__ __forceinline__ void bound(float2& e, float2 tau, float2 q1, float2 q2, float2 b0,
+                                      float2 den, float2 p, float2 q, float2 mx, float bmax) {
+  bound(e.x, tau.x, q1.x, q2.x, b0.x, den.x, p.x, q.x, mx.x, bmax);
+  bound(e.y, tau.y, q1.y, q2.y, b0.y, den.y, p.y, q.y, mx.y, bmax);
 }
 
 // (phi_1 - phi_2) p + (phi_1 + phi_2) q from b_l in pairs; where a phi_l
@@ -158,7 +169,7 @@ __device__ __forceinline__ X correction(X b0, X b1, X b2, X p, X q, const LineWe
   const X n1 = mul(q1, e1), n2 = mul(q2, e2);
   const X den = madd(mul(b1, b2), madd(w.g0, tau, b0), mul(mul(tau, b0), add(q1, q2)));
   const X num = mul(tau, madd(p, sub(n1, n2), mul(q, add(n1, n2))));
-  bound(e, tau.h, n1.h, n2.h, den.h, p.h, q.h, mx, w.bmax);
+  bound(e, tau.h, q1.h, q2.h, b0.h, den.h, p.h, q.h, mx, w.bmax);
   return div(num, den);
 }
 
@@ -211,9 +222,11 @@ __device__ __forceinline__ double weighted(double b0, double b1, double b2, doub
   const double P12 = mul(b1, b2), P = mul(b0, P12), tb = mul(tau, b0);
   const double W0 = madd(tau, P12, P);
   const double W1 = mul(w.g1, madd(tb, b2, P)), W2 = mul(w.g2, madd(tb, b1, P));
-  const double r = madd(-w.g2, p2, madd(-w.g1, p1, p0));
-  const double num = madd(W2, p2, madd(W1, p1, mul(W0, r)));
-  return mul(num, recip_fp64(add(madd(w.g0, W0, W1), W2)));
+  // the small products first, so that one operation each rounds the full sums
+  const double r = sub(p0, madd(w.g2, p2, mul(w.g1, p1)));
+  const double num = madd(W0, r, madd(W1, p1, mul(W2, p2)));
+  const double den = madd(w.g0, W0, add(W1, W2)), id = recip_fp64(den), q = mul(num, id);
+  return madd(madd(-q, den, num), id, q);
 }
 // f-hat of a side minus the side's split flux at its own point:
 // 6 (p_1 - f_i) = y1 + 3 H_i, 6 (p_2 - f_i) = 3 H_i - y2,

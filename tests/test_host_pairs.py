@@ -1,0 +1,260 @@
+"""The FP64 stages' arithmetic in pairs of FP32 numbers, compiled for the host:
+its error against long double is no larger than that of the all-FP64 form
+(hweno_math.cuh), on resolved and under-resolved waves, noise of all sizes, jumps
+and steep profiles, for the scalar equations and Euler, 1D and 2D tiles.
+
+The errors of L^1, L^2 and v~ are taken as 2-norms over the line. Both forms' are
+sums of independent roundings, so their ratio of one line scatters, most where
+few points carry the error; the geometric mean over SEEDS lines does by about a
+tenth: bound 1.15.
+"""
+import ctypes
+
+import numpy as np
+import pytest
+
+import _host_build as H
+
+L = np.longdouble
+SEEDS, BOUND = 12, 1.15
+DX = 2.0 ** -8
+PAPER = dict(lin_w=(0.98, 0.01, 0.01), lim_d=(0.98, 0.01, 0.01), eps=1e-6, limiter=1, eig_avg=0)
+EQ = dict(burgers=(0, 1), euler=(1, 3), buckley=(2, 1), euler2d=(1, 4))
+GAMMA = 1.4
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return H.load(tmp_path_factory.mktemp("host"))
+
+
+# --- the scheme in long double (Sec. 2.1-2.2) ---------------------------------
+def q(a, b):
+    return L(a) / L(b)
+
+
+def combine(b, p, g, eps):
+    tau = ((np.abs(b[0] - b[1]) + np.abs(b[0] - b[2])) / 2) ** 2
+    w = [L(gg) * (1 + tau / (x + L(eps))) for x, gg in zip(b, g)]
+    return (w[0] * (p[0] - L(g[1]) * p[1] - L(g[2]) * p[2]) / L(g[0]) + w[1] * p[1]
+            + w[2] * p[2]) / (w[0] + w[1] + w[2])
+
+
+def side(f, h, o):
+    (fm, f0, fp), (Hm, H0, Hp) = f, h
+    sH, dH, lp, dif = Hm + Hp, Hm - Hp, fm - 2 * f0 + fp, fm - fp
+    a2, a4 = q(3, 8) * dH + q(5, 4) * lp, -dH / 4 - lp / 2
+    a3, a5 = -(q(11, 24) * sH + q(17, 6) * H0) - q(15, 8) * dif, sH / 4 + H0 + q(3, 4) * dif
+    b0 = (H0 ** 2 + q(13, 3) * (a2 + q(63, 130) * a4) ** 2
+          + q(781, 20) * (a3 + q(8825, 10934) * a5) ** 2 + q(1421461, 2275) * a4 ** 2
+          + q(21520059541, 1377684) * a5 ** 2)
+    b = [b0] + [H0 ** 2 + q(13, 3) * x ** 2 for x in (H0 - f0 + fm, H0 + f0 - fp)]
+    p = [q(11, 60) * (fm + fp) + q(19, 30) * f0 + dH / 20 + H0 / 2,
+         fm / 6 + q(5, 6) * f0 + q(2, 3) * H0, q(5, 6) * f0 + fp / 6 + H0 / 3]
+    return combine(b, p, o["lin_w"], o["eps"])
+
+
+def limiter(u, v, o):
+    (um, u0, up), (Vm, Vp) = u, v
+    q0 = q(3, 4) * (up - um) - (Vm + Vp) / 4
+    a2, a3 = (Vm - Vp) / 4 + um - 2 * u0 + up, (Vm + Vp + um - up) / 4
+    a4 = (Vp - Vm) / 4 - (um - 2 * u0 + up) / 2
+    b0 = ((q0 + a3 / 4) ** 2 + q(13, 3) * (a2 + q(63, 130) * a4) ** 2 + q(781, 20) * a3 ** 2
+          + q(1421461, 2275) * a4 ** 2)
+    q1, q2 = u0 - um, up - u0
+    return combine([b0, q1 ** 2, q2 ** 2], [q0, q1, q2], o["lim_d"], o["eps"])
+
+
+def prim(u):
+    v = [x / u[0] for x in u[1:-1]]
+    kin = sum(x * x for x in v) / 2
+    p = (L(GAMMA) - 1) * (u[-1] - u[0] * kin)
+    return v, kin, p
+
+
+def eigen(v, Hh):
+    """Left and right eigenvectors at velocities v and enthalpy Hh, as
+    functions of a vector."""
+    kin = sum(x * x for x in v) / 2
+    c = np.sqrt((L(GAMMA) - 1) * (Hh - kin))
+    b = (L(GAMMA) - 1) / c ** 2
+
+    def left(x):
+        A = (b * kin * x[0] - b * sum(a * y for a, y in zip(v, x[1:-1])) + b * x[-1]) / 2
+        B = (v[0] * x[0] - x[1]) / c / 2
+        return [A + B, x[0] - 2 * A] + [y - a * x[0] for a, y in zip(v[1:], x[2:-1])] + [A - B]
+
+    def right(s):
+        n = s[0] + s[1] + s[-1]
+        out = [n, v[0] * n + c * (s[-1] - s[0])]
+        out += [a * n + y for a, y in zip(v[1:], s[2:-1])]
+        return out + [Hh * (s[0] + s[-1]) + kin * s[1] + sum(a * y for a, y in zip(v[1:], s[2:-1]))
+                      + v[0] * c * (s[-1] - s[0])]
+    return left, right
+
+
+def reference(eq, U, V, alpha, o):
+    u, v, dx, al = [x.astype(L) for x in U], [x.astype(L) for x in V], L(DX), L(alpha)
+    at = lambda x, k: np.roll(x, -k)  # x_{i+k}
+    if eq == "burgers":
+        F, h = [u[0] ** 2 / 2], [u[0] * v[0]]
+    elif eq == "buckley":
+        D = 4 * u[0] ** 2 + (1 - u[0]) ** 2
+        F, h = [4 * u[0] ** 2 / D], [8 * u[0] * (1 - u[0]) / D ** 2 * v[0]]
+    else:
+        w, kin, p = prim(u)
+        dw = [(y - a * v[0]) / u[0] for a, y in zip(w, v[1:-1])]
+        dp = (L(GAMMA) - 1) * (v[-1] - sum(a * y for a, y in zip(w, v[1:-1])) + kin * v[0])
+        F = [u[1]] + [m * w[0] for m in u[1:-1]] + [(u[-1] + p) * w[0]]
+        h = ([v[1]] + [dm * w[0] + m * dw[0] for m, dm in zip(u[1:-1], v[1:-1])]
+             + [(v[-1] + dp) * w[0] + (u[-1] + p) * dw[0]])
+        F[1], h[1] = F[1] + p, h[1] + dp
+    fs = [[(a + s * al * b) / 2 for a, b in zip(F, u)] for s in (1, -1)]
+    hs = [[dx * (a + s * al * b) / 2 for a, b in zip(h, v)] for s in (1, -1)]
+    same = (lambda x: list(x),) * 2
+    if eq.startswith("euler"):
+        Hh = (u[-1] + p) / u[0]
+        if o["eig_avg"]:
+            mean = [(a + at(a, 1)) / 2 for a in u]
+            wm, _, pm = prim(mean)
+            face = eigen(wm, (mean[-1] + pm) / mean[0])
+        else:
+            r = np.sqrt(u[0])
+            roe = lambda a: (r * a + at(r, 1) * at(a, 1)) / (r + at(r, 1))
+            face = eigen([roe(a) for a in w], roe(Hh))
+        point = eigen(w, Hh) if o["limiter"] == 1 else same
+    else:
+        face = point = same
+
+    def project(to, x, k):
+        return to([at(a, k) for a in x])
+    cols = [[project(face[0], x, k) for k in ks] for x, ks in
+            ((fs[0], (-1, 0, 1)), (hs[0], (-1, 0, 1)), (fs[1], (2, 1, 0)), (hs[1], (2, 1, 0)))]
+    fh = face[1]([side([x[i] for x in cols[0]], [x[i] for x in cols[1]], o)
+                  + side([x[i] for x in cols[2]], [-x[i] for x in cols[3]], o)
+                  for i in range(len(u))])
+
+    def dp0(f, g):
+        return (f[0] - 8 * f[1] + 7 * f[2]) / 4 + (g[0] - 2 * g[1] - 5 * g[2]) / 12
+    hh = [dp0([at(fs[0][c], k) for k in (-1, 0, 1)], [at(hs[0][c], k) for k in (-1, 0, 1)])
+          - dp0([at(fs[1][c], k) for k in (2, 1, 0)], [-at(hs[1][c], k) for k in (2, 1, 0)])
+          for c in range(len(u))]
+    us = [project(point[0], u, k) for k in (-1, 0, 1)]
+    vs = [project(point[0], [dx * a for a in v], k) for k in (-1, 1)]
+    vt = point[1]([limiter([x[i] for x in us], [x[i] for x in vs], o) for i in range(len(u))])
+    return [np.array([-(a - at(a, -1)) / dx for a in fh]),
+            np.array([-(a - at(a, -1)) / dx ** 2 for a in hh]), np.array([a / dx for a in vt])]
+
+
+# --- data -----------------------------------------------------------------
+def conserved(rho, u, p, m, v=0.0):
+    rows = [rho, rho * u] + ([rho * v + 0 * u] if m == 4 else [])
+    return np.stack(rows + [p / (GAMMA - 1) + 0.5 * rho * (u * u + (v * v if m == 4 else 0))])
+
+
+def state(eq, kind, size, n, seed):
+    """U and V (per point): waves of `size` points each, noise of amplitude
+    `size` about a mean or about zero, in the derivative, jumps, a steep front."""
+    g = np.random.default_rng(seed)
+    x, m, ph = np.arange(n) + 0.5, EQ[eq][1], g.uniform(0, 6.28, 3)
+    noise = lambda shape=n: g.uniform(-1, 1, shape)
+    if m == 1:
+        amp = 0.4 if eq == "buckley" else 1.0
+        if kind == "wave":
+            k = 2 * np.pi / size
+            return 0.5 + amp * np.sin(k * x + ph[0]), amp * k * np.cos(k * x + ph[0])
+        if kind == "noise":
+            return 0.7 + size * noise(), size * noise()
+        if kind == "noise about zero":
+            return size * noise(), size * noise()
+        if kind == "jump":
+            return 0.5 + np.where(x < n * g.uniform(0.3, 0.7), 0.3, -0.2), 0 * x
+        k = 2 * np.pi / n
+        s = np.sin(k * x + ph[0])
+        return (0.5 + amp * np.tanh(size * s),
+                amp * size * k * np.cos(k * x + ph[0]) / np.cosh(size * s) ** 2)
+
+    def wave(x, amp, k):
+        a = [amp * np.sin(k * x + b) for b in ph]
+        return conserved(1 + a[0], 0.3 + 0.7 * a[1], 1 + 0.8 * a[2], m, 0.2 - 0.4 * a[1])
+    if kind == "noise":
+        return (conserved(1 + size * noise(), 0.3 + size * noise(), 1 + size * noise(), m,
+                          0.2 + size * noise()), size * noise((m, n)))
+    amp, k = {"wave": (0.6, 2 * np.pi / size), "weak wave": (0.2, 2 * np.pi / size)}.get(
+        kind, (0.2, 2 * np.pi / n))
+    U = wave(x, amp, k)
+    V = (wave(x + 1e-5, amp, k) - wave(x - 1e-5, amp, k)) / 2e-5
+    if kind == "derivative noise":
+        V = V + size * noise((m, n))
+    if kind == "jump":
+        U = U * np.where(x < n * g.uniform(0.3, 0.7), 1.0, g.uniform(0.3, 3.0))
+    return U, V
+
+
+def errors(lib, eq, kind, size, n, seed, opts):
+    o = dict(PAPER, **opts)
+    U, V = (np.ascontiguousarray(np.atleast_2d(a)) for a in state(eq, kind, size, n, seed))
+    V = V / DX
+    m = len(U)
+    if eq == "burgers":
+        alpha = np.abs(U).max()
+    elif eq == "buckley":
+        alpha = 2.3
+    else:
+        w, _, p = prim([a for a in U])
+        alpha = float((np.abs(w[0]) + np.sqrt(GAMMA * p / U[0])).max())
+    ref = reference(eq, U, V, alpha, o)
+    w3, d3 = np.array(o["lin_w"], float), np.array(o["lim_d"], float)
+    res, listed = [], np.zeros(2, np.int32)
+    for form in (0, 1, 2):
+        out = [np.zeros_like(U) for _ in range(3)]
+        lib.host_line(form, EQ[eq][0], m, n, ctypes.c_double(DX), ctypes.c_double(alpha), H.ptr(U),
+                      H.ptr(V), H.ptr(w3), H.ptr(d3), ctypes.c_double(o["eps"]),
+                      ctypes.c_double(GAMMA), o["limiter"], o["eig_avg"],
+                      *[H.ptr(a) for a in out], H.ptr(listed))
+        res.append([float(np.sqrt(((a - b) ** 2).sum())) for a, b in zip(out, ref)])
+    return np.array(res), listed / (2 * n)
+
+
+def ratios(lib, eq, kind, size, n, **opts):
+    logs, listed = [], 0
+    for seed in range(SEEDS):
+        e, part = errors(lib, eq, kind, size, n, seed, opts)
+        logs.append(np.log(np.maximum(e[:2], 1e-300) / e[2]))
+        listed = listed + part / SEEDS
+    return np.exp(np.mean(logs, axis=0)), listed
+
+
+SCALAR = ([("wave", s, n) for s, n in ((60, 60), (30, 60), (15, 60), (10, 60), (6.7, 60), (11, 100),
+                                       (7.7, 100), (22, 200), (15.4, 200), (400, 400))]
+          + [("noise", a, 100) for a in (1e-8, 1e-4, 1e-3, 1e-2, 0.1, 0.3)]
+          + [("noise about zero", a, 100) for a in (1e-6, 1e-4, 1e-3, 1e-2, 0.1)]
+          + [("jump", 1, 100), ("steep", 3, 100), ("steep", 10, 100)])
+EULER = ([("wave", s, n) for s, n in ((60, 60), (30, 60), (15, 60), (6.7, 60), (25, 100), (11, 100),
+                                      (22, 200), (400, 400))]
+         + [("weak wave", s, n) for s, n in ((15, 60), (6.7, 60), (11, 100), (7.7, 100))]
+         + [("noise", a, 100) for a in (1e-8, 1e-4, 1e-2, 0.03, 0.1, 0.3)]
+         + [("derivative noise", a, 100) for a in (1e-3, 1e-2, 0.03, 0.1)] + [("jump", 1, 200)])
+
+
+@pytest.mark.parametrize("eq,kind,size,n", [(e, *c) for e in ("burgers", "buckley") for c in SCALAR]
+                         + [(e, *c) for e in ("euler", "euler2d") for c in EULER])
+def test_no_larger_error_than_all_fp64(lib, eq, kind, size, n):
+    r, _ = ratios(lib, eq, kind, size, n)
+    assert r.max() <= BOUND, r
+
+
+@pytest.mark.parametrize("opts", [dict(eps=1e6), dict(eps=1e-20), dict(limiter=2),
+                                  dict(lin_w=(1 / 3, 1 / 3, 1 / 3), lim_d=(0.2, 0.4, 0.4))])
+@pytest.mark.parametrize("eq", ["burgers", "buckley", "euler", "euler2d"])
+def test_options(lib, eq, opts):
+    for kind, size in (("wave", 15), ("noise", 0.1)):
+        r, _ = ratios(lib, eq, kind, size, 100, **opts)
+        assert r.max() <= BOUND, (kind, r)
+
+
+@pytest.mark.parametrize("eq", ["burgers", "buckley", "euler", "euler2d"])
+def test_resolved_flow_stays_in_pairs(lib, eq):
+    """... and the error there is below the all-FP64 form's."""
+    r, listed = ratios(lib, eq, "wave", 400, 400)
+    assert listed.max() == 0 and r.max() < 0.95
