@@ -88,46 +88,40 @@ __device__ __forceinline__ double weighted_vjp(double b0, double b1, double b2, 
   // From 2^240 on they are scaled by the power of two of b_0 (the others
   // exceed it by at most 2%), tau, of which the weights take tau / b, by the
   // same, and the cotangents of the b_l back: finite up to indicators of about
-  // 1e280.
-  const int big = __double2hiint(b0) & 0x7ff00000;
-  const bool scaled = big >= (1023 + 240) << 20 && big != 0x7ff00000;
-  double down = 1.0;
-  if (scaled) {
-    down = __hiloint2double((2046 << 20) - big, 0);
-    b0 *= down;
-    b1 *= down;
-    b2 *= down;
-  }
+  // 1e260. By integer operations on the exponents (a branch around FP64 ones
+  // cost 2% of the 2D adjoint); with sh = 0 nothing changes.
+  const int ex = __double2hiint(b0) & 0x7ff00000;
+  const int sh = ex > (1023 + 240) << 20 && ex != 0x7ff00000 ? ex - (1023 << 20) : 0;
+  auto shift = [](double x, int by) {  // x 2^by; 0 or less where it underflows
+    return __hiloint2double(max(__double2hiint(x) + by, 0), __double2loint(x));
+  };
+  b0 = shift(b0, -sh);
+  b1 = shift(b1, -sh);
+  b2 = shift(b2, -sh);
   const double e1 = b0 - b1, e2 = b0 - b2;
-  const double ht = 0.5 * (fabs(e1) + fabs(e2));
-  double tau = ht * ht;
-  if (scaled) tau *= __hiloint2double(big, 0);
+  const double ht = 0.5 * (fabs(e1) + fabs(e2)), tau = shift(ht * ht, sh);
   const double q1 = g1 * b2, q2 = g2 * b1, n1 = q1 * e1, n2 = q2 * e2;
   const double b12 = b1 * b2, bt = b0 + tau;
   const double iD = recip_fp64(b12 * (b0 + g0 * tau) + tau * (b0 * (q1 + q2)));
   const double tD = tau * iD, f1 = tD * n1, f2 = tD * n2;
   double f0 = b12 * bt * iD;
   if (__double2hiint(f0) >= 0x3fe00000) f0 = 1.0 - (f1 + f2);  // from 1/2 on
-  double r0 = -(f1 * P1 + f2 * P2);
+  const double r0 = -(f1 * P1 + f2 * P2);
   gp0 = mu * f0;
   gp1 = mu * f1;
   gp2 = mu * f2;
   gb0 = gb1 = gb2 = 0.0;
   if (!frozen) {
     const double m = mu * iD, mt = m * tau;
-    double r1 = f0 * P1 + f2 * P, r2 = f0 * P2 - f1 * P, x = r0 * b12;
+    const double r1 = f0 * P1 + f2 * P, r2 = f0 * P2 - f1 * P, x = r0 * b12;
     const double gt = ht * m * (x + (r1 * n1 + r2 * n2));  // t / 2 times the cotangent of tau
     const double t1 = signed_by(gt, e1), t2 = signed_by(gt, e2);
-    if (scaled) {  // (not gt, where tau's power cancels it)
-      r0 *= down;
-      r1 *= down;
-      r2 *= down;
-      x *= down;
-    }
-    const double k = m * (r0 * bt) - mt * (g1 * r1 + g2 * r2), mb = mt * b0;
-    gb0 = (m * x + mt * (r1 * q1 + r2 * q2)) + (t1 + t2);
-    gb1 = (b2 * k + g2 * (mb * r2)) - t1;
-    gb2 = (b1 * k + g1 * (mb * r1)) - t2;
+    const double k = m * bt * r0 - mt * (g1 * r1 + g2 * r2), mb = mt * b0;
+    // (in gt the powers of tau and of the b_l cancel)
+    const double down = __hiloint2double((1023 << 20) - sh, 0);
+    gb0 = (m * x + mt * (r1 * q1 + r2 * q2)) * down + (t1 + t2);
+    gb1 = (b2 * k + g2 * (mb * r2)) * down - t1;
+    gb2 = (b1 * k + g1 * (mb * r1)) * down - t2;
   }
   return f0 * p0 + (f1 * p1 + f2 * p2);
 }
