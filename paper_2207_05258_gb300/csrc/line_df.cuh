@@ -179,7 +179,8 @@ struct LineData<D2, T> {
   __device__ __forceinline__ D2 dU(int c, int k) const { return r.dU(c, k); }
   __device__ __forceinline__ D2 Nx(int c, int k) const { return r.Nx(c, k); }
   __device__ __forceinline__ D2 gm1() const { return gm1_pair(sp); }
-  // velocities and enthalpy at point k, or the Roe average of k and k + S
+  // velocities and enthalpy at point k, or of the Roe average or the mean state
+  // of k and k + S
   __device__ __forceinline__ void state(int k, bool edge, D2& un, D2& ut, D2& H) const {
     if (!edge) {
       un = r.E(1, k);
@@ -188,6 +189,22 @@ struct LineData<D2, T> {
       return;
     }
     const D2 sl = r.E(0, k), sr = r.E(0, k + S);
+    if (sp.eig_avg != 0) {  // mean state (gamma E = rho H + (gamma - 1) rho q)
+      const D2 rl = square(sl), rr = square(sr), ir = div(D2{1.f, 0.f}, add(rl, rr));
+      auto mean = [&](D2 a, D2 b) { return mul(madd(rl, a, mul(rr, b)), ir); };
+      const D2 ul = r.E(1, k), ur = r.E(1, k + S);
+      D2 tl{}, tr{};
+      un = mean(ul, ur);
+      if constexpr (T::M == 4) {
+        tl = r.E(3, k);
+        tr = r.E(3, k + S);
+        ut = mean(tl, tr);
+      }
+      using C = LineChar<D2, T::M, 0>;
+      const D2 q = sub(mean(C::kinetic(ul, tl), C::kinetic(ur, tr)), C::kinetic(un, ut));
+      H = madd(gm1(), q, mean(r.E(2, k), r.E(2, k + S)));
+      return;
+    }
     const D2 is = div(D2{1.f, 0.f}, add(sl, sr));
     auto roe = [&](int e) { return mul(madd(sl, r.E(e, k), mul(sr, r.E(e, k + S))), is); };
     un = roe(1);
@@ -374,7 +391,6 @@ __device__ __forceinline__ float interface_side(const LineData<X, T>& in,
 template <class T>
 __device__ __forceinline__ bool interface_weak(const T& r, int k, int S, float e, double alpha,
                                                const SchemeParams& sp) {
-  if (T::M > 1 && sp.eig_avg != 0) return false;  // (the mean state is taken in FP64)
   float level;
   if constexpr (T::EUL) {
     const float s = fminf(r.E(0, k).h, r.E(0, k + S).h);

@@ -167,10 +167,17 @@ void line_fp64(int eq, int n, double dx, double alpha, const double* U, const do
     double z[4], f[4];
     Char2<double, 0> ch;
     if (EUL) {
+      // the Roe average, or the arithmetic mean state
       const double a = std::sqrt(P[g].u[0]), b = std::sqrt(P[g + 1].u[0]), is = 1.0 / (a + b);
       auto roe = [&](double x, double y) { return (a * x + b * y) * is; };
       ch = system(roe(P[g].un, P[g + 1].un), roe(P[g].ut, P[g + 1].ut),
                   roe(P[g].Ep * P[g].ir, P[g + 1].Ep * P[g + 1].ir));
+      if (o.eig_avg) {
+        auto mean = [&](int c) { return 0.5 * (P[g].u[c] + P[g + 1].u[c]); };
+        const double ir = 1.0 / mean(0), un = mean(1) * ir, ut = M == 4 ? mean(2 % M) * ir : 0.0;
+        const double kin = 0.5 * (mean(1) * un + (M == 4 ? mean(2 % M) * ut : 0.0));
+        ch = system(un, ut, (mean(M - 1) + gm1 * (mean(M - 1) - kin)) * ir);
+      }
     }
     for (int q = 0; q < M; ++q) {
       auto x = [&](int k, int i) { return EUL ? left(ch, q, k, i) : s[k][q][i]; };

@@ -258,3 +258,15 @@ def test_resolved_flow_stays_in_pairs(lib, eq):
     """... and the error there is below the all-FP64 form's."""
     r, listed = ratios(lib, eq, "wave", 400, 400)
     assert listed.max() == 0 and r.max() < 0.95
+
+
+@pytest.mark.parametrize("eq", ["euler", "euler2d"])
+def test_mean_state(lib, eq):
+    """Eigenvectors at the arithmetic mean state, evaluated in pairs as those of
+    the Roe average (no interface of a resolved flow is listed)."""
+    _, listed = ratios(lib, eq, "wave", 400, 400, eig_avg=1)
+    assert listed.max() == 0
+    for kind, size in (("wave", 400), ("weak wave", 25), ("noise", 1e-2), ("derivative noise", 1e-2),
+                       ("jump", 1)):
+        r, _ = ratios(lib, eq, kind, size, 200, eig_avg=1)
+        assert r.max() <= BOUND, (kind, r)
