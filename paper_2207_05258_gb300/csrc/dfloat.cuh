@@ -32,7 +32,7 @@ __device__ __forceinline__ D2 renorm(float s, float e) {  // |e| <= |s|
   return D2{h, __fadd_rn(e, -__fadd_rn(h, -s))};
 }
 __device__ __forceinline__ D2 neg(D2 a) { return D2{-a.h, -a.l}; }
-// a + b; the error is 2^-47 of |a| + |b| (differences included)
+// a + b; the error is at most 2^-46 of |a| + |b| (differences included)
 __device__ __forceinline__ D2 add(D2 a, D2 b) {
   const float s = __fadd_rn(a.h, b.h);
   const float t = __fadd_rn(s, -a.h);
@@ -150,6 +150,16 @@ __device__ __forceinline__ D2 scale_add(D2 b, float a, D2 c) { return add(scale(
 __device__ __forceinline__ double scale_add(double b, double a, double c) {
   return __fma_rn(b, a, c);
 }
+
+// a b - c d and a - b c (in FP64 without the rounding of one product)
+template <class X>
+__device__ __forceinline__ X mul_sub(X a, X b, X c, X d) { return sub(mul(a, b), mul(c, d)); }
+template <class X>
+__device__ __forceinline__ X sub_mul(X a, X b, X c) { return sub(a, mul(b, c)); }
+__device__ __forceinline__ double mul_sub(double a, double b, double c, double d) {
+  return madd(a, b, -mul(c, d));
+}
+__device__ __forceinline__ double sub_mul(double a, double b, double c) { return madd(-b, c, a); }
 
 // c ? a : b, word by word
 __device__ __forceinline__ D2 pick2(bool c, D2 a, D2 b) {

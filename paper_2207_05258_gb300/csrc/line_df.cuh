@@ -56,6 +56,10 @@ struct LineTile {
   __device__ __forceinline__ D2& p(int row, int k) const {
     return reinterpret_cast<D2*>(base + nd * L)[at(row, np, k, L)];
   }
+  // a pair row as doubles (double_rows)
+  __device__ __forceinline__ double& pd(int row, int k) const {
+    return base[nd * L + at(row, np, k, L)];
+  }
   __device__ __forceinline__ double& o(int row, int j) const {
     return base[(nd + np) * L + at(row, no, j, LI)];
   }
@@ -76,6 +80,10 @@ struct LineTile {
   __device__ __forceinline__ D2 dU(int c, int k) const {
     if constexpr (SLIM) return mul(add(X(0, c, k), X(1, c, k)), ial);
     else return p(4 * M + c, k);
+  }
+  __device__ __forceinline__ float dU_lead(int c, int k) const {
+    if constexpr (SLIM) return (X(0, c, k).h + X(1, c, k).h) * ial.h;
+    else return p(4 * M + c, k).h;
   }
   __device__ __forceinline__ D2 Nx(int c, int k) const {
     if constexpr (SLIM) return mul(add(H(0, c, k), H(1, c, k)), ial);
@@ -164,11 +172,12 @@ __device__ __forceinline__ void edge_pairs(const T& r, int k, int S, D2 alp) {
 }
 
 // The data of a line as X: pairs from the tile's pair rows, or doubles
-// formed from its double rows.
-template <class X, class T>
+// formed from its double rows (ROWS: where they are of more than one double,
+// read from the rows that double_rows has made of them).
+template <class X, class T, bool ROWS = false>
 struct LineData;
 template <class T>
-struct LineData<D2, T> {
+struct LineData<D2, T, false> {
   const T& r;
   int S;
   const SchemeParams& sp;
@@ -212,8 +221,8 @@ struct LineData<D2, T> {
     if constexpr (T::M == 4) ut = roe(3);
   }
 };
-template <class T>
-struct LineData<double, T> {
+template <class T, bool ROWS>
+struct LineData<double, T, ROWS> {
   const T& r;
   int S;
   double alpha, dx;
@@ -222,9 +231,11 @@ struct LineData<double, T> {
                                       const SchemeParams& sp_)
       : r(r_), S(S_), alpha(al), dx(d), sp(sp_) {}
   __device__ __forceinline__ double H(int sd, int c, int k) const {
+    if constexpr (ROWS) return r.pd(sd * T::M + c, k);
     return mul(0.5 * dx, madd(alpha, r.N(c, k), sd ? -r.h(c, k) : r.h(c, k)));
   }
   __device__ __forceinline__ double X(int sd, int c, int k) const {
+    if constexpr (ROWS) return r.pd((2 + sd) * T::M + c, k);
     const double dF = sub(r.F(c, k + S), r.F(c, k));
     return mul(0.5, madd(alpha, dU(c, k), sd ? -dF : dF));
   }
@@ -244,12 +255,25 @@ struct LineData<double, T> {
     }
     H = mul(madd(gm1(), madd(-0.5, ke, u[M - 1]), u[M - 1]), ir);
   }
+  // the rows of the eigen-system's inputs (LineTile::E)
+  static constexpr int kE = (T::SLIM ? 4 : 6) * T::M;
   // point k's velocities and enthalpy
   __device__ __forceinline__ void prim_at(int k, double& un, double& ut, double& H) const {
+    if constexpr (ROWS) {
+      un = r.pd(kE + 1, k);
+      H = r.pd(kE + 2, k);
+      if constexpr (T::M == 4) ut = r.pd(kE + 3, k);
+      return;
+    }
     double a[T::M];
 #pragma unroll
     for (int c = 0; c < T::M; ++c) a[c] = r.U(c, k);
     prim(a, un, ut, H);
+  }
+  // sqrt(rho)
+  __device__ __forceinline__ double root(int k) const {
+    if constexpr (ROWS) return r.pd(kE, k);
+    return mul(r.U(0, k), rsqrt_fp64(r.U(0, k)));
   }
   __device__ __forceinline__ void state(int k, bool edge, double& un, double& ut, double& H) const {
     if (!edge) {
@@ -258,9 +282,7 @@ struct LineData<double, T> {
       double uL, tL = 0.0, HL, uR, tR = 0.0, HR;
       prim_at(k, uL, tL, HL);
       prim_at(k + S, uR, tR, HR);
-      const double sl = mul(r.U(0, k), rsqrt_fp64(r.U(0, k)));
-      const double sr = mul(r.U(0, k + S), rsqrt_fp64(r.U(0, k + S)));
-      const double is = recip_fp64(add(sl, sr));
+      const double sl = root(k), sr = root(k + S), is = recip_fp64(add(sl, sr));
       auto roe = [&](double x, double y) { return mul(add(mul(sl, x), mul(sr, y)), is); };
       un = roe(uL, uR);
       ut = roe(tL, tR);
@@ -274,6 +296,41 @@ struct LineData<double, T> {
   }
 };
 
+// Makes of the pair rows doubles of the same quantities, bit for bit what
+// LineData<double, T> forms on the fly: once per point and edge instead of by
+// every item that reads them (Euler: about 160 of 1050 FP64 instructions per
+// point where all items are listed; rhs of such a batch of 614 k points 1296 ->
+// 1122 us). For tiles with many listed items, when the
+// pairs are no longer needed; followed by a barrier.
+template <class T>
+__device__ __forceinline__ void double_rows(const T& r, int S, double alpha, double dx,
+                                            const SchemeParams& sp) {
+  constexpr int M = T::M;
+  const LineData<double, T> in(r, S, alpha, dx, sp);
+  for (int k = threadIdx.x; k < r.L; k += blockDim.x) {
+#pragma unroll
+    for (int c = 0; c < M; ++c) {
+      r.pd(c, k) = in.H(0, c, k);
+      r.pd(M + c, k) = in.H(1, c, k);
+    }
+    if constexpr (T::EUL) {
+      double un, ut = 0.0, H;
+      in.prim_at(k, un, ut, H);
+      r.pd(in.kE, k) = in.root(k);
+      r.pd(in.kE + 1, k) = un;
+      r.pd(in.kE + 2, k) = H;
+      if constexpr (M == 4) r.pd(in.kE + 3, k) = ut;
+    }
+    if (k + S < r.L) {
+#pragma unroll
+      for (int c = 0; c < M; ++c) {
+        r.pd(2 * M + c, k) = in.X(0, c, k);
+        r.pd(3 * M + c, k) = in.X(1, c, k);
+      }
+    }
+  }
+}
+
 // c ? a + y : a
 template <class X>
 __device__ __forceinline__ X add_if(bool c, X a, X y) {
@@ -285,8 +342,8 @@ __device__ __forceinline__ X add_if(bool c, X a, X y) {
 // k, the "-" side about k + S. The latter reverses the stencil and negates H;
 // with -H^- and -M for H^+ and P (M the difference of f^- along an edge) its
 // expressions are those of the "+" side.
-template <class X, class T>
-__device__ __forceinline__ void side_differences(const LineData<X, T>& in, int sd, int c, int k,
+template <class X, class T, bool R>
+__device__ __forceinline__ void side_differences(const LineData<X, T, R>& in, int sd, int c, int k,
                                                  int S, X* x) {
   using P2 = typename Num<X>::Scale;
   const int k0 = sd ? k + S : k, km = sd ? k0 + S : k0 - S, kp = sd ? k : k0 + S;
@@ -316,8 +373,8 @@ using CharOf = LineChar<X, T::M == 1 ? 3 : T::M, T::M == 1 ? 0 : DIR>;
 
 // The characteristic system of the interface between k and k + S (`edge`) or
 // of point k.
-template <int DIR, class X, class T>
-__device__ __forceinline__ CharOf<T, X, DIR> char_system(const LineData<X, T>& in, int k,
+template <int DIR, class X, class T, bool R>
+__device__ __forceinline__ CharOf<T, X, DIR> char_system(const LineData<X, T, R>& in, int k,
                                                          bool edge) {
   CharOf<T, X, DIR> ch;
   if constexpr (T::EUL) {
@@ -334,8 +391,8 @@ __device__ __forceinline__ CharOf<T, X, DIR> char_system(const LineData<X, T>& i
 // pairs, to 60 times the linear parts; returns, in pairs, 12 times the sum of
 // the fields' bounds of side_correction in units of the density. ONE: field
 // q0 alone, to f[0].
-template <int DIR, bool ONE = false, class X, class T>
-__device__ __forceinline__ float interface_side(const LineData<X, T>& in,
+template <int DIR, bool ONE = false, class X, class T, bool R>
+__device__ __forceinline__ float interface_side(const LineData<X, T, R>& in,
                                                 const CharOf<T, X, DIR>& ch,
                                                 const LineWeights<X>& w, int sd, int k, int S,
                                                 X* f, X* lin, int q0 = 0) {
@@ -419,16 +476,24 @@ __device__ __forceinline__ float in_density(const float* x, float H) {
   return fmaxf(fabsf(x[0]), fmaxf(m * rsqrtf(H), fabsf(x[T::M - 1]) * fast_rcp(H)));
 }
 
-// Whether the interface between k and k + S is to be tried in pairs; decided
-// before any of the work. Euler: its linear part and derivative flux in pairs
-// have an error of 2^-48 of the differences, below that of the FP64 form while
-// these are at most kFine of alpha U (1/16: up to 1.08 of it, 1/32: 0.6).
-// Scalar equations take the linear part in FP64 where it matters (fine_grid).
-// False for data outside the pairs' range.
+// How the interface between k and k + S is evaluated, decided before any of the
+// work. `pairs`: tried in pairs; `linear`: with the linear part in pairs, which
+// has an error of 2^-48 of the differences it is made of (in FP64: one of F's
+// rounding). Euler tries only interfaces whose differences are at most kFine
+// of alpha U, where the linear part's and the derivative flux's errors stay
+// below the FP64 form's (1/16: up to 1.08 of it, 1/32: 0.6). Scalar equations
+// take the linear part in FP64 where a difference exceeds 2^-3 of F (coarse
+// grids, sonic points; error of L^1 over the FP64 form's: wave of 15 points
+// 4.2 -> 0.4). All their interfaces are tried: a test for those that would be
+// listed afterwards cost the Buckley-Leverett batch 6% and took 1% off a flow
+// of noise. None is tried where alpha or the density leaves the pairs' range.
+struct Route {
+  bool pairs, linear;
+};
 constexpr float kFine = 1.f / 20.f;
 template <class T>
-__device__ __forceinline__ bool interface_fine(const LineData<D2, T>& in, int k, int S,
-                                               double alpha) {
+__device__ __forceinline__ Route interface_route(const LineData<D2, T>& in, int k, int S,
+                                                 double alpha) {
   const float al = scale_pair(alpha).h;
   if constexpr (T::EUL) {
     const float s = fminf(in.r.E(0, k).h, in.r.E(0, k + S).h);
@@ -436,24 +501,39 @@ __device__ __forceinline__ bool interface_fine(const LineData<D2, T>& in, int k,
 #pragma unroll
     for (int c = 0; c < T::M; ++c) x[c] = difference_top(in, c, k, S);
     const float H = fminf(in.r.E(2, k).h, in.r.E(2, k + S).h);
-    // (one comparison per operand: fmaxf would drop a NaN)
-    return x[0] <= kFine * al * s * s && in_density<T>(x, H) <= kFine * al * s * s;
+    // (x[0] by itself: fmaxf would drop a NaN)
+    return Route{x[0] <= kFine * al * s * s && in_density<T>(x, H) <= kFine * al * s * s, true};
   } else {
-    return true;
+    auto larger = [&](double a, double b) { return fmaxf(fabsf(to_float(a)), fabsf(to_float(b))); };
+    const float top = fmaxf(fmaxf(fabsf(in.H(0, 0, k).h), fabsf(in.H(1, 0, k + S).h)),
+                            fmaxf(fabsf(in.X(0, 0, k).h), fabsf(in.X(1, 0, k).h)));
+    return Route{al > 0.f, top <= 0x1p-3f * larger(in.r.F(0, k), in.r.F(0, k + S))};
   }
 }
-// The linear part in pairs has an error of 2^-48 of the differences it is made
-// of, that in FP64 one of F's rounding. The scalar equations take it in FP64
-// where a difference exceeds 2^-3 of F (coarse grids, sonic points; error of
-// L^1 over the plain FP64 form's: wave of 15 points 4.2 -> 0.4).
+// Whether the limiter's point k is tried in pairs, from the second differences (in units of
+// the density, the component's own): not where they exceed 1/16 of the density,
+// or a quarter of the first differences, and tau's unit.
 template <class T>
-__device__ __forceinline__ bool fine_grid(const LineData<D2, T>& in, int k, int S) {
-  if constexpr (T::EUL) return true;
-  const float top = fmaxf(fmaxf(fabsf(in.H(0, 0, k).h), fabsf(in.H(1, 0, k + S).h)),
-                          fmaxf(fabsf(in.X(0, 0, k).h), fabsf(in.X(1, 0, k).h)));
-  const float F = fmaxf(fabsf(to_float(in.r.F(0, k))), fabsf(to_float(in.r.F(0, k + S))));
-  return top <= 0x1p-3f * F;
+__device__ __forceinline__ bool limiter_fine(const LineData<D2, T>& in, int k, int S) {
+  const T& r = in.r;
+  const float g = fmaxf(in.sp.wp[4].h, in.sp.wp[5].h);
+  float lap[T::M];
+  bool fine = true;
+#pragma unroll
+  for (int c = 0; c < T::M; ++c) {
+    const float q1 = r.dU_lead(c, k - S), q2 = r.dU_lead(c, k);
+    lap[c] = q2 - q1;
+    fine &= fabsf(lap[c]) <= 0.25f * (fabsf(q1) + fabsf(q2)) || g * lap[c] * lap[c] < 0x1p-14f;
+  }
+  if constexpr (T::EUL) {
+    if (in.sp.limiter != 2) {
+      const float s = r.E(0, k).h, x = in_density<T>(lap, r.E(2, k).h);
+      fine = x <= 0.0625f * s * s || g * x * x < 0x1p-14f;
+    }
+  }
+  return fine;
 }
+
 // The linear part of the scalar c in FP64.
 template <class T>
 __device__ __forceinline__ double linear_part_fp64(const T& r, int k, int S, double alpha,
@@ -468,12 +548,12 @@ __device__ __forceinline__ double linear_part_fp64(const T& r, int k, int S, dou
 }
 
 // c from the sums over both sides (lin64: the scalar linear part, where
-// fine_grid is false).
-template <int DIR, class X, class T>
-__device__ __forceinline__ void interface_value(const LineData<X, T>& in,
+// `linear` is false).
+template <int DIR, class X, class T, bool R>
+__device__ __forceinline__ void interface_value(const LineData<X, T, R>& in,
                                                 const CharOf<T, X, DIR>& ch, int k, int S,
-                                                double alpha, X* f, const X* lin, double lin64,
-                                                double* cc) {
+                                                double alpha, X* f, const X* lin, bool linear,
+                                                double lin64, double* cc) {
   constexpr int M = T::M;
   if constexpr (T::EUL) {
     X out[M];
@@ -490,7 +570,7 @@ __device__ __forceinline__ void interface_value(const LineData<X, T>& in,
       cc[c] = to_double(madd(dconst(1.0 / 60.0), lin[c], mul(f[c], dconst(1.0 / 12.0))));
   }
   if constexpr (!T::EUL && std::is_same<X, D2>::value)
-    if (!fine_grid(in, k, S)) cc[0] = add(lin64, to_double(mul(f[0], dconst(1.0 / 12.0))));
+    if (!linear) cc[0] = add(lin64, to_double(mul(f[0], dconst(1.0 / 12.0))));
 }
 
 // The derivative flux dx (h-hat^+ + h-hat^-) of component c at the interface
@@ -571,18 +651,17 @@ __device__ __forceinline__ float interface_sides(const LineData<D2, T>& in,
 // c (to cc) and, in pairs, the derivative flux (to dd) of the interface between
 // points k and k + S; in pairs, false when the correction is not small (the
 // values are then not to be used).
-template <class X, int DIR, class T>
+template <class X, int DIR, bool ROWS = false, class T>
 __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double alpha, double dx,
                                                const SchemeParams& sp, double* cc,
                                                double* dd = nullptr) {
-  const LineData<X, T> in(r, S, alpha, dx, sp);
+  const LineData<X, T, ROWS> in(r, S, alpha, dx, sp);
+  Route route{true, true};
   if constexpr (!std::is_same<X, double>::value) {
-    if (!interface_fine(in, k, S, alpha)) {
+    route = interface_route(in, k, S, alpha);
+    if (!route.pairs) {
 #pragma unroll
-      for (int c = 0; c < T::M; ++c) {
-        cc[c] = 0.0;
-        dd[c] = T::EUL ? 0.0 : derivative_flux_fp64(r, c, k, S, alpha, dx);
-      }
+      for (int c = 0; c < T::M; ++c) cc[c] = dd[c] = 0.0;
       return false;
     }
   }
@@ -594,20 +673,20 @@ __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double 
     for (int c = 0; c < T::M; ++c) f[c] = lin[c] = X{};
 #pragma unroll 1
     for (int sd = 0; sd < 2; ++sd) interface_side<DIR>(in, ch, w, sd, k, S, f, lin);
-    interface_value<DIR>(in, ch, k, S, alpha, f, lin, 0.0, cc);
+    interface_value<DIR>(in, ch, k, S, alpha, f, lin, true, 0.0, cc);
     return true;
   } else {
     const float e = interface_sides<DIR>(in, ch, w, k, S, f, lin, alpha, dx, dd);
     double lin64 = 0.0;
-    if (!fine_grid(in, k, S)) lin64 = linear_part_fp64(r, k, S, alpha, dx);
-    interface_value<DIR>(in, ch, k, S, alpha, f, lin, lin64, cc);
+    if (!route.linear) lin64 = linear_part_fp64(r, k, S, alpha, dx);
+    interface_value<DIR>(in, ch, k, S, alpha, f, lin, route.linear, lin64, cc);
     return interface_weak(r, k, S, e, alpha, sp);
   }
 }
 
 // The limiter's four differences at point k, component c.
-template <class X, class T>
-__device__ __forceinline__ void limiter_differences(const LineData<X, T>& in, int c, int k, int S,
+template <class X, class T, bool R>
+__device__ __forceinline__ void limiter_differences(const LineData<X, T, R>& in, int c, int k, int S,
                                                     X* x) {
   x[0] = in.dU(c, k - S);
   x[1] = in.dU(c, k);
@@ -618,8 +697,8 @@ __device__ __forceinline__ void limiter_differences(const LineData<X, T>& in, in
 // The limited derivative from its characteristic fields (chars) or
 // components z: pairs, 4 times the corrections to the linear
 // dx q_0' = 3/4 (u_{i+1} - u_{i-1}) - dx (v_{i-1} + v_{i+1}) / 4; FP64, dx v~.
-template <int DIR, class X, class T>
-__device__ __forceinline__ void limiter_sum(const LineData<X, T>& in, const CharOf<T, X, DIR>& ch,
+template <int DIR, class X, class T, bool R>
+__device__ __forceinline__ void limiter_sum(const LineData<X, T, R>& in, const CharOf<T, X, DIR>& ch,
                                             int k, int S, double idx, bool chars, X* z,
                                             double* vt) {
   constexpr int M = T::M;
@@ -690,11 +769,18 @@ __device__ __forceinline__ bool limiter_weak(const T& r, int k, float e, const S
 }
 
 // The limited derivative at point k; in pairs, false as interface_line.
-template <class X, int DIR, class T>
+template <class X, int DIR, bool ROWS = false, class T>
 __device__ __forceinline__ bool limiter_line(const T& r, int k, int S, double dx, double idx,
                                              const SchemeParams& sp, double* vt) {
   constexpr int M = T::M;
-  const LineData<X, T> in(r, S, 0.0, dx, sp);
+  const LineData<X, T, ROWS> in(r, S, 0.0, dx, sp);
+  if constexpr (!std::is_same<X, double>::value) {
+    if (!limiter_fine(in, k, S)) {
+#pragma unroll
+      for (int c = 0; c < M; ++c) vt[c] = 0.0;
+      return false;
+    }
+  }
   float sum = 0.f;
   X x[M][4], z[M];
 #pragma unroll
@@ -770,6 +856,18 @@ template <class T>
 struct Group {
   static constexpr int NC = T::M == 1 ? 1 : 4;  // lanes per side
   static constexpr int kInterface = 2 * NC, kPoint = NC;  // lanes per item
+  // FP64 instructions of a warp of items: in groups, and one item per thread
+  static constexpr int group_f = T::M == 1 ? 75 : 150, whole_f = T::M == 1 ? 130 : 450;
+  static constexpr int group_l = T::M == 1 ? 60 : 115, whole_l = T::M == 1 ? 60 : 300;
+  // Whether n items are sooner done in groups: the FP64 pipes of an SM's four
+  // sub-partitions set the time, however many warps share them. (With the
+  // warps of the CTA for the four, the wide form's 16 took a whole tile of
+  // listed items in groups: rhs of an Euler instance of 200 points, all items
+  // listed, 92 us; with this rule and double_rows 53.)
+  __host__ __device__ static constexpr bool few(int n, int lanes, int group, int whole) {
+    const int per = 32 / lanes;
+    return ((n + per - 1) / per + 3) / 4 * group <= ((n + 31) / 32 + 3) / 4 * whole;
+  }
 };
 
 // c of the interface (k, k + S), output index j, by the lanes of a group;
@@ -885,10 +983,13 @@ __device__ __forceinline__ void listed_items(const T& r, const unsigned short* l
   constexpr int M = T::M;
   using G = Group<T>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // groups: 150 instructions per 32 / kInterface interfaces and warp; whole
-  // items: 450 per 32 (limiter: 115 and 300)
   constexpr int gf = 32 / G::kInterface, gl = 32 / G::kPoint;
-  const bool few_f = nf <= 3 * gf * nw, few_l = nl <= 3 * gl * nw;
+  const bool few_f = G::few(nf, G::kInterface, G::group_f, G::whole_f);
+  const bool few_l = G::few(nl, G::kPoint, G::group_l, G::whole_l);
+  if (!few_f || !few_l) {  // uniform
+    double_rows(r, S, alpha, dx, sp);
+    __syncthreads();
+  }
   const int uf = few_f ? (nf + gf - 1) / gf : (nf + 31) / 32;
   const int ul = few_l ? (nl + gl - 1) / gl : (nl + 31) / 32;
   // Euler: the listed interfaces' derivative fluxes, a component per lane
@@ -909,7 +1010,7 @@ __device__ __forceinline__ void listed_items(const T& r, const unsigned short* l
       } else if (u * 32 + lane < nf) {
         const int j = list_f[u * 32 + lane];
         double x[M];
-        interface_line<double, DIR>(r, at(j, false), S, alpha, dx, sp, x);
+        interface_line<double, DIR, true>(r, at(j, false), S, alpha, dx, sp, x);
 #pragma unroll
         for (int c = 0; c < M; ++c) r.C(c, j) = x[c];
       }
@@ -923,7 +1024,7 @@ __device__ __forceinline__ void listed_items(const T& r, const unsigned short* l
       } else if (v * 32 + lane < nl) {
         const int j = list_l[v * 32 + lane];
         double x[M];
-        limiter_line<double, DIR>(r, at(j, true), S, dx, idx, sp, x);
+        limiter_line<double, DIR, true>(r, at(j, true), S, dx, idx, sp, x);
 #pragma unroll
         for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
       }
@@ -936,14 +1037,17 @@ __device__ __forceinline__ void listed_items(const T& r, const unsigned short* l
 // threads per item share its work by roles, so that the phase takes the time
 // of one role's instruction stream and every sub-partition has warps to
 // interleave. Roles: the two sides of an interface (FIELDS: one per side and
-// field), the limiter (FIELDS: one per field), the derivative flux. The
+// field), the limiter (FIELDS: one per field), the derivative flux and (LIN:
+// scalar equations in 1D; else the same threads' second task) the linear part
+// in FP64, each of whose chains of FP64 operations takes as long as a side.
+// The
 // arithmetic of every quantity is that of interface_line and limiter_line,
 // operation for operation, so the results are the same bits.
 // ---------------------------------------------------------------------------
-template <int M, bool FIELDS>
+template <int M, bool FIELDS, bool LIN = false>
 struct WideRoles {
   static constexpr int sides = FIELDS ? 2 * M : 2, limiter = FIELDS ? M : 1;
-  static constexpr int count = sides + limiter + 1;
+  static constexpr int count = sides + limiter + 1 + LIN;
   // exchange rows of LI pairs: sides' fields, "-" side's linear parts, the
   // limiter's fields; then the bounds of the sides' and the limiter's fields
   static constexpr int rows = 7 * M;
@@ -959,13 +1063,13 @@ struct ItemLists {
 // Phases 3 and 3b for role `role` of interface j (left point kf) and point j
 // (kl). xch: exchange rows. Every thread of the CTA calls it; C, D and lim
 // are ready after the next barrier.
-template <int DIR, bool FIELDS, class T, class L, class At>
+template <int DIR, bool FIELDS, bool LIN = false, class T, class L, class At>
 __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j, bool has_f, int kf,
                                            bool has_l, int kl, int S, double alpha, double dx,
                                            double idx, const SchemeParams& sp, L& ls, At at,
                                            int rot) {
   constexpr int M = T::M;
-  using R = WideRoles<M, FIELDS>;
+  using R = WideRoles<M, FIELDS, LIN>;
   const LineData<D2, T> in(r, S, alpha, dx, sp);
   auto row = [&](int q) -> D2& { return xch[q * r.LI + j]; };
   CharOf<T, D2, DIR> ch;
@@ -974,8 +1078,10 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
   const bool lim_role = role >= R::sides && role < R::sides + R::limiter;
   const int lq = role - R::sides;
   const bool limited = sp.limiter != 0, chars = T::EUL && sp.limiter != 2;
-  // interfaces that are tried in pairs (every role finds the same)
-  const bool try_f = has_f && interface_fine(in, kf, S, alpha);
+  // items that are tried in pairs (every role of an item finds the same)
+  const Route route = has_f ? interface_route(in, kf, S, alpha) : Route{false, true};
+  const bool try_f = route.pairs;
+  const bool try_l = FIELDS && lim_role && has_l && limited && limiter_fine(in, kl, S);
   if (role < R::sides) {
     if (try_f) {
       const LineWeights<D2> w = line_weights<D2>(sp, false);
@@ -997,7 +1103,7 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
     if (has_l && limited) {
       if constexpr (FIELDS) {
         float e = 0.f;
-        row(3 * M + lq) = limiter_field<DIR>(in, ch, kl, S, sp, lq, e);
+        if (try_l) row(3 * M + lq) = limiter_field<DIR>(in, ch, kl, S, sp, lq, e);
         row(6 * M + lq).h = e;
       } else {
         double x[M];
@@ -1007,15 +1113,16 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
         for (int c = 0; c < M; ++c) r.lim(c, j) = x[c];
       }
     }
-  } else if (T::EUL ? try_f : has_f) {
+  } else if (role == R::sides + R::limiter && (T::EUL ? try_f : has_f)) {
 #pragma unroll 1  // (code to fetch)
     for (int c = 0; c < M; ++c) {
       Q2 x[5];
       sides_differences(in, c, kf, S, x);
       r.D(c, j) = derivative_flux(in, x, c, kf, S, alpha, dx);
     }
-    if (!fine_grid(in, kf, S)) r.C(0, j) = linear_part_fp64(r, kf, S, alpha, dx);
   }
+  if (role == R::count - 1 && try_f && !route.linear)
+    r.C(0, j) = linear_part_fp64(r, kf, S, alpha, dx);
   __syncthreads();
   if (role == 0 && has_f && !try_f) ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
   if (role == 0 && try_f) {
@@ -1030,14 +1137,16 @@ __device__ __forceinline__ void wide_items(const T& r, D2* xch, int role, int j,
         e[1] += row(5 * M + c).h;
       }
     }
-    interface_value<DIR>(in, ch, kf, S, alpha, f, lin, r.C(0, j), cc);
+    interface_value<DIR>(in, ch, kf, S, alpha, f, lin, route.linear, r.C(0, j), cc);
     if (!interface_weak(r, kf, S, e[0] + e[1], alpha, sp))
       ls.f[atomicAdd(&ls.nf, 1)] = (unsigned short)j;
 #pragma unroll
     for (int c = 0; c < M; ++c) r.C(c, j) = cc[c];
   }
   if constexpr (FIELDS) {
-    if (lim_role && lq == 0 && has_l && limited) {
+    if (lim_role && lq == 0 && has_l && limited && !try_l)
+      ls.l[atomicAdd(&ls.nl, 1)] = (unsigned short)j;
+    if (lim_role && lq == 0 && try_l) {
       D2 z[M];
       double x[M];
       float e = 0.f;

@@ -291,7 +291,7 @@ constexpr bool wide_fields(int P) { return EQ == HWENO_EULER && P <= kFieldsMax;
 template <int EQ>
 constexpr int wide_threads(int P) {
   return (wide_fields<EQ>(P) ? WideRoles<Dim1<EQ>::M, true>::count
-                             : WideRoles<Dim1<EQ>::M, false>::count) * (P + 4);
+                             : WideRoles<Dim1<EQ>::M, false, EQ != HWENO_EULER>::count) * (P + 4);
 }
 template <int EQ>
 constexpr size_t wide_bytes(int P) {
@@ -342,8 +342,9 @@ __device__ __forceinline__ unsigned long long stage_wide_df(const Args1D& a, con
   if (er >= 0 && er < M && j < np + 3) edge_pair(r, er, j, 1, alp);
   __syncthreads();
   // 3: items
-  wide_items<0, FIELDS>(r, xch, role, j, j <= np, j + 1, j < np, j + 2, 1, alpha, dx, idx, a.sp, ls,
-                        [](int i, bool lim) { return lim ? i + 2 : i + 1; }, 0);
+  wide_items<0, FIELDS, EQ != HWENO_EULER>(r, xch, role, j, j <= np, j + 1, j < np, j + 2, 1, alpha,
+                                           dx, idx, a.sp, ls,
+                                           [](int i, bool lim) { return lim ? i + 2 : i + 1; }, 0);
   __syncthreads();
   // 4: points, a component per role
   const Update1D update(mode, dt, idx, idx2);

@@ -17,8 +17,8 @@
 // phi_2 |p_2 - p_0|), and where the linear part is taken in pairs that has one
 // of 2^-48 of the differences. The FP64 form starts from the full values and
 // has an error of a few 2^-53 of alpha U. Items are evaluated in pairs while
-// their error stays below that: kWeakPhi, kWeakLevel and the like here, kFine
-// and fine_grid in line_df.cuh. Where they fail (shocks, under-resolved jumps
+// their error stays below that: kWeakPhi, kWeakLevel and the like here,
+// interface_route in line_df.cuh. Where they fail (shocks, under-resolved jumps
 // and waves, noise, and whatever leaves the FP32 range: any overflow or NaN
 // fails the same tests) the caller evaluates the item in FP64.
 #pragma once
@@ -319,10 +319,10 @@ struct LineChar {
   __device__ __forceinline__ Factors factors(const X* x) const {
     Factors f;
     f.x0 = x[0];
-    f.A = madd(b, x[kE], sub(mul(bq, x[0]), mul(bu, x[kn])));
-    if constexpr (M == 4) f.A = sub(f.A, mul(bt, x[kt]));
-    f.B = sub(mul(huc, x[0]), mul(hic, x[kn]));
-    if constexpr (M == 4) f.S = sub(x[kt], mul(ut, x[0]));
+    f.A = madd(b, x[kE], mul_sub(bq, x[0], bu, x[kn]));
+    if constexpr (M == 4) f.A = sub_mul(f.A, bt, x[kt]);
+    f.B = mul_sub(huc, x[0], hic, x[kn]);
+    if constexpr (M == 4) f.S = sub_mul(x[kt], ut, x[0]);
     return f;
   }
   // R s

@@ -263,4 +263,37 @@ void host_line(int form, int eq, int m, int n, double dx, double alpha, const do
                      : line_pairs<4, true, true>;
   f(eq, n, dx, alpha, U, V, o, L1, L2, Vt, listed);
 }
+
+// Arithmetic of dfloat.cuh and weno_df.cuh: operation `op` on a[i] and b[i]
+// (pairs made by to_pair, but those of op 4), results r[i] and, pairs, both words
+void host_arith(int op, int n, const double* a, const double* b, double* r, float* h, float* l) {
+  for (int i = 0; i < n; ++i) {
+    D2 x = to_pair(a[i]);
+    const D2 y = to_pair(b[i]);
+    switch (op) {
+      case 0: break;
+      case 1: x = div(x, y); break;
+      case 2: x = rsqrt2(x); break;
+      case 3: x = mul(x, y); break;
+      case 4: x = D2{(float)a[i], (float)b[i]}; break;
+      case 5: x = madd(x, y, D2{1.f, 0.f}); break;
+      case 6: x = add(x, y); break;
+    }
+    h[i] = x.h;
+    l[i] = x.l;
+    r[i] = op == 4 ? to_double(x.h) : op == 7 ? recip_fp64(a[i])
+           : op == 8 ? rsqrt_fp64(a[i]) : op == 9 ? (double)to_float(a[i]) : to_double(x);
+  }
+}
+// whether n listed items go to groups of lanes (interfaces, limiter points)
+int host_few(int m, int limiter, int n) {
+  using A = LineTile<1, 0, false>;
+  using B = LineTile<3, 0, true>;
+  auto few = [&](auto g) {
+    using G = decltype(g);
+    return limiter ? G::few(n, G::kPoint, G::group_l, G::whole_l)
+                   : G::few(n, G::kInterface, G::group_f, G::whole_f);
+  };
+  return m == 1 ? few(Group<A>{}) : few(Group<B>{});
+}
 }
