@@ -677,10 +677,11 @@ __device__ __forceinline__ bool interface_line(const T& r, int k, int S, double 
     return true;
   } else {
     const float e = interface_sides<DIR>(in, ch, w, k, S, f, lin, alpha, dx, dd);
+    const bool weak = interface_weak(r, k, S, e, alpha, sp);
     double lin64 = 0.0;
-    if (!route.linear) lin64 = linear_part_fp64(r, k, S, alpha, dx);
+    if (weak && !route.linear) lin64 = linear_part_fp64(r, k, S, alpha, dx);
     interface_value<DIR>(in, ch, k, S, alpha, f, lin, route.linear, lin64, cc);
-    return interface_weak(r, k, S, e, alpha, sp);
+    return weak;
   }
 }
 
