@@ -145,8 +145,9 @@ typedef struct hweno_options {
                       1 arithmetic mean */
   int tile_variant; /* 1D tile shape 0 .. HWENO_TILE_VARIANTS - 1 (see
                        hweno_autotune; results do not depend on it); ignored
-                       in 2D. 0, the default: 128 threads, 124 points; large
-                       FP64 Euler batches 256 threads, 252 points */
+                       in 2D. 0: 128 threads, 124 points. A new context of a
+                       large FP64 Euler batch starts with 2 (256 threads, 252
+                       points), any other with 0 */
   int fused_small;  /* 1D: 1 = when every instance has at most
                        HWENO_FUSED_MAX_POINTS points, hweno_step runs the whole
                        step (wave speed, three stages, time update) in one
@@ -206,7 +207,8 @@ int hweno_default_options(hweno_options* opt);
  * set (nx, ny < 4; batch < 1; 2D with batch > 1; periodic on one side only;
  * DMR kinds outside y-low/y-high or with Burgers; Buckley-Leverett in 2D or
  * with reflective walls), HWENO_ENOMEM / HWENO_ECUDA
- * for allocation or runtime failures. Options start at hweno_default_options. */
+ * for allocation or runtime failures. Options start at hweno_default_options,
+ * tile_variant at the shape for the batch's size (hweno_get_options). */
 int hweno_create(hweno_ctx** out, int equation, const hweno_grid* grid, double gamma,
                  const hweno_bc* bc);
 

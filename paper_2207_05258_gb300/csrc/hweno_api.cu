@@ -52,9 +52,10 @@ struct hweno_ctx {
   int ct_first[kNumVariants1D][HWENO_MAX_SIZE_CLASSES + 1] = {};
   int class_variant[HWENO_MAX_SIZE_CLASSES] = {};
   bool mixed = false;  // stages launched per class (set by hweno_autotune_classes)
-  // the current variant (aliases of the arrays above)
+  // the current variant (aliases of the arrays above), and the one whose tiles
+  // set the order of hweno_totals' sums
   int ntiles = 0;
-  int variant = 0;
+  int variant = 0, sum_variant = 0;
   int tile = kTile1D;
   int tiles_cap = 0;  // largest table (smallest tile)
   int* d_tile0_inst = nullptr;   // variant 0, used by the adjoint
@@ -295,7 +296,7 @@ int use_variant(hweno_ctx* c, int v) {
   if (c->graph) cudaGraphExecDestroy(c->graph);
   c->graph = nullptr;
   c->mixed = false;
-  c->variant = v;
+  c->variant = c->sum_variant = v;
   c->tile = tile_points(v);
   c->d_tile_inst = c->d_vt_inst[v];
   c->d_tile_start = c->d_vt_start[v];
@@ -305,19 +306,18 @@ int use_variant(hweno_ctx* c, int v) {
   return HWENO_OK;
 }
 
-// The tile shape that stands for option value v: FP64 Euler batches of at
-// least four waves of 252-point tiles (256 threads, two CTAs per SM) take
-// those for the default 124 points, unless they cover more than 5% more
-// threads: warps of one CTA on a sub-partition share their instruction fetch
-// (Riemann batch of 1.28 M points 1.65 -> 1.52 ms per plain step). Results do not
-// depend on the shape.
-int default_tile(const hweno_ctx* c, int v) {
+// The tile shape that a new context starts with: FP64 Euler batches of at least
+// four waves of 252-point tiles (256 threads, two CTAs per SM) take those, unless
+// they cover more than 5% more threads than 124-point ones: warps of one CTA on a
+// sub-partition share their instruction fetch (Riemann batch of 1.28 M points
+// 1.65 -> 1.52 ms per plain step). Results do not depend on the shape.
+int default_tile(const hweno_ctx* c) {
   constexpr int large = 2;
   static_assert(kVariants1D[large].threads == 256 && kVariants1D[large].ppt == 1, "252 points");
   const long long n = c->vt_ntiles[0], n256 = c->vt_ntiles[large];
-  const bool take = v == 0 && !c->fp32 && c->eq == HWENO_EULER && n256 >= 4 * 304 &&
+  const bool take = !c->fp32 && c->eq == HWENO_EULER && n256 >= 4 * 2 * kSMs &&
                     40 * n256 <= 21 * n;
-  return take ? large : v;
+  return take ? large : 0;
 }
 
 // Size classes of a 1D batch: the distinct instance sizes when there are at
@@ -931,10 +931,15 @@ int hweno_create(hweno_ctx** out, int equation, const hweno_grid* grid, double g
   c->d_inst_tiles = c->d_vt_tiles[0];
   c->ntiles0 = c->ntiles = c->vt_ntiles[0];
   select_hx(c);
-  if (c->dim == 1 && (rc = use_variant(c, default_tile(c, 0))) != HWENO_OK) {
-    free_all(c);
-    delete c;
-    return rc;
+  if (c->dim == 1) {
+    const int v = default_tile(c);
+    if ((rc = use_variant(c, v)) != HWENO_OK) {
+      free_all(c);
+      delete c;
+      return rc;
+    }
+    c->opt.tile_variant = v;
+    c->sum_variant = 0;  // (until a shape is chosen, sums in the order of 124-point tiles)
   }
   *out = c;
   return HWENO_OK;
@@ -947,8 +952,7 @@ int hweno_set_options(hweno_ctx* c, const hweno_options* o) {
   const hweno_options old = c->opt;
   c->opt = *o;
   int rc = HWENO_OK;
-  if (c->dim == 1 && o->tile_variant != old.tile_variant)
-    rc = use_variant(c, default_tile(c, o->tile_variant));
+  if (c->dim == 1 && o->tile_variant != c->variant) rc = use_variant(c, o->tile_variant);
   if (rc != HWENO_OK) c->opt = old;
   select_hx(c);
   // a graph recorded by hweno_run holds the old scheme parameters
@@ -1440,8 +1444,7 @@ int hweno_totals(hweno_ctx* c, const void* U, double* totals, void* stream) {
   if (!c) return HWENO_EINVAL;
   if (!U || !totals) return fail(c, HWENO_EINVAL, "null array");
   const double cell = c->dim == 2 ? ((c->x1 - c->x0) / c->nx[0]) * ((c->y1 - c->y0) / c->ny) : 0.0;
-  // 1D: the option's tile table (not default_tile's), which sets the order of the sum
-  const int v = c->dim == 1 ? c->opt.tile_variant : 0;
+  const int v = c->sum_variant;  // (2D: 0)
   const int ntot = c->dim == 1 ? c->vt_ntiles[v] : c->ntiles_tot;
   const cudaError_t e = launch_totals(c->m, c->fp32, c->dim, U, ntot,
                                       c->dim == 1 ? tile_points(v) : c->tile, c->d_vt_inst[v],

@@ -115,6 +115,7 @@ constexpr TileVariant kVariants1D[] = {{128, 1}, {64, 1}, {256, 1}, {128, 2}, {6
 constexpr int kNumVariants1D = HWENO_TILE_VARIANTS;
 static_assert(sizeof(kVariants1D) / sizeof(kVariants1D[0]) == kNumVariants1D, "variant table");
 constexpr int tile_points(int v) { return kVariants1D[v].threads * kVariants1D[v].ppt - 4; }
+constexpr int kSMs = 152;  // of a GB300; sets where launches fill the GPU
 constexpr int kVariants1DPoints = 252;  // largest tile of any variant
 constexpr int kThreads1D = 128;
 constexpr int kTile1D = tile_points(0);

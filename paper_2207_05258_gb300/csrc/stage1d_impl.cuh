@@ -598,7 +598,7 @@ k_stage_wide_1d_f64(const __grid_constant__ Args1D a, int mode, int P) {
 
 // The wide form is taken while there is at most one tile per SM: the tiled
 // kernel's CTAs of four warps would then leave SMs or sub-partitions idle.
-inline bool wide_fits(int P, int ntiles) { return P <= kWideMax && ntiles <= 152; }
+inline bool wide_fits(int P, int ntiles) { return P <= kWideMax && ntiles <= kSMs; }
 
 template <int EQ, bool FIELDS>
 cudaError_t stage_wide_launch(int mode, int P, const Args1D& a, int ntiles, cudaStream_t s) {

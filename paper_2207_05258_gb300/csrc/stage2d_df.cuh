@@ -427,16 +427,16 @@ cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
 }
 
 // The wide form of a sweep while its tiles number at most one per SM; CTAs of
-// 256 threads from four waves (of 2 x 152) of them, unless their wider tiles
+// 256 threads from four waves (of two per SM) of them, unless their wider tiles
 // cover more than 5% more threads; else CTAs of 128.
 inline bool large_tiles(long long tiles, long long tiles256) {
-  return tiles256 >= 4 * 304 && 40 * tiles256 <= 21 * tiles;
+  return tiles256 >= 4 * 2 * kSMs && 40 * tiles256 <= 21 * tiles;
 }
 template <int EQ>
 cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
   auto tiles = [&](int TX) { return (long long)((a.nx + TX - 1) / TX) * a.ny; };
   const long long n = tiles(Shape2D<kThreads2D>::TX);
-  if (n <= 152) return xsweep_f64<EQ, kWideThreads2D>(mode, a, s);
+  if (n <= kSMs) return xsweep_f64<EQ, kWideThreads2D>(mode, a, s);
   return large_tiles(n, tiles(Shape2D<kThreadsF64>::TX)) ? xsweep_f64<EQ, kThreadsF64>(mode, a, s)
                                                          : xsweep_f64<EQ, kThreads2D>(mode, a, s);
 }
@@ -445,7 +445,7 @@ cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
   constexpr int R = Shape2D<kThreads2D>::R;
   auto tiles = [&](int C) { return (long long)((a.nx + C - 1) / C) * ((a.ny + R - 1) / R); };
   const long long n = tiles(Shape2D<kThreads2D>::C);
-  if (n <= 152) return ysweep_f64<EQ, kWideThreads2D>(mode, a, s);
+  if (n <= kSMs) return ysweep_f64<EQ, kWideThreads2D>(mode, a, s);
   return large_tiles(n, tiles(Shape2D<kThreadsF64>::C)) ? ysweep_f64<EQ, kThreadsF64>(mode, a, s)
                                                         : ysweep_f64<EQ, kThreads2D>(mode, a, s);
 }
