@@ -19,11 +19,9 @@
 // one 32-byte sector of a row. Both give 128 interfaces, one per thread, and
 // 51 to 55 KB of shared memory, four CTAs per SM.
 
-// Large grids take CTAs of 256 threads (252 points; 8 columns x 31 rows), two
-// per SM: the warps of a sub-partition that belong to one CTA run the same
-// code at about the same time and share its fetch (double Mach 1920 x 480
-// 3.43 -> 3.12 ms per step; 256^2, with fewer than four waves of them, 0.335
-// -> 0.346).
+// Large Euler grids take CTAs of 256 threads (252 points; 8 columns x 31 rows),
+// two per SM: the warps of a sub-partition that belong to one CTA run the same
+// code at about the same time and share its fetch (large_tiles).
 constexpr int kThreadsF64 = 256;
 template <int NT>
 struct Shape2D {  // NT: 128, 256, or kWideThreads2D (tiles of 128)
@@ -426,9 +424,12 @@ cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// The wide form of a sweep while its tiles number at most one per SM; CTAs of
-// 256 threads from four waves (of two per SM) of them, unless their wider tiles
-// cover more than 5% more threads; else CTAs of 128.
+// The wide form of a sweep while its tiles number at most one per SM. Euler
+// takes CTAs of 256 threads from four waves (of two per SM) of them on, unless
+// their wider tiles cover more than 5% more threads (a step with them always /
+// never, ms: 256^2 0.348 / 0.335, 512^2 1.067 / 1.019 (x-sweep padded by 20%),
+// 640^2 1.468 / 1.488, 1000 x 500 1.687 / 1.782, 1024^2 3.39 / 3.52); Burgers, with
+// a quarter of the instructions to fetch, never (1024^2 0.894 / 0.839).
 inline bool large_tiles(long long tiles, long long tiles256) {
   return tiles256 >= 4 * 2 * kSMs && 40 * tiles256 <= 21 * tiles;
 }
@@ -437,8 +438,10 @@ cudaError_t xsweep_f64(int mode, const Args2D& a, cudaStream_t s) {
   auto tiles = [&](int TX) { return (long long)((a.nx + TX - 1) / TX) * a.ny; };
   const long long n = tiles(Shape2D<kThreads2D>::TX);
   if (n <= kSMs) return xsweep_f64<EQ, kWideThreads2D>(mode, a, s);
-  return large_tiles(n, tiles(Shape2D<kThreadsF64>::TX)) ? xsweep_f64<EQ, kThreadsF64>(mode, a, s)
-                                                         : xsweep_f64<EQ, kThreads2D>(mode, a, s);
+  if constexpr (EQ == HWENO_EULER)
+    if (large_tiles(n, tiles(Shape2D<kThreadsF64>::TX)))
+      return xsweep_f64<EQ, kThreadsF64>(mode, a, s);
+  return xsweep_f64<EQ, kThreads2D>(mode, a, s);
 }
 template <int EQ>
 cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
@@ -446,6 +449,8 @@ cudaError_t ysweep_f64(int mode, const Args2D& a, cudaStream_t s) {
   auto tiles = [&](int C) { return (long long)((a.nx + C - 1) / C) * ((a.ny + R - 1) / R); };
   const long long n = tiles(Shape2D<kThreads2D>::C);
   if (n <= kSMs) return ysweep_f64<EQ, kWideThreads2D>(mode, a, s);
-  return large_tiles(n, tiles(Shape2D<kThreadsF64>::C)) ? ysweep_f64<EQ, kThreadsF64>(mode, a, s)
-                                                        : ysweep_f64<EQ, kThreads2D>(mode, a, s);
+  if constexpr (EQ == HWENO_EULER)
+    if (large_tiles(n, tiles(Shape2D<kThreadsF64>::C)))
+      return ysweep_f64<EQ, kThreadsF64>(mode, a, s);
+  return ysweep_f64<EQ, kThreads2D>(mode, a, s);
 }
