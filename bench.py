@@ -224,6 +224,14 @@ def describe(w):
             % (w.nx[0], w.ny))
 
 
+def cluster_kernel(w, precision):
+    """The kernel of the cluster step (launch_step_cluster)."""
+    if precision == "fp64" and (w.equation != "euler" or max(w.nx) > 448):
+        return "k_step_cluster_f64 (in place of k_step_cluster_%s1d)" % (
+            "split_" if max(w.nx) <= 448 else "")
+    return "k_step_cluster_split_1d" if max(w.nx) <= 448 else "k_step_cluster_1d"
+
+
 def _r4(x):
     return None if x is None else round(x, 4)
 
@@ -514,6 +522,9 @@ def run_ours(args, rank, world, dev_index):
         run_s = pers[3] * 1e-3
         achieved = ALGO_FLOPS_PER_POINT_STEP[(w.equation, w.dim)] * pers[1] / run_s / 1e12
         rtraffic = MEASURED_RUN_TRAFFIC_PER_POINT_STEP.get(args.precision)
+    f64 = "_f64" if args.precision == "fp64" else ""
+    # (FP64 states: most operations run as pairs of FP32 numbers, so that the
+    # rate of the scheme's operations can exceed the FP64 pipe's)
     roof = {"bound": "alu", "achieved": round(achieved, 4), "peak": peak, "unit": "TFLOP/s",
             "frac": round(achieved / peak, 4),
             **({"dfma_loop_tflops": round(fp64_loop, 4),
@@ -523,14 +534,14 @@ def run_ours(args, rank, world, dev_index):
                        (None if rtraffic is None else rtraffic * pers[1]),
             "kernel": ("k_run_1d<%s,%s> (K = %d steps per launch)" % (w.equation, args.precision,
                                                                      args.steps) if use_pers else
-                       "%s<%s,%s>%s" % ("k_step_cluster_split_1d" if max(w.nx) <= 448 else
-                                        "k_step_cluster_1d", w.equation, args.precision,
-                                        " (K = %d steps per launch)" % args.steps
+                       "%s<%s,%s>%s" % (cluster_kernel(w, args.precision), w.equation,
+                                        args.precision, " (K = %d steps per launch)" % args.steps
                                         if use_crun else "") if use_clus else
-                       "k_stage_1d<%s,%s>" % (w.equation, args.precision) if w.dim == 1 else
+                       "k_stage_1d%s<%s,%s>" % (f64, w.equation, args.precision) if w.dim == 1 else
                        "k_stage_2d<%s,%s> (fused x and y parts)" % (w.equation, args.precision)
                        if fused2d else
-                       "k_xsweep_2d + k_ysweep_2d <%s,%s>" % (w.equation, args.precision)),
+                       "k_xsweep_2d%s + k_ysweep_2d%s <%s,%s>" % (f64, f64, w.equation,
+                                                                  args.precision)),
             "kernel_share_of_step": (round(pers[3] / pers[0], 4) if use_pers else
                                      1.0 if use_crun else
                                      round(clus[3] / clus[0], 4) if use_clus else
@@ -558,14 +569,11 @@ def run_ours(args, rank, world, dev_index):
            **({"plain": plain} if use_clus else {}),
            "config": {"workload": describe(w),
                       "instances": w.batch, "points": w.points, "precision": args.precision,
-                      "l2": ("flushed before the timed launch (256 MiB write): the working "
-                             "set (%.1f MB) fits in the 129 MB L2" % working_set_mb(w, args.precision)
-                             if use_crun else
-                             "flushed between timed steps (256 MiB write): the working set "
-                             "(%.1f MB) fits in the 129 MB L2" % working_set_mb(w, args.precision)
-                             if small else
-                             "no flush inside the timed graph of K steps: the per-step working "
-                             "set (state + stage buffers, %.0f MB) exceeds the 129 MB L2"
+                      "l2": ("flushed before the timed launch (working set %.1f MB)"
+                             % working_set_mb(w, args.precision) if use_crun else
+                             "flushed between timed steps (working set %.1f MB)"
+                             % working_set_mb(w, args.precision) if small else
+                             "inputs larger than L2 (working set %.0f MB)"
                              % (working_set_mb(w, args.precision))),
                       "timing": ("the K steps as one launch on thread-block clusters "
                                  "(hweno_run_persistent, fused_small = 2) after an L2 flush, "
@@ -991,6 +999,33 @@ def _compact(out):
     return c
 
 
+def headline(out):
+    """The JSON line as printed: short enough (2.5 KB with the other workloads)
+    to survive where only the end of a program's output is kept. Left out are
+    the notes and the autotuner's table per size class and, where the other
+    workloads are in it, all of those but value and roofline fraction and the
+    other launch forms; main() prints the whole record on stderr."""
+    def cut(x):
+        if not isinstance(x, dict):
+            return x
+        return {k: cut(v) for k, v in x.items()
+                if k not in ("note", "peak_source", "size_classes", "sample")}
+
+    def entry(v):
+        if "roofline" not in v:  # a sub-configuration that failed
+            return v
+        return {"value": v["value"], "roofline": {"frac": v["roofline"]["frac"]}}
+
+    line = cut(out)
+    if "configs" in out:
+        for k in ("us_per_step", "no_graph", "graph", "plain", "persistent", "point_updates_timed"):
+            line.pop(k, None)
+        line.get("fp32", {}).pop("persistent", None)
+        line["configs"] = {k: entry(v) if "value" in v or "error" in v else
+                           {p: entry(x) for p, x in v.items()} for k, v in out["configs"].items()}
+    return line
+
+
 def other_configs(args, dev_index):
     """The other benchmark workloads, each with its own roofline, for the
     headline line: 1D Burgers N = 400, the smooth 2D Euler grids 256^2 to
@@ -1046,7 +1081,8 @@ def main():
                 v.get("gpu_launches", 0) for c in out["configs"].values()
                 for v in (c.values() if "value" not in c else [c]))
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        print("detail: " + json.dumps(out), file=sys.stderr, flush=True)
+        print(json.dumps(headline(out), separators=(",", ":")), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
