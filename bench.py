@@ -77,19 +77,20 @@ PEAK_TFLOPS = {"fp64": 1.25, "fp32": 152 * 128 * 2 * 2.07e9 / 1e12}
 # mean of the three stage launches of one step of the autotuned tile).
 MEASURED_STAGE_TRAFFIC_PER_POINT = {"fp64": None, "fp32": 52.5}
 # Persistent kernel, per point-step (all three stages; FP64: 1024 instances,
-# 1 283 400 points, one launch of 2 steps of the autotuned tile).
-MEASURED_RUN_TRAFFIC_PER_POINT_STEP = {"fp64": 394.3, "fp32": None}
+# 1 267 800 points, one launch of 2 steps of the autotuned tile).
+MEASURED_RUN_TRAFFIC_PER_POINT_STEP = {"fp64": 395.5, "fp32": None}
 # One 2D stage per point, per workload, precision and stage form (0: the
-# x-sweep + y-sweep launches of stage 1, 1: the fused stage-1 launch; smooth
-# Euler at 1024^2, double Mach at 1920x480); applied to grids whose working
-# set exceeds the L2.
-MEASURED_STAGE_TRAFFIC_2D_PER_POINT = {("euler2d_smooth", "fp64", 0): 504.1,
+# x-sweep + y-sweep launches, of stage 1 in FP32 and of stage 3, which also reads
+# the step's input, in FP64; 1: the fused stage-1 launch; smooth Euler at
+# 1024^2, double Mach at 1920x480); applied to grids whose working set exceeds
+# the L2.
+MEASURED_STAGE_TRAFFIC_2D_PER_POINT = {("euler2d_smooth", "fp64", 0): 544.4,
                                        ("euler2d_smooth", "fp32", 0): 222.3,
                                        ("euler2d_smooth", "fp64", 1): 210.7,
                                        ("euler2d_smooth", "fp32", 1): 89.7,
-                                       ("double_mach", "fp64", 0): 489.6}
+                                       ("double_mach", "fp64", 0): 525.9}
 # One 2D Euler adjoint step (six reverse sweeps, 128-thread CTAs) per point, 512^2.
-MEASURED_ADJOINT_TRAFFIC_PER_POINT_STEP = {("euler", 2): 1862.6}
+MEASURED_ADJOINT_TRAFFIC_PER_POINT_STEP = {("euler", 2): 1850.3}
 
 
 def parse():
