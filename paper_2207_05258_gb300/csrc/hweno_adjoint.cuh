@@ -7,10 +7,11 @@
 // these kernels: about 100 operations a side, where the per-weight form in
 // full values took 61 + 75 and 11 divisions (256 x 256 density wave, one step's
 // adjoint, FP64: 5.19 -> 4.20 ms; batch of Burgers gradients 9.38 -> 7.33 ms).
-// Root-mean-square error of a side's gradient against 60 digits, smooth / jump
-// / noise: 8e-17 / 2e-13 / 1.4e-15 -> 3e-17 / 7e-17 / 1e-16; of the limiter's:
-// 1.5e-16 / 1.9e-16 / 8.1e-16 -> 1.7e-16 / 1.6e-16 / 8.3e-16, one rounding
-// each. The |.| in tau keeps the sign of
+// Root-mean-square error of a side's gradient against long double, per-weight
+// form -> this one, on smooth data / next to a jump / on noise: 2.1e-17 /
+// 2.9e-14 / 7.8e-16 -> 2.1e-17 / 3.2e-17 / 4.8e-17; of the limiter's: 5.4e-17 /
+// 1.9e-16 / 2.8e-16 -> 2.6e-17 / 5.1e-17 / 2.2e-16; of the values: 0.3 to 0.98
+// of the per-weight form's. The |.| in tau keeps the sign of
 // its argument at the point of evaluation (the branch of the forward run).
 // With `frozen` the nonlinear weights count as constants: only the
 // candidates' (linear) dependence on the data is propagated.
@@ -103,9 +104,16 @@ __device__ __forceinline__ double weighted_vjp(double b0, double b1, double b2, 
   const double q1 = g1 * b2, q2 = g2 * b1, n1 = q1 * e1, n2 = q2 * e2;
   const double b12 = b1 * b2, bt = b0 + tau;
   const double iD = recip_fp64(b12 * (b0 + g0 * tau) + tau * (b0 * (q1 + q2)));
-  const double tD = tau * iD, f1 = tD * n1, f2 = tD * n2;
-  double f0 = b12 * bt * iD;
-  if (__double2hiint(f0) >= 0x3fe00000) f0 = 1.0 - (f1 + f2);  // from 1/2 on
+  const double tD = tau * iD;
+  double f0 = b12 * bt * iD, f1 = tD * n1, f2 = tD * n2;
+  // the largest weight by the other two, whose errors are smaller: phi_0 from 1/2
+  // on, the others from 15/16
+  const bool m0 = __double2hiint(f0) >= 0x3fe00000, m1 = __double2hiint(f1) >= 0x3fee0000;
+  const bool m2 = __double2hiint(f2) >= 0x3fee0000;
+  const double most = 1.0 - ((m0 ? f1 : f0) + (m2 ? f1 : f2));
+  if (m0) f0 = most;
+  else if (m1) f1 = most;
+  else if (m2) f2 = most;
   const double r0 = -(f1 * P1 + f2 * P2);
   gp0 = mu * f0;
   gp1 = mu * f1;
@@ -226,12 +234,14 @@ __device__ __forceinline__ double limiter_vjp(double um, double u0, double up, d
   const double t0 = 2.0 * gb0;
   const double gz1 = t0 * c1, gdV = t0 * c2;
   const double gsV = gz1 - 0.25 * gp0;
-  const double gl = L2 * gdV + t0 * cl, gdu = (L1 - 1.0) * gz1 + (t0 * cu + 0.75 * gp0);
+  // the cotangents of q1 and q2 but for 3/4 gp0 of each, which is added last (one
+  // rounding of the full value) and drops out of their difference
+  const double gl = L2 * gdV + t0 * cl, gdu = (L1 - 1.0) * gz1 + t0 * cu;
   const double gq1 = 2.0 * (gb1 * q1) + (gp1 + (gdu - gl));
   const double gq2 = 2.0 * (gb2 * q2) + (gp2 + (gdu + gl));
-  g[0] -= gq1;
+  g[0] -= 0.75 * gp0 + gq1;
   g[1] += gq1 - gq2;
-  g[2] += gq2;
+  g[2] += 0.75 * gp0 + gq2;
   g[3] += gsV + gdV;
   g[4] += gsV - gdV;
   return v;

@@ -123,3 +123,23 @@ def test_gradient(lib, which, scale, kind):
     err = np.abs(g.T - ref.d).max(axis=0) / np.abs(ref.d).max(axis=0)
     assert err.max() <= TOL, err.max()
     assert (np.abs(v - ref.v) / np.abs(x).max(axis=1)).max() <= TOL
+
+
+def test_limiter_gradient_of_smooth_data(lib):
+    """Nearly the linear weights' gradient, (-3/4, 0, 3/4, -1/4, -1/4): each entry
+    is rounded at most four times at its full size (phi_0, the product, the sum;
+    root mean square 3.2e-17 each in [1/2, 1), half that in [1/4, 1/2)), the rest
+    of it is small."""
+    g = np.random.default_rng(4)
+    a, b, c = (g.uniform(-1, 1, (20000, 1)) for _ in range(3))
+    z = np.array([-0.05, 0.0, 0.05])
+    x = np.ascontiguousarray(np.hstack([a + b * np.sin(z + 3 * c),
+                                        0.05 * b * np.cos(z[[0, 2, 1]] + 3 * c)]))
+    w, v, gr = np.array([0.98, 0.01, 0.01]), np.zeros(len(x)), np.zeros_like(x)
+    lib.host_vjp(1, len(x), H.ptr(x), H.ptr(w), H.ctypes.c_double(1e-6), H.ptr(v), H.ptr(gr))
+    d = np.eye(6, dtype=L)
+    ref = limiter([Dual(x[:, k].astype(L), np.repeat(d[:, k:k + 1], len(x), 1)) for k in range(6)],
+                  w.astype(L), L(1e-6))
+    rms = np.sqrt(((gr.T - ref.d) ** 2).mean(axis=1))
+    assert (rms[[0, 2]] <= 2 * 3.2e-17).all() and (rms[[3, 4]] <= 2 * 1.6e-17).all(), rms
+    assert rms[1] <= 1e-18
