@@ -20,7 +20,7 @@ def load(directory):
         return _loaded[0]
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc())))
     lib = os.path.join(str(directory), "libhost_kernels.so")
-    cmd = ["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-w",
+    cmd = ["g++", "-O1", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-w",
            "-I", HERE, "-I", build.CSRC, "-I", build.INCLUDE, "-I", os.path.join(cuda, "include"),
            os.path.join(HERE, "_host_kernels.cpp"), "-o", lib]
     r = subprocess.run(cmd, capture_output=True, text=True)
