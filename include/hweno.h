@@ -122,15 +122,15 @@ typedef struct hweno_options {
   double lin_w[3]; /* gamma_0..2 of the reconstruction: >= 1e-6 each, sum 1 (Sec. 2.1) */
   double lim_d[3]; /* d_0..2 of the limiter: >= 1e-6 each, sum 1 (Sec. 2.2) */
   double eps;      /* epsilon of the nonlinear weights, in [1e-20, 1e6]. The
-                      FP64 kernels resolve the nonlinear weights of two sides
-                      and two fields over one common denominator, a product
-                      of up to sixteen factors of the size of beta + eps; the
-                      bounds on eps and the linear weights keep it above the
-                      FP64 underflow limit. Large data (beta grows like the
-                      square of the split-flux jumps) would push it past the
-                      overflow limit, so each side's numerator and
-                      denominator are rescaled by an exact power of two; this
-                      holds for split-flux jumps up to about 1e35 (tested
+                      kernels bring a side's weights over their common
+                      denominator, a product of three indicators beta + eps
+                      and tau (FP64 stages scale them to the largest, by an
+                      exact power of two; the fused 2D stage and the cluster
+                      step's latency form resolve two sides and several fields
+                      over one denominator of up to sixteen such factors, each
+                      side scaled); the bounds on eps and the linear weights
+                      keep it above the FP64 underflow limit. This holds for
+                      split-flux jumps up to about 1e35 (tested
                       against the CPU oracle with Euler states scaled by 1e6,
                       1e12, 1e20 and Burgers by 1e4, 1e8). Other eps values
                       are HWENO_EINVAL. */
@@ -155,7 +155,7 @@ typedef struct hweno_options {
                        tiled kernels. Results agree to rounding. One CTA has
                        1/152 of the GPU's FP64 pipe, so for a few FP64
                        instances the tiled kernels are faster (Burgers N = 400:
-                       40 vs 34.5 us per step); the fused step pays off in FP32
+                       52 vs 37 us per step); the fused step pays off in FP32
                        or for batches of many small instances.
                        2 = when every instance has at most
                        HWENO_CLUSTER_MAX_POINTS points, one launch per step
@@ -180,7 +180,7 @@ typedef struct hweno_options {
                        computed by both neighbours). Results agree to
                        rounding; hweno_autotune picks the faster form for the
                        caller's grid (FP64: the sweeps at every size, 256 x 256
-                       Euler 0.33 vs 1.05 ms per step). hweno_rhs always uses the sweeps. */
+                       Euler 0.34 vs 1.05 ms per step). hweno_rhs always uses the sweeps. */
 } hweno_options;
 
 /* Largest instance of the cluster step (fused_small = 2): 8 tiles of 124. */

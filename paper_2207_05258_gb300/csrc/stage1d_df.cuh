@@ -10,12 +10,11 @@
 // (weno_df.cuh), about 7 000 other instructions per point, which issue next to
 // the FP64 pipe. Interfaces and points whose correction is not small
 // (a percent or so in flows with shocks) go on a list and are evaluated in
-// FP64. Measured, 2048 Riemann problems (2.5 M points): 12.8 -> 3.37 ms per
-// step (FP64 pipe 48% busy, issue slots 40%; stalls per issue: no instruction
-// 3.3, fixed latency 1.7, shared memory 1.1); Buckley-Leverett, 246 k points:
-// 0.40 -> 0.14 ms (FP64 pipe 74%). Error against 128-bit arithmetic relative to
-// the all-FP64 form (2-norms; Riemann problems, density waves, blast waves,
-// N = 60..800): U 0.6-1.0, V 0.3-0.95, L^1 0.1-0.4, L^2 0.04-0.8, v~ 0.02-1.
+// FP64. Measured, 2048 Riemann problems (2.5 M points): 12.8 -> 3.40 ms per
+// step (FP64 pipe 47% busy, issue slots 42%; stalls per issue: no instruction
+// 0.7, fixed latency 1.8, shared memory 1.6, barriers 1.7, in the persistent
+// run's 256-thread CTAs); Buckley-Leverett, 246 k points: 0.40 -> 0.14 ms (FP64
+// pipe 72%). Error relative to the all-FP64 form: weno_df.cuh.
 // The loops over fields stay rolled: unrolled, the straight code outruns the
 // instruction caches (6.9 ms per step when the sides were unrolled too).
 //
@@ -278,8 +277,8 @@ __device__ __forceinline__ void stage_tile_df(const Args1D& a, const StageIO& io
 // components of a point. Results are the bits of stage_tile_df. Measured: the
 // tiled form leaves a stage of one small instance to four warps on one SM
 // (FP32 chains at 0.3 instructions per cycle); Riemann problem N = 200, one
-// step 92 -> 87 us; cluster steps: blast waves N = 800 83 -> 60 us per step,
-// Burgers N = 400 17.5 -> 14 us.
+// step 92 -> 88 us; cluster steps: blast waves N = 800 83 -> 64 us per step,
+// Burgers N = 400 17.5 -> 15 us.
 // ---------------------------------------------------------------------------
 constexpr int kWideMax = 124;   // points of a wide tile
 constexpr int kFieldsMax = 60;  // ... with one role per field

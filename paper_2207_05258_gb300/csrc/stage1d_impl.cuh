@@ -1577,9 +1577,9 @@ cudaError_t step_cluster_f64_try(const Args1D& a, const FusedArgs& f, int max_n,
 // a point over four warps) when the device holds such clusters. Else FP32
 // takes 124-point tiles and FP64 the wide form (28-point tiles for the scalar
 // equations). Measured, FP64, us per step, latency form / wide form: Burgers
-// N = 60..440 18.5 / 14, Euler Riemann problem 51 / 47.5 but blast waves,
+// N = 60..440 18.5 / 15, Euler Riemann problem 51 / 47.5 but blast waves,
 // with FP64 items in most tiles, 51 / 60; 124-point tiled cluster / wide form
-// at N = 460..992: Burgers 35 / 15, Euler 108 / 52 to 74.
+// at N = 460..992: Burgers 35 / 16 to 20, Euler 108 / 60 to 64.
 template <int EQ, class Real>
 cudaError_t step_cluster_launch(const Args1D& a, const FusedArgs& f, int max_n, cudaStream_t s) {
   if constexpr (std::is_same<Real, double>::value) {

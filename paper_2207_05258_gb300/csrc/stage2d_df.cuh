@@ -5,18 +5,17 @@
 //
 // What bounds them: an all-FP64 stage (x- and y-sweep) needs about 2 200 FP64
 // instructions per point at 65 to 77 cycles per warp and sub-partition; here
-// about 340 remain (FP64 pipe 42% and 53% busy on the double Mach grid), next
-// to about 18 500 others, whose fetch and latency take the rest of the time
-// (stalls per issue: no instruction 3.1 and 1.8, fixed latency 1.7 and 1.9).
-// Measured per step: double Mach 1920 x 480 13.2 -> 3.12 ms; 256^2 1.06 ->
-// 0.34 ms; Burgers rhs 321 x 203, 95 -> 50 us. Error against 128-bit
-// arithmetic relative to the all-FP64 sweeps (2-norms): U 0.8-0.95, V, W
-// 0.66-1.0, L^1 0.1-0.5, L^2, L^3 0.45-0.55, v~, w~ 0.01-0.6.
+// about 335 remain (FP64 pipe 46% and 53% busy on the double Mach grid), next
+// to about 18 500 others, whose latency and fetch take the rest of the time
+// (stalls per issue: fixed latency 1.7 and 1.9, shared memory 1.4 and 1.6, no
+// instruction 1.0 and 0.4). Measured per step: double Mach 1920 x 480 13.2 ->
+// 3.19 ms; 256^2 1.06 -> 0.34 ms; Burgers rhs 321 x 203, 96 -> 52 us. Error
+// relative to the all-FP64 sweeps: weno_df.cuh.
 //
 // Tiles (128 threads; Shape2D for large grids): the x-sweep takes row segments
-// of 124 points. The y-sweep takes blocks of 4 columns x 31 rows: 35 rows loaded for 31 (16 columns x 7 rows
-// load 11 for 7, and the point phase is FP64 work), while the 4 columns are
-// one 32-byte sector of a row. Both give 128 interfaces, one per thread, and
+// of 124 points. The y-sweep takes blocks of 4 columns x 31 rows: 35 rows
+// loaded for 31 (16 columns x 7 rows load 11 for 7, and the point phase is FP64
+// work), while the 4 columns are one 32-byte sector of a row. Both give 128 interfaces, one per thread, and
 // 51 to 55 KB of shared memory, four CTAs per SM.
 
 // Large Euler grids take CTAs of 256 threads (252 points; 8 columns x 31 rows),
